@@ -45,7 +45,7 @@ typedef enum {
   LP_ERR_OOM = 3,         /* device or host allocation failed            */
   LP_ITER_LIMIT = 4,      /* max_iter reached before the tolerance       */
   LP_ERR_NUMERICAL = 5,   /* NaN or Inf met in an iterate or residual    */
-  LP_ERR_TIMEOUT = 6,     /* reserved: a bounded device wait expired     */
+  LP_ERR_TIMEOUT = 6,     /* a bounded wait on the device expired        */
   LP_ERR_NOT_SOLVED = 7   /* no solve has run on this handle yet         */
 } lp_status;
 
@@ -102,12 +102,15 @@ typedef struct {
   int32_t spmv_mode;      /* reserved, must be 0 */
   int32_t precision;      /* LP_PRECISION_FP64 (default) or LP_PRECISION_MIXED */
   int32_t lane_auto;      /* > 0: per matrix, halve single_lane_max and lane_steps until the
-                             layout has at least lane_auto x (SM count) slices (warps); 0: use
-                             the given lane policy as is (32) */
-  int32_t autotune;       /* 1: at lp_create, time every unroll variant of the column and row
-                             passes on this problem and keep the fastest (overrides spmv_unroll
-                             and spmv_unroll_rows; results do not depend on the variant: every
-                             variant sums each row in the same order); 0: use them as given (1) */
+                             layout has at least lane_auto x (SM count) slices (warps), in FP64
+                             not below 8 elements per lane; 0: use the given lane policy as is (32) */
+  int32_t autotune;       /* 1: at lp_create, choose how the iterations run: an LP that fits into
+                             the SMs' shared memory (without split rows, check_every <= 1024) runs
+                             K iterations and the check in one cooperative launch; for others every
+                             unroll variant of the column and row passes is timed on this problem
+                             and the fastest kept (overrides spmv_unroll and spmv_unroll_rows).
+                             Iterates do not depend on the choice: every variant sums each row in
+                             the same order.  0: the per-pass kernels with the unrolls given (1) */
   int32_t sigma_method;   /* estimator of sigma_max(A) when eta = 0: LP_SIGMA_LANCZOS (default;
                              at most min(power_iters, 1024) steps) or LP_SIGMA_POWER (Section 7's
                              power iteration); both stop when the estimate of sigma_max^2 changes
@@ -142,6 +145,7 @@ typedef struct {
   int32_t spmv_unroll, spmv_unroll_rows; /* kernel variants in use (tuned or given) */
   int32_t sigma_steps;  /* steps of the sigma_max estimator (0 when eta was given) */
   int32_t graph_kernels; /* kernel launches per replay of the graph of K iterations + check
+                            (1: the resident kernel runs them all)
                             (0 until the first lp_solve / lp_iterate builds it) */
   int32_t n_split_slices; /* chunk slices of split rows in A and A^T together (split_row_len) */
 } lp_info;

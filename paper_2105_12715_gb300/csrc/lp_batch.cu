@@ -1733,8 +1733,8 @@ lp_status lp_batch_create(int32_t count, const int32_t *host_row_start,
   HostSell HA, HAT;
   const LanePolicy policy{opt.long_row_threshold, opt.lane_steps, opt.single_lane_max};
   const int64_t target = (int64_t)opt.lane_auto * h->nsm;
-  const LanePolicy pa = choose_policy(rp, perm_y, policy, target, brk_rows);
-  const LanePolicy pat = choose_policy(cp, perm_x, policy, target, brk_cols);
+  const LanePolicy pa = choose_policy(rp, perm_y, policy, target, 1, brk_rows);
+  const LanePolicy pat = choose_policy(cp, perm_x, policy, target, 1, brk_cols);
   build_sell(m, n, rp, hci, hv, perm_y, inv_x, pa, HA, brk_rows);
   build_sell(n, m, cp, ri.data(), cv.data(), perm_x, inv_y, pat, HAT, brk_cols);
 

@@ -234,18 +234,33 @@ inline int64_t count_slices(const std::vector<int64_t> &ptr, const std::vector<i
   return ns;
 }
 
+// Gives rows more lanes: halves single_max and lane_steps, each down to
+// floor_steps; false once neither can shrink.
+inline bool more_lanes(LanePolicy &p, int32_t floor_steps) {
+  const int32_t sm = p.single_max > floor_steps ? std::max(floor_steps, p.single_max / 2) : p.single_max;
+  const int32_t ls = p.lane_steps > floor_steps ? std::max(floor_steps, p.lane_steps / 2) : p.lane_steps;
+  if (sm == p.single_max && ls == p.lane_steps) return false;
+  p.single_max = sm;
+  p.lane_steps = ls;
+  return true;
+}
+// Fewest elements per lane that more_lanes goes down to.  FP64: 8.  Every extra
+// factor of two in lanes costs each row a butterfly step, an FP64 addition of
+// the whole warp, and GB300's FP64 pipe (2 per cycle per SM) is what a small LP
+// runs out of first (5k x 25k, resident kernel, 64 iterations and a check: 0.52 ms
+// with 8, 0.73 with 4, 0.53 with 16).  FP32 additions cost a 32nd of that: down to 1.
+inline int32_t policy_floor(bool mixed) { return mixed ? 1 : 8; }
+
 // Launch-shape tuning by a model: a pass runs one warp per slice, and
 // fewer slices than `target` warps leave SMs idle while each warp walks a
 // long chain of dependent gathers.  Starting from the given policy, give
 // rows more lanes (halving single_max and lane_steps) until the layout
-// has at least `target` slices or rows get one element per lane.
+// has at least `target` slices or rows get floor_steps elements per lane.
 inline LanePolicy choose_policy(const std::vector<int64_t> &ptr, const std::vector<int32_t> &perm,
-                                LanePolicy p, int64_t target,
+                                LanePolicy p, int64_t target, int32_t floor_steps,
                                 const std::vector<int32_t> &breaks = {}) {
   if (target <= 0) return p;
-  while (count_slices(ptr, perm, p, breaks) < target && (p.single_max > 1 || p.lane_steps > 1)) {
-    p.single_max = p.single_max / 2;
-    p.lane_steps = std::max(1, p.lane_steps / 2);
+  while (count_slices(ptr, perm, p, breaks) < target && more_lanes(p, floor_steps)) {
   }
   return p;
 }

@@ -121,6 +121,7 @@ struct DevState {
   unsigned int sel_counter[2];
   int32_t mixed;        // 1: mixed-precision iterations (MixVecs)
   double mix_s;         // scale of the current correction
+  unsigned int bar_gen;  // resident kernel: grid barriers passed since the counters were zero
 };
 
 // Device arrays of one problem, permuted order.
@@ -178,6 +179,23 @@ struct CheckScratch {
   // the bracket after the first pass) and a count; null: every pass scans all elements
   int32_t *cand[2], *ccnt[2];
   int64_t cand_cap;
+};
+
+// Arguments of the resident kernel (lp_resident.cu): K iterations and the check
+// of one problem in one cooperative launch.
+constexpr int kResBarLines = 8;
+constexpr int kResPart = 20;  // doubles per block in part (NQ quantities)
+struct ResidentArgs {
+  SellMat A, AT;
+  DevVecs v;
+  MixVecs mv;
+  DevState *st;
+  double *w, *trace;
+  CheckScratch cs;
+  double *part;   // [P][kResPart]
+  double *npart;  // [2][P][8]
+  unsigned int *bar;     // [kResBarLines][32] arrival counters of the grid barrier
+  int32_t n, m;
 };
 
 // Launch with programmatic stream serialization: the kernel may be scheduled
@@ -284,6 +302,11 @@ void launch_fill(double *p, double val, int64_t n, cudaStream_t s);
 void launch_weights(DevState *st, double *w, cudaStream_t s);
 void launch_norms(const DevVecs &v, DevState *st, double *partials, int pstride,
                   int grid, int n, int m, cudaStream_t s);
+size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed);
+size_t resident_smem_limit(int device, bool mixed);
+bool resident_fits(int P, int nsm, size_t smem, bool mixed);
+cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixed,
+                            cudaStream_t s);
 int check_grid_for(const SellMat &A, int num_sms);
 int split_grid(const SellMat &A);
 void launch_primal_mix(const SellMat &AT, const MixVecs &mv, DevState *st, const double *w,

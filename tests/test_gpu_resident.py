@@ -1,0 +1,107 @@
+"""The resident kernel (autotune = 1, LPs that fit on the SMs) against the
+per-pass kernels (autotune = 0): the same lanes, chains and butterflies, so the
+iterates agree bit for bit; the check's sums are reduced in another order, so
+its gaps and residuals agree to rounding and the restart decisions are equal."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from paper_2105_12715_gb300 import lpgen  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def lpm():
+    from paper_2105_12715_gb300 import lp
+    return lp
+
+
+def without_rows(n):
+    d = lpgen.tiny_standard_form(1, m=1, n=n, per_col=1)
+    return dataclasses.replace(d, m=0, row_ptr=np.zeros(1, np.int32), col_idx=np.zeros(0, np.int32),
+                               val=np.zeros(0), b=np.zeros(0), row_type=np.zeros(0, np.int8),
+                               ub=np.ones(n), c=np.linspace(-1.0, 1.0, n))
+
+
+CASES = {  # one slice; 4, 5 and 17 slices per block's share; ragged tails; empty rows and columns
+    "1x1": lambda: lpgen.tiny_standard_form(0, m=1, n=1, per_col=1),
+    "no_rows": lambda: without_rows(33),
+    "31x33": lambda: lpgen.tiny_standard_form(1, m=31, n=33, per_col=3),
+    "200x400": lambda: lpgen.tiny_standard_form(0),
+    "empty_lines": lambda: lpgen.adversarial(7),
+    "dense_lines": lambda: lpgen.adversarial(9, m=400, n=450),
+    "997x4999": lambda: lpgen.large_mixed(3, m=997, n=4999),
+    "5000x25000": lambda: lpgen.large_mixed(4, m=5000, n=25000),
+    "20000x90001": lambda: lpgen.large_mixed(5, m=20000, n=90001),
+}
+
+
+def run(lpm, data, autotune, **opts):
+    with lpm.LP(data, eta=0.05, autotune=autotune, **opts) as g:
+        status = g.solve(1e-300)
+        return status, g.state(), g.trace(64), g.info()
+
+
+@pytest.mark.parametrize("name", list(CASES))
+@pytest.mark.parametrize("precision", [0, 1])
+def test_same_iterates_as_the_per_pass_kernels(lpm, name, precision):
+    data = CASES[name]()
+    opts = dict(check_every=24, max_iter=24 * 6 + 7, precision=precision)  # and a partial block
+    s1, a, t1, i1 = run(lpm, data, 1, **opts)
+    s0, b, t0, i0 = run(lpm, data, 0, **opts)
+    assert i1.graph_kernels == 1 and i0.graph_kernels > 48
+    assert (s1, i1.iters, i1.restarts, i1.returned) == (s0, i0.iters, i0.restarts, i0.returned)
+    if precision == 0:  # the correction's data carry the check's rounding in mixed precision
+        for k in a:
+            np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    else:
+        for k in a:
+            np.testing.assert_allclose(a[k], b[k], rtol=0, err_msg=k,
+                                       atol=1e-6 * max(1.0, np.abs(b[k]).max(initial=0.0)))
+    np.testing.assert_array_equal(t1[:, [0, 2]], t0[:, [0, 2]])
+    if precision == 0:
+        # a gap sums n + m positive terms in another order: n eps relative, and residuals
+        # of size |b| cancel down to the KKT error
+        np.testing.assert_allclose(t1[:, [1, 3, 4, 5]], t0[:, [1, 3, 4, 5]], rtol=1e-9, atol=1e-11)
+
+
+@pytest.mark.parametrize("scheme", ["NONE", "FIXED", "FLEXIBLE"])
+def test_schemes(lpm, scheme):
+    data = lpgen.large_mixed(6, m=700, n=3100)
+    opts = dict(check_every=16, max_iter=16 * 20, fixed_len=48, omega=0.25,
+                restart_scheme=getattr(lpm, "LP_RESTART_" + scheme))
+    s1, a, t1, i1 = run(lpm, data, 1, **opts)
+    s0, b, t0, i0 = run(lpm, data, 0, **opts)
+    assert i1.graph_kernels == 1 and (s1, i1.restarts) == (s0, i0.restarts)
+    for k in a:
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    np.testing.assert_allclose(t1, t0, rtol=1e-9, atol=1e-11)
+
+
+def test_check_periods_at_the_edge(lpm):
+    """K = 1 and K = 1024 run resident; K = 1025 exceeds the weights' space."""
+    data = lpgen.tiny_standard_form(2)
+    for k, resident in ((1, True), (1024, True), (1025, False)):
+        _, a, _, i1 = run(lpm, data, 1, check_every=k, max_iter=2 * k)
+        _, b, _, _ = run(lpm, data, 0, check_every=k, max_iter=2 * k)
+        assert (i1.graph_kernels == 1) == resident
+        for key in a:
+            np.testing.assert_array_equal(a[key], b[key], err_msg=f"{k} {key}")
+
+
+def test_converges_and_repeats(lpm):
+    """Solves to 1e-8, twice from the same start on one handle: same bits."""
+    data = lpgen.large_mixed(11, m=300, n=1500)
+    with lpm.LP(data, omega=0.0625, max_iter=400000) as g:
+        outs = []
+        for _ in range(2):
+            g.set_state()
+            assert g.solve(1e-8) == lpm.LP_OK
+            outs.append(g.solution() + (g.info().iters,))
+        assert g.info().graph_kernels == 1
+    assert outs[0][2] == outs[1][2]
+    np.testing.assert_array_equal(outs[0][0], outs[1][0])
+    np.testing.assert_array_equal(outs[0][1], outs[1][1])
+    assert abs(np.dot(data.c, outs[0][0]) - data.obj_star) <= 1e-6 * (1 + abs(data.obj_star))
