@@ -106,7 +106,7 @@ typedef struct {
                              not below 8 elements per lane; 0: use the given lane policy as is (32) */
   int32_t autotune;       /* 1: at lp_create, choose how the iterations run: an LP that fits into
                              the SMs' shared memory (without split rows, check_every <= 1024) runs
-                             K iterations and the check in one cooperative launch; for others every
+                             K iterations and the check in one launch; for others every
                              unroll variant of the column and row passes is timed on this problem
                              and the fastest kept (overrides spmv_unroll and spmv_unroll_rows).
                              Iterates do not depend on the choice: every variant sums each row in

@@ -27,7 +27,11 @@
  * a work list rebuilt at each check), and the checks of all problems due at
  * a block boundary run together (one block of threads per problem for
  * reductions and for the multiplier search).  Problems that have stopped
- * cost nothing.  Errors, streams and ownership as in lp.h.
+ * cost nothing.  A batch of small problems (each fits into the shared memory of
+ * a few SMs and none holds the others up; opt->autotune = 1) takes one launch
+ * per block of K_base iterations and checks instead, every problem in a
+ * thread-block cluster of its own, with the same iterates.  Errors, streams
+ * and ownership as in lp.h.
  */
 #ifndef LP_GB300_LP_BATCH_H
 #define LP_GB300_LP_BATCH_H

@@ -216,7 +216,9 @@ cudaError_t capture_block(lp_problem *h) {
   if (e != cudaSuccess) return e;
   cudaError_t launched = cudaSuccess;
   if (h->res_blocks > 0) {
-    launched = launch_resident(h->res, h->res_blocks, h->res_smem, h->mixed, s);
+    launched = h->res.cluster > 0
+                   ? launch_cluster(h->res, 1, h->res_smem, h->mixed, true, s)
+                   : launch_resident(h->res, h->res_blocks, h->res_smem, h->mixed, s);
   } else {
     for (int k = 0; k < h->opt.check_every; ++k) launch_iteration(h, k, s);
     launch_check(h->A, h->AT, h->v, h->st, h->w, h->cs, h->n, h->m, h->nsearch, h->trace, true, s,
@@ -272,18 +274,23 @@ lp_status set_run_params(lp_problem *h, double tol, cudaStream_t s) {
   return LP_OK;
 }
 
-// Decides whether the resident kernel (lp_resident.cu) runs this problem, and on
-// how many blocks.  It does whenever autotune is on, no row is split, and the
-// matrix and the vectors fit into the shared memory of P blocks, one per SM:
-// for 5k x 25k (246k nonzeros, FP64) a block of 64 iterations and its check
-// takes 0.50 ms instead of 1.02, for 20k x 100k (1.0M nonzeros, mixed
-// precision) 0.82 ms instead of 1.37, for 200 x 400 0.32 ms instead of 0.49.
-// A larger matrix would have to be streamed again in every pass, which the
-// per-pass kernels do with more warps in flight.  P: four slices per block and
-// pass at least, so that a tiny LP's barriers and reductions span few blocks
-// (200 x 400: 1.38 ms on 4 blocks, 1.48 ms on 13 for 256 iterations).
+// Decides whether a resident kernel (lp_resident.cu) runs this problem, which
+// one, and on how many blocks.  One does whenever autotune is on, no row is
+// split, and the matrix and the vectors fit into the shared memory of P blocks,
+// one per SM: for 5k x 25k (246k nonzeros, FP64) 64 iterations and a check take
+// 0.50 ms instead of 1.02, for 20k x 100k (1.0M nonzeros, mixed precision) 0.82
+// ms instead of 1.37.  A larger matrix would have to be streamed again in every
+// pass, which the per-pass kernels do with more warps in flight.
+// Few rows and columns (2,048; in mixed precision, whose layout has more and
+// shorter slices, 768): one cluster of up to 8 blocks, whose barrier takes 500
+// cycles instead of 2,800 but whose work has only 8 SMs (200 x 400: 0.25 ms in a
+// cluster, 0.33 on the grid; 2k x 10k: 0.41 and 0.43; 600 x 1400 in mixed
+// precision: 0.72 and 0.35).  Else the grid, with at least four slices per block
+// and pass, so that the barriers and reductions of a small LP span few blocks.
 lp_status plan_resident(lp_problem *h, cudaStream_t s) {
-  constexpr int kSlicesPerBlock = 4, kMaxCheckEvery = 1024;  // the weights lie in shared memory
+  constexpr int kSlicesPerBlock = 4, kClusterBlocks = 8;
+  const int kClusterElems = h->mixed ? 768 : 2048;
+  constexpr int kMaxCheckEvery = 1024;  // the weights lie in shared memory
   const lp_options &opt = h->opt;
   if (!opt.autotune || h->A.nsplit > 0 || h->AT.nsplit > 0 || opt.check_every > kMaxCheckEvery)
     return LP_OK;
@@ -297,28 +304,50 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
                         cudaMemcpyDeviceToHost, s));
   LP_CU(cudaStreamSynchronize(s));
   const int most = std::max(h->AT.nslices, h->A.nslices);
-  const int P = std::max(1, std::min(h->nsm, (most + kSlicesPerBlock - 1) / kSlicesPerBlock));
+  // shared memory of the largest of P blocks; block b owns the slices b, b + P, ...
+  auto block_bytes = [&](int P, bool cluster) {
+    size_t smem = 0;
+    for (int b = 0; b < P; ++b) {
+      int cols = 0, rows = 0;
+      int64_t elems = 0;
+      for (int i = b; i < h->AT.nslices; i += P) {
+        cols += ic[i + 1].row0 - ic[i].row0;
+        elems += (ic[i].len_g >> 3) * kWarp;
+      }
+      for (int i = b; i < h->A.nslices; i += P) {
+        rows += ir[i + 1].row0 - ir[i].row0;
+        elems += (ir[i].len_g >> 3) * kWarp;
+      }
+      const int nc = (h->AT.nslices - b + P - 1) / P, nr = (h->A.nslices - b + P - 1) / P;
+      smem = std::max(smem, resident_fixed_bytes(nc, nr, cols, rows, opt.check_every, h->mixed,
+                                                 cluster ? h->n : 0, cluster ? h->m : 0) +
+                                (size_t)(elems * elem));
+    }
+    return smem;
+  };
+  int P = 0, cluster = 0;
   size_t smem = 0;
-  for (int b = 0; b < P; ++b) {  // block b owns the slices b, b + P, ...
-    int cols = 0, rows = 0;
-    int64_t elems = 0;
-    for (int i = b; i < h->AT.nslices; i += P) {
-      cols += ic[i + 1].row0 - ic[i].row0;
-      elems += (ic[i].len_g >> 3) * kWarp;
+  if ((int64_t)h->n + h->m <= kClusterElems) {
+    for (int C = kClusterBlocks; C >= 1 && !cluster; C /= 2) {
+      if (C > 1 && C > most) continue;
+      smem = block_bytes(C, true);
+      if (smem <= limit && cluster_fits(C, smem, h->mixed, true, false)) cluster = C;
     }
-    for (int i = b; i < h->A.nslices; i += P) {
-      rows += ir[i + 1].row0 - ir[i].row0;
-      elems += (ir[i].len_g >> 3) * kWarp;
-    }
-    const int nc = (h->AT.nslices - b + P - 1) / P, nr = (h->A.nslices - b + P - 1) / P;
-    smem = std::max(smem, resident_fixed_bytes(nc, nr, cols, rows, opt.check_every, h->mixed) +
-                              (size_t)(elems * elem));
+    P = cluster;
   }
-  if (smem > limit || !resident_fits(P, h->nsm, smem, h->mixed)) return LP_OK;
+  if (!cluster) {
+    P = std::max(1, std::min(h->nsm, (most + kSlicesPerBlock - 1) / kSlicesPerBlock));
+    smem = block_bytes(P, false);
+    if (smem > limit || !resident_fits(P, h->nsm, smem, h->mixed)) return LP_OK;
+  }
   lp_status e;
   if ((e = h->alloc(&h->res.part, (int64_t)P * kResPart)) != LP_OK) return e;
   if ((e = h->alloc(&h->res.npart, (int64_t)2 * P * 8)) != LP_OK) return e;
   if ((e = h->alloc(&h->res.bar, kResBarLines * 32)) != LP_OK) return e;
+  if (h->mixed &&
+      (e = h->alloc(&h->res.rpart, (int64_t)2 * (h->cs.cols_grid + h->cs.rows_grid))) != LP_OK)
+    return e;
+  h->res.cluster = cluster;
   h->res.A = h->A;
   h->res.AT = h->AT;
   h->res.v = h->v;

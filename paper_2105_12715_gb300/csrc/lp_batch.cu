@@ -30,6 +30,8 @@
 //   b_restart_copy: z^{n+1,0} <- zbar, z <- zbar for restarting problems;
 //   b_list_scan / b_list_fill: the next block's slice work lists and
 //       averaging weights (running problems only).
+// A batch of small problems runs whole blocks, checks included, in one launch
+// of the cluster kernel instead (lp_resident.cu; plan_batch_resident).
 // Also here: the batch tuner, mixed precision (combine / recenter per
 // problem), and the recorded forward and adjoint of the unrolled maps.
 // All reductions run in a fixed order: results are bitwise reproducible
@@ -56,7 +58,6 @@ namespace lpg {
 namespace {
 
 constexpr int kMaxClasses = 8;
-constexpr int kCheckChunk = 8;  // slices per warp and reduction in the check kernels
 constexpr int kStatusIterLimit = 4;
 constexpr int kListThreads = 1024;
 constexpr int kSearchWarps = 8;
@@ -65,40 +66,6 @@ static_assert(kSearchThreads == kBuckets, "bracket selection uses one thread per
 constexpr size_t kSearchHistBytes = sizeof(double) * kSearchWarps * kBuckets * 3;
 constexpr size_t kSearchCntBytes = sizeof(unsigned) * kSearchWarps * kBuckets;
 constexpr size_t kSearchSmem = kSearchHistBytes + kSearchCntBytes + sizeof(double) * kSearchWarps * kWarp * 3;
-
-// Per-problem state (device, one per problem).
-struct BInst {
-  int32_t col0, ncol, row0, nrow;  // ranges in the permuted index spaces
-  int32_t cs0, cs1, rs0, rs1;      // slice ranges in A^T and A
-  int32_t cc0, cc1, rc0, rc1;      // check-chunk ranges in A^T and A
-  int32_t wlc0, wlr0;              // this problem's offsets in the work lists (if running)
-  int32_t K;                       // check period (multiple of K_base)
-  int32_t status;                  // kRunning or a final lp_status
-  int32_t returned, restart_now, use_cur, due;
-  int32_t pw_done, pw_iters;
-  int64_t t0;                      // inner iterations since the restart, at block start
-  int64_t iters, checks, restarts;
-  int64_t since;                   // iterations since the last check
-  int64_t iter_cap;                // stop (iteration limit) once iters reaches it
-  int64_t tau0, fixed_len;
-  double tau, sigma, omega;
-  double norm_b, norm_c;
-  double rho_stored, last_rho, last_r;
-  double kkt_a[5], kkt_c[5];
-  double pw_est, pw_nw;
-  double mix_s;                    // mixed precision: scale of the current correction
-  LSearch ls[2];
-};
-
-// Batch-wide parameters and counters (device).
-struct BGlobal {
-  double tol, beta, pw_tol;
-  int32_t count, Kb, scheme, pw_max;
-  int32_t running;     // problems still iterating after the last check
-  int32_t pw_running;  // problems still estimating sigma_max after the last step
-  int32_t wl_n[2];     // work-list lengths: [0] column slices, [1] row slices
-  int32_t mixed;       // 1: mixed-precision iterations
-};
 
 struct SearchArrays {
   uint64_t *keys[2];
@@ -1231,6 +1198,9 @@ struct lp_batch {
   int32_t *h_running = nullptr;  // pinned [2]
   cudaEvent_t ev[2] = {nullptr, nullptr};
   bool solved = false;
+  ResidentArgs res{};     // cluster kernel (lp_resident.cu), when res.cluster > 0
+  size_t res_smem = 0;
+  bool res_inside = false;  // the matrix stays in shared memory
 
   ~lp_batch() {
     if (ckpt) cudaFree(ckpt);
@@ -1417,14 +1387,25 @@ lp_status batch_build_graph(lp_batch *h) {
   if (h->exec) return LP_OK;
   cudaStream_t s = h->cap_stream;
   LP_CU(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  for (int k = 0; k < h->opt.check_every; ++k) {
-    h->launch_primal(k, s);
-    h->launch_dual(k, s);
+  cudaError_t launched = cudaSuccess;
+  if (h->res.cluster > 0) {  // each cluster iterates, checks and counts its own problem
+    launched = cudaMemsetAsync(&h->G->running, 0, sizeof(int32_t), s);
+    if (launched == cudaSuccess)
+      launched = launch_cluster(h->res, h->count, h->res_smem, h->mixed, h->res_inside, s);
+  } else {
+    for (int k = 0; k < h->opt.check_every; ++k) {
+      h->launch_primal(k, s);
+      h->launch_dual(k, s);
+    }
+    h->launch_check(s);
   }
-  h->launch_check(s);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(s, &g);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
+  if (e == cudaSuccess && launched != cudaSuccess) {
+    cudaGraphDestroy(g);
+    e = launched;
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "capture of an iteration block");
   h->graph = g;
   LP_CU(cudaGraphInstantiate(&h->exec, g, 0));
   return LP_OK;
@@ -1585,6 +1566,68 @@ lp_status batch_tune(lp_batch *h, cudaStream_t s) {
   return LP_OK;
 }
 
+// Decides whether the cluster kernel (lp_resident.cu) runs the batch, every
+// problem in a cluster of C blocks, and whether the matrix stays in shared
+// memory.  Two launches per iteration cost a batch of small problems 8 us and
+// more, and a check ten launches; in the cluster kernel 512 problems of 200 x
+// 400 are bound by the FP64 pipe (21,500 cycles per iteration with four blocks
+// per SM, of which the FP64 instructions take 19,800): 0.80 ms per 64
+// iterations and check instead of 1.30 (1.74 with the lanes of the batch's
+// former layout).
+//   C: as many blocks (up to 8) as give every SM one, or two (128 problems of
+// 1000 x 2000: 1.21 ms per 64 iterations and check with C = 2, 1.43 with 1; 42
+// mixed-precision ones of 471 x 942: 0.75 with C = 4, 0.92 with 2).  The matrix
+// stays inside when all blocks then still fit at once (at most two per SM by
+// registers); otherwise it streams from L2 and four blocks fit.
+//   The batch goes this way when its largest problem does not hold the others
+// up: its FP64 time per iteration on C SMs is at most 16,000 cycles (less than
+// the launches cost) or 1.3 times the batch's mean per SM.
+void plan_batch_resident(lp_batch *h, const HostSell &HA, const HostSell &HAT,
+                         const std::vector<BInst> &hi) {
+  constexpr int kMaxCheckEvery = 1024;  // the weights lie in shared memory
+  constexpr double kWarpOp = 19.0;      // cycles of an SM per FP64 instruction of a warp
+  constexpr double kLaunchCycles = 16e3, kImbalance = 1.3;
+  const lp_options &opt = h->opt;
+  if (!opt.autotune || opt.check_every > kMaxCheckEvery) return;
+  const size_t limit = resident_smem_limit(h->device, h->mixed);
+  if (limit == 0) return;
+  const int64_t elem = h->mixed ? 8 : 12;  // bytes of an index and a value
+  double total = 0.0, largest = 0.0;
+  for (const BInst &B : hi) {  // products, butterflies, projections and averages
+    double w = 0.0;
+    for (int s = B.cs0; s < B.cs1; ++s) w += 4 + (HAT.info[s].len_g >> 3) + (HAT.info[s].len_g & 7);
+    for (int s = B.rs0; s < B.rs1; ++s) w += 3 + (HA.info[s].len_g >> 3) + (HA.info[s].len_g & 7);
+    total += kWarpOp * w;
+    largest = std::max(largest, kWarpOp * w);
+  }
+  int C = 1;
+  while (C < kMaxCluster && (int64_t)h->count * C <= h->nsm) C *= 2;  // at most two blocks per SM
+  if (largest / C > std::max(kLaunchCycles, kImbalance * total / h->nsm)) return;
+  size_t with = 0, without = 0;
+  for (const BInst &B : hi)
+    for (int b = 0; b < C; ++b) {
+      int cols = 0, rows = 0, nc = 0, nr = 0;
+      int64_t elems = 0;
+      for (int s = B.cs0 + b; s < B.cs1; s += C, ++nc) {
+        cols += HAT.info[s + 1].row0 - HAT.info[s].row0;
+        elems += (HAT.info[s].len_g >> 3) * kWarp;
+      }
+      for (int s = B.rs0 + b; s < B.rs1; s += C, ++nr) {
+        rows += HA.info[s + 1].row0 - HA.info[s].row0;
+        elems += (HA.info[s].len_g >> 3) * kWarp;
+      }
+      const size_t fixed = resident_fixed_bytes(nc, nr, cols, rows, opt.check_every, h->mixed,
+                                                B.ncol, B.nrow);
+      without = std::max(without, fixed);
+      with = std::max(with, fixed + (size_t)(elems * elem));
+    }
+  const int64_t per_sm = ((int64_t)h->count * C + h->nsm - 1) / h->nsm;
+  h->res_inside = per_sm <= 2 && (int64_t)with * per_sm <= (int64_t)limit;
+  h->res_smem = h->res_inside ? with : without;
+  if (h->res_smem > limit || !cluster_fits(C, h->res_smem, h->mixed, h->res_inside, true)) return;
+  h->res.cluster = C;
+}
+
 double ms_since(std::chrono::steady_clock::time_point t0) {
   return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
 }
@@ -1733,8 +1776,10 @@ lp_status lp_batch_create(int32_t count, const int32_t *host_row_start,
   HostSell HA, HAT;
   const LanePolicy policy{opt.long_row_threshold, opt.lane_steps, opt.single_lane_max};
   const int64_t target = (int64_t)opt.lane_auto * h->nsm;
-  const LanePolicy pa = choose_policy(rp, perm_y, policy, target, 1, brk_rows);
-  const LanePolicy pat = choose_policy(cp, perm_x, policy, target, 1, brk_cols);
+  const LanePolicy pa = choose_policy(rp, perm_y, policy, target,
+                                         policy_floor(opt.precision == LP_PRECISION_MIXED), brk_rows);
+  const LanePolicy pat = choose_policy(cp, perm_x, policy, target,
+                                          policy_floor(opt.precision == LP_PRECISION_MIXED), brk_cols);
   build_sell(m, n, rp, hci, hv, perm_y, inv_x, pa, HA, brk_rows);
   build_sell(n, m, cp, ri.data(), cv.data(), perm_x, inv_y, pat, HAT, brk_cols);
 
@@ -2031,6 +2076,26 @@ lp_status lp_batch_create(int32_t count, const int32_t *host_row_start,
   LP_CU(cudaMemcpy(h->I, hi.data(), sizeof(BInst) * count, cudaMemcpyHostToDevice));
   for (int q = 0; q < kMaxClasses; ++q) h->class_k[q] = 0;
   for (int32_t q = 0; q < count; ++q) h->class_k[h->size_class[q]] = opt.check_every;
+  plan_batch_resident(h.get(), HA, HAT, hi);
+  if (h->res.cluster > 0) {
+    ResidentArgs &r = h->res;
+    if ((e = h->alloc(&r.part, (int64_t)count * r.cluster * kResPart)) != LP_OK) return e;
+    if ((e = h->alloc(&r.npart, (int64_t)2 * count * r.cluster * 8)) != LP_OK) return e;
+    r.A = h->A;
+    r.AT = h->AT;
+    r.v = h->v;
+    r.mv = h->mv;
+    for (int k = 0; k < 2; ++k) {
+      r.cs.keys[k] = h->sa.keys[k];
+      r.cs.d2[k] = h->sa.d2[k];
+      r.cs.g2[k] = h->sa.g2[k];
+      r.cs.gd[k] = h->sa.gd[k];
+    }
+    r.n = n;
+    r.m = m;
+    r.inst = h->I;
+    r.glob = h->G;
+  }
   if (tune.autotune) {
     const auto t_tune = std::chrono::steady_clock::now();
     if ((e = batch_reset(h.get(), s)) != LP_OK) return e;

@@ -181,8 +181,43 @@ struct CheckScratch {
   int64_t cand_cap;
 };
 
-// Arguments of the resident kernel (lp_resident.cu): K iterations and the check
-// of one problem in one cooperative launch.
+// Per-problem state of a batch (device, one per problem).
+struct BInst {
+  int32_t col0, ncol, row0, nrow;  // ranges in the permuted index spaces
+  int32_t cs0, cs1, rs0, rs1;      // slice ranges in A^T and A
+  int32_t cc0, cc1, rc0, rc1;      // check-chunk ranges in A^T and A
+  int32_t wlc0, wlr0;              // this problem's offsets in the work lists (if running)
+  int32_t K;                       // check period (multiple of K_base)
+  int32_t status;                  // kRunning or a final lp_status
+  int32_t returned, restart_now, use_cur, due;
+  int32_t pw_done, pw_iters;
+  int64_t t0;                      // inner iterations since the restart, at block start
+  int64_t iters, checks, restarts;
+  int64_t since;                   // iterations since the last check
+  int64_t iter_cap;                // stop (iteration limit) once iters reaches it
+  int64_t tau0, fixed_len;
+  double tau, sigma, omega;
+  double norm_b, norm_c;
+  double rho_stored, last_rho, last_r;
+  double kkt_a[5], kkt_c[5];
+  double pw_est, pw_nw;
+  double mix_s;                    // mixed precision: scale of the current correction
+  LSearch ls[2];
+};
+
+// Batch-wide parameters and counters (device).
+struct BGlobal {
+  double tol, beta, pw_tol;
+  int32_t count, Kb, scheme, pw_max;
+  int32_t running;     // problems still iterating after the last check
+  int32_t pw_running;  // problems still estimating sigma_max after the last step
+  int32_t wl_n[2];     // work-list lengths: [0] column slices, [1] row slices
+  int32_t mixed;       // 1: mixed-precision iterations
+};
+
+// Arguments of the resident kernels (lp_resident.cu): K iterations and the check
+// of one problem in one cooperative launch, or of one problem per cluster.
+constexpr int kCheckChunk = 8;  // batch: slices per warp and reduction in the check kernels
 constexpr int kResBarLines = 8;
 constexpr int kResPart = 20;  // doubles per block in part (NQ quantities)
 struct ResidentArgs {
@@ -192,10 +227,14 @@ struct ResidentArgs {
   DevState *st;
   double *w, *trace;
   CheckScratch cs;
-  double *part;   // [P][kResPart]
-  double *npart;  // [2][P][8]
+  double *part;   // per problem [P][kResPart]
+  double *npart;  // per problem [2][P][8]
+  double *rpart;  // mixed precision, single problem: [2][cols_grid + rows_grid] radius sums
   unsigned int *bar;     // [kResBarLines][32] arrival counters of the grid barrier
   int32_t n, m;
+  int32_t cluster;       // blocks per problem of the cluster kernel
+  BInst *inst;           // batch: the problems, one cluster each (null: the single problem st)
+  BGlobal *glob;
 };
 
 // Launch with programmatic stream serialization: the kernel may be scheduled
@@ -302,9 +341,13 @@ void launch_fill(double *p, double val, int64_t n, cudaStream_t s);
 void launch_weights(DevState *st, double *w, cudaStream_t s);
 void launch_norms(const DevVecs &v, DevState *st, double *partials, int pstride,
                   int grid, int n, int m, cudaStream_t s);
-size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed);
+size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed, int ncol,
+                            int nrow);
 size_t resident_smem_limit(int device, bool mixed);
 bool resident_fits(int P, int nsm, size_t smem, bool mixed);
+bool cluster_fits(int C, size_t smem, bool mixed, bool res, bool batch);
+cudaError_t launch_cluster(const ResidentArgs &a, int problems, size_t smem, bool mixed, bool res,
+                           cudaStream_t s);
 cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixed,
                             cudaStream_t s);
 int check_grid_for(const SellMat &A, int num_sms);

@@ -1,6 +1,8 @@
 // One kernel per check block for LPs that fit on the SMs: K iterations, the
 // check, the multiplier search, the restart decision and the restart, with
-// the matrix and the owned part of every vector in shared memory.
+// the matrix and the owned part of every vector in shared memory.  A larger LP
+// takes the whole grid (cooperative launch); a small one, and every problem of a
+// batch of small ones, a cluster of 1 to 8 blocks.
 //
 // What bounds a small or medium LP in the two-launches-per-iteration path is
 // neither bytes nor FP64 but the chain of each launch: scheduling, the slice
@@ -28,6 +30,13 @@
 // warp, and the owned rows and columns are laid out one per thread where the
 // averages and the check's terms are formed.
 //
+// In a cluster every block holds whole copies of xhat and y in shared memory and
+// the owners store into all of them, so a gather costs 30 cycles instead of 700
+// and the barrier 500 instead of 2,800: 200 x 400, 64 iterations and a check,
+// 0.25 ms on 8 blocks (0.33 on the grid, 0.49 with the per-pass kernels).  What
+// bounds a batch is the FP64 pipe: 512 problems of 200 x 400 run at 21,500
+// cycles per iteration with four blocks per SM, 19,800 of them FP64 issue.
+//
 // The multiplier lambda* of Section 6.3 is found by Newton's method on
 // F(mu) = sum min(d^2, mu g^2) = r^2, mu = lambda^2: F is concave and piecewise
 // linear, so from mu = 0 the iterates increase to mu* and are exact once the
@@ -37,6 +46,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "lp_internal.h"
 #include "spmv_core.cuh"
@@ -44,15 +54,17 @@
 namespace lpg {
 namespace {
 
-constexpr int kRT = 512;               // threads per block
-constexpr int kRW = kRT / kWarp;       // warps per block
+constexpr int kGridThreads = 512;      // threads per block of the grid kernel
+constexpr int kClusterThreads = 256;   // and of the cluster kernel
 constexpr int kU = 8;                  // gathers in flight per lane
 constexpr int kNewtonMax = 1024;       // Newton steps (each clamps at least one more coordinate)
+constexpr int kStatusIterLimit = 4;
 constexpr int kStatusTimeout = 6;
 constexpr int kBarLines = kResBarLines;  // arrival counters of the grid barrier
 constexpr unsigned long long kWaitNs = 2000000000ull;  // longest wait at a barrier
 
-// One local slice: first element in shared memory, first local row,
+// One local slice: first element (in shared memory, or from the problem's first
+// element on when the matrix stays in global memory), first local row,
 // steps << 16 | log2 of the lanes per row << 8 | rows, and its global number.
 struct __align__(16) LSlice {
   int32_t soff, slot0;
@@ -66,33 +78,44 @@ struct __align__(16) LSlice {
 // Position in the local list (most steps first) of a warp's slice of a round:
 // the first round goes up the warps and the later ones come down, so the warps
 // with the longest slices get the shortest of the rest, or none.
+template <int NT>
 __device__ __forceinline__ int pick(int round, int warp) {
-  return round == 0 ? warp : round * kRW + kRW - 1 - warp;
+  constexpr int W = NT / kWarp;
+  return round == 0 ? warp : round * W + W - 1 - warp;
 }
+
+// Scalars of the problem, read once by one thread.
+struct Scalars {
+  double tau, sigma, omega, norm_b, norm_c, tol, beta, rho_stored, last_r, mix_s;
+  int64_t t0, restarts, tau0, fixed_len;
+  int32_t K, scheme, due, returned;
+};
 
 struct Header {
   int32_t ncl, nrl;  // local columns and rows
   int32_t nce, nre;  // elements
   int32_t dead;      // a wait ran out
-  // Scalars computed by one warp: an FP64 instruction of a warp occupies its
-  // quarter of the SM for 76 cycles (measured), a square root or a division dozens
-  // of them, so the other warps read the results here.
+  // Results of one warp: an FP64 instruction of a warp occupies its quarter of
+  // the SM for 76 cycles (measured), a square root or a division dozens of
+  // them, so the other warps read the results here.
   int32_t status, returned, restart, use_cur;
   int32_t done[2];
   int32_t count[2];  // coordinates clamped at the last Newton step
   double sw, isw, inv;
   double kkt[2][5], r2[2], lam[2], rho_r[2];
   double rho, r, mix_s;
+  Scalars sc;
 };
 
 template <typename T>
 struct Sm {  // shared-memory arrays of a block
   Header *h;
   LSlice *cs, *rs;
-  double *red;  // [kRW][32] sums of the warps
-  double *tot;  // [32] sums of the grid
+  double *red;  // [warps][32] sums of the warps
+  double *tot;  // [32] sums over the blocks
   double *nw;   // [8] Newton sums
   double *w;    // [K] averaging weights
+  T *ex, *ey;   // cluster kernel: this block's copies of xhat and y
   int32_t *crow, *rrow;     // permuted index of each local column and row
   double *cs0, *cs1, *rs0, *rs1;  // check sums of both candidates
   // FP64: c, x, xbar, order keys of the bounds.  Mixed: cf, dx, dxbar, lf, uf
@@ -103,6 +126,15 @@ struct Sm {  // shared-memory arrays of a block
   int32_t *rt;
   int32_t *cidx, *ridx;
   T *cval, *rval;
+};
+
+// What one group of blocks works on: a problem's slices, block `rank` of P
+// owning every P-th of them, and its ranges in the permuted index spaces.
+struct Share {
+  int c0, nc, r0, nr, stride;       // this block's slices: c0 + i stride, i < nc; rows alike
+  int cfirst, rfirst;               // the problem's first slices
+  int col0, ncol, row0, nrow;
+  int rank, P;
 };
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
@@ -119,24 +151,28 @@ __device__ __forceinline__ unsigned long long now_ns() {
   return t;
 }
 
-// Barrier over the P resident blocks of a cooperative launch: kBarLines arrival
-// counters that only grow, a 128-byte line each (152 arrivals at one address
-// cost 900 cycles more), block b on counter b mod kBarLines; one lane of warp 0
-// waits on each.  Block-wide barriers on both sides order the other threads'
-// accesses.  The wait is bounded: after kWaitNs the block gives up, and every
-// other block's wait runs out the same way.
-struct GridBar {
+// How the blocks of a group exchange xhat and y and wait for one another.
+// Grid: the vectors lie in global memory.  The barrier of a cooperative launch
+// is kBarLines arrival counters that only grow, a 128-byte line each (152
+// arrivals at one address cost 900 cycles more), block b on counter b mod
+// kBarLines; one lane of warp 0 waits on each.  Block-wide barriers on both
+// sides order the other threads' accesses.  The wait is bounded: after kWaitNs
+// the block gives up, and every other block's wait runs out the same way.
+template <typename T>
+struct GridLink {
+  static constexpr bool kCluster = false;
   unsigned *counter;
   unsigned gen;  // barriers passed since the counters were zero
   int32_t *dead;
+  T *gx, *gy;
+  __device__ __forceinline__ const T *x() const { return gx; }
+  __device__ __forceinline__ const T *y() const { return gy; }
+  __device__ __forceinline__ void put_x(int j, T v) const { gx[j] = v; }
+  __device__ __forceinline__ void put_y(int i, T v) const { gy[i] = v; }
   __device__ __forceinline__ void arrive() {
     __syncthreads();
     ++gen;
     if (threadIdx.x == 0) red_release(counter + (blockIdx.x % kBarLines) * 32);
-  }
-  __device__ __forceinline__ bool sync() {
-    arrive();
-    return wait();
   }
   __device__ __forceinline__ bool wait() {
     const int P = (int)gridDim.x, lane = (int)threadIdx.x;
@@ -160,47 +196,121 @@ struct GridBar {
     __syncthreads();
     return *(volatile int32_t *)dead == 0;
   }
+  __device__ __forceinline__ bool sync() {
+    arrive();
+    return wait();
+  }
+};
+
+__device__ __forceinline__ void put_shared(uint32_t addr, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+}
+__device__ __forceinline__ void put_shared(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+// Cluster: every block keeps whole copies of the two vectors in shared memory;
+// an owner stores its element into all of them (distributed shared memory) and
+// the hardware's cluster barrier orders the passes (500 cycles, no polling).
+template <typename T>
+struct ClusterLink {
+  static constexpr bool kCluster = true;
+  int C;
+  T *ex, *ey;  // copies, indexed by permuted column - col0 and row - row0
+  int col0, row0;
+  uint32_t ax, ay;  // their shared-memory addresses
+  __device__ __forceinline__ const T *x() const { return ex; }
+  __device__ __forceinline__ const T *y() const { return ey; }
+  __device__ __forceinline__ void put(uint32_t addr, T v) const {
+    for (int c = 0; c < C; ++c) {
+      uint32_t to;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(addr), "r"(c));
+      put_shared(to, v);
+    }
+  }
+  __device__ __forceinline__ void put_x(int j, T v) const {
+    if (C == 1) ex[j - col0] = v;
+    else put(ax + (uint32_t)sizeof(T) * (uint32_t)(j - col0), v);
+  }
+  __device__ __forceinline__ void put_y(int i, T v) const {
+    if (C == 1) ey[i - row0] = v;
+    else put(ay + (uint32_t)sizeof(T) * (uint32_t)(i - row0), v);
+  }
+  __device__ __forceinline__ void arrive() {
+    __syncthreads();
+    if (C > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  }
+  __device__ __forceinline__ bool wait() {
+    if (C > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    return true;
+  }
+  __device__ __forceinline__ bool sync() {
+    arrive();
+    return wait();
+  }
 };
 
 // Row sum of one slice, in the order of process_item: `a` is the lane's
 // starting value (-c or -b in the row's first lane), ip and vp the lane's
-// indices and values in shared memory.  All lanes of a row return its sum.
-// The gathers are plain loads: the barrier's acquire makes L1 safe to use.
-template <typename T>
+// indices and values.  All lanes of a row return its sum.  The gathers are
+// plain loads: the barrier's acquire makes L1 safe to use.  SHIFT: vec starts at
+// element `base` of the index space (padding, index 0, reads element base).
+template <bool SHIFT, typename T>
 __device__ __forceinline__ T slice_sum(T a, const int32_t *ip, const T *vp, int steps, int lg,
-                                       const T *vec) {
-  for (int t = 0; t < steps; t += kU) {
-    T g[kU];
+                                       const T *vec, int base) {
+  if constexpr (SHIFT) {  // streamed from global memory: indices and values load together
+    constexpr int U = 4;
+    for (int t = 0; t < steps; t += U) {
+      int j[U];
+      T c[U];
 #pragma unroll
-    for (int u = 0; u < kU; ++u)
-      if (t + u < steps) g[u] = vec[ip[kWarp * (t + u)]];
+      for (int u = 0; u < U; ++u)
+        if (t + u < steps) {
+          j[u] = __ldg(ip + kWarp * (t + u));
+          c[u] = __ldg(vp + kWarp * (t + u));
+        }
 #pragma unroll
-    for (int u = 0; u < kU; ++u)
-      if (t + u < steps) a = fma_t(vp[kWarp * (t + u)], g[u], a);
+      for (int u = 0; u < U; ++u)
+        if (t + u < steps) a = fma_t(c[u], vec[max(j[u] - base, 0)], a);
+    }
+  } else {
+    for (int t = 0; t < steps; t += kU) {
+      T g[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+        if (t + u < steps) g[u] = vec[ip[kWarp * (t + u)]];
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+        if (t + u < steps) a = fma_t(vp[kWarp * (t + u)], g[u], a);
+    }
   }
   for (int o = (1 << lg) >> 1; o > 0; o >>= 1) a += __shfl_xor_sync(kFull, a, o);
   return a;
 }
 
 // Sums of the check, both candidates at once, from plain arrays (written
-// before a grid barrier, whose acquire lets plain loads use L1) and FP64 values.
+// before a barrier, whose acquire lets plain loads use L1) and FP64 values;
+// sval: the resident values, or null to read them from global memory.  base: the
+// first element that the resident indices count from.
+template <int NT, bool RES>
 __device__ __forceinline__ void check_sums(const LSlice *sl, int count, const int32_t *sidx,
                                            const double *sval, const SellMat &A,
-                                           const double *v0, const double *v1, double *o0,
-                                           double *o1) {
+                                           int base, const double *v0, const double *v1,
+                                           double *o0, double *o1) {
   const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x >> 5;
-  for (int q = 0, i; (i = pick(q, warp)) < count; ++q) {
+  for (int q = 0, i; (i = pick<NT>(q, warp)) < count; ++q) {
     const LSlice s = sl[i];
     const int lg = s.lg(), steps = s.steps();
-    const int32_t *ip = sidx + s.soff + lane;
-    const double *vp = (sval ? sval + s.soff : A.val + A.info[s.gid].off) + lane;
+    const int64_t off = A.info[s.gid].off;
+    const int32_t *ip = (RES ? sidx + s.soff : A.idx + off) + lane;
+    const double *vp = (sval ? sval + s.soff : A.val + off) + lane;
     double a0 = 0.0, a1 = 0.0;
     for (int t = 0; t < steps; t += 4) {
       double g[4], h[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (t + u < steps) {
-          const int j = ip[kWarp * (t + u)];
+          const int j = ip[kWarp * (t + u)] + (RES ? base : 0);
           g[u] = v0[j];
           h[u] = v1[j];
         }
@@ -255,23 +365,24 @@ __device__ __forceinline__ double sum_parts(const double *part, int stride, int 
   return s;
 }
 
-// Local slices of one operator (every P-th of the global ones), most steps
-// first: records, and the numbers of local rows and elements.  One warp.
-__device__ void build_slices(const SellMat &A, int blk, int P, LSlice *sl, int32_t *nslot,
-                             int32_t *nelem) {
+// Local slices of one operator, most steps first: records, and the numbers of
+// local rows and elements.  One warp.
+template <bool RES>
+__device__ void build_slices(const SellMat &A, int first, int count, int stride, int pfirst,
+                             LSlice *sl, int32_t *nslot, int32_t *nelem) {
   const int lane = threadIdx.x & (kWarp - 1);
   int slot = 0, el = 0;
-  const int count = (A.nslices - blk + P - 1) / P;
   for (int i0 = 0; i0 < count; i0 += kWarp) {
     const int i = i0 + lane;
-    int rows = 0, steps = 0, lg = 0, rank = 0;
+    int rows = 0, steps = 0, lg = 0, rank = 0, goff = 0;
     if (i < count) {
-      const SliceInfo a = A.info[blk + i * P];
-      rows = A.info[blk + i * P + 1].row0 - a.row0;
+      const SliceInfo a = A.info[first + i * stride];
+      rows = A.info[first + i * stride + 1].row0 - a.row0;
       steps = a.len_g >> 3;
       lg = a.len_g & 7;
+      if (!RES) goff = (int)(a.off - A.info[pfirst].off);
       for (int j = 0; j < count; ++j) {
-        const int o = A.info[blk + j * P].len_g >> 3;
+        const int o = A.info[first + j * stride].len_g >> 3;
         rank += (o > steps || (o == steps && j < i)) ? 1 : 0;
       }
     }
@@ -285,8 +396,9 @@ __device__ void build_slices(const SellMat &A, int blk, int P, LSlice *sl, int32
       }
     }
     if (i < count)
-      sl[rank] = LSlice{el + kWarp * (pl - steps), slot + ps - rows,
-                        (uint32_t)steps << 16 | (uint32_t)lg << 8 | (uint32_t)rows, blk + i * P};
+      sl[rank] = LSlice{RES ? el + kWarp * (pl - steps) : goff, slot + ps - rows,
+                        (uint32_t)steps << 16 | (uint32_t)lg << 8 | (uint32_t)rows,
+                        first + i * stride};
     slot += __shfl_sync(kFull, ps, kWarp - 1);
     el += kWarp * __shfl_sync(kFull, pl, kWarp - 1);
   }
@@ -302,22 +414,27 @@ __device__ __forceinline__ unsigned char *carve(unsigned char *&p, size_t bytes)
   return q;
 }
 
-// Copies the local slices of one operator, and the permuted indices of their
-// rows, into shared memory.
-template <typename T>
-__device__ __forceinline__ void load_slices(const SellMat &A, const T *gval,
-                                            const LSlice *sl, int count, int32_t *row,
-                                            int32_t *sidx, T *sval) {
+// The permuted indices of the local rows, and (RES) the local slices' elements
+// into shared memory, their indices counted from `base` on (padding: 0).
+template <typename T, int NT, bool RES>
+__device__ __forceinline__ void load_slices(const SellMat &A, const T *gval, const LSlice *sl,
+                                            int count, int base, int32_t *row, int32_t *sidx,
+                                            T *sval) {
   const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x >> 5;
   constexpr int VC = 16 / sizeof(T);  // values per 16-byte chunk
-  for (int i = warp; i < count; i += kRW) {
+  for (int i = warp; i < count; i += NT / kWarp) {
     const LSlice s = sl[i];
     const SliceInfo g = A.info[s.gid];
     for (int r = lane; r < s.rows(); r += kWarp) row[s.slot0 + r] = g.row0 + r;
+    if (!RES) continue;
     const int len = s.steps() * kWarp;
     const int4 *gi = reinterpret_cast<const int4 *>(A.idx + g.off);
     int4 *si = reinterpret_cast<int4 *>(sidx + s.soff);
-    for (int e = lane; e < len / 4; e += kWarp) si[e] = __ldg(gi + e);
+    for (int e = lane; e < len / 4; e += kWarp) {
+      const int4 j = __ldg(gi + e);
+      si[e] = make_int4(max(j.x - base, 0), max(j.y - base, 0), max(j.z - base, 0),
+                        max(j.w - base, 0));
+    }
     const int4 *gv = reinterpret_cast<const int4 *>(gval + g.off);
     int4 *sv = reinterpret_cast<int4 *>(sval + s.soff);
     for (int e = lane; e < len / VC; e += kWarp) sv[e] = __ldg(gv + e);
@@ -327,54 +444,262 @@ __device__ __forceinline__ void load_slices(const SellMat &A, const T *gval,
 // Bytes of shared memory per local column and row.
 template <typename T>
 constexpr size_t col_bytes() {
-  return 4 + 16 + sizeof(T) * 2 + 8 + 2 * sizeof(T);
+  return sizeof(T) == 8 ? 4 + 8 + 8 + 8 + 16 : 4 + 4 + 4 + 8 + 8 + 16;
 }
 template <typename T>
 constexpr size_t row_bytes() {
-  return 4 + 16 + sizeof(T) * 2 + 8 + (sizeof(T) == 8 ? 4 : 8);
+  return sizeof(T) == 8 ? 4 + 8 + 8 + 8 + 4 : 4 + 4 + 4 + 8 + 8 + 16;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant__ ResidentArgs a) {
+// Mixed precision: the radius of a restart scales the next correction (mix_s),
+// whose data are rounded to FP32, so its last bits must not depend on the
+// kernel.  These sums of (z - z0)^2 over the columns and the rows repeat the
+// order of the per-pass kernels' check.
+//
+// Of the owned rows of one slice, lane by lane.
+__device__ __forceinline__ double slice_dist2(const SellMat &A, int slice, const double *z,
+                                              const double *z0, double q) {
+  const int lane = threadIdx.x & (kWarp - 1);
+  const SliceInfo a = A.info[slice];
+  const int lg = a.len_g & 7, row = a.row0 + (lane >> lg);
+  if ((lane & ((1 << lg) - 1)) == 0 && row < A.info[slice + 1].row0) {
+    const double d = z[row] - z0[row];
+    q = fma(d, d, q);
+  }
+  return q;
+}
+
+// Single problem (check_kernel, block_reduce_store_mask, check_finalize_kernel):
+// the check's blocks of 8 warps, their sums one entry each of out.
+template <int NT>
+__device__ __forceinline__ void radius_parts(const ResidentArgs &a, const Share &sh, double *red,
+                                             int cand, double *out) {
+  constexpr int G = NT / kBlock, W = kWarpsPerBlock;
+  const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x >> 5, g = warp / W, w = warp % W;
+  const int gc = a.cs.cols_grid, gr = a.cs.rows_grid;
+  for (int v0 = sh.rank * G; v0 < gc + gr; v0 += sh.P * G) {
+    const int v = v0 + g;
+    double q = 0.0;
+    if (v < gc) {
+      const double *x = cand ? a.v.x : a.v.xbar;
+      for (int it = v * W + w; it < a.AT.nslices; it += gc * W) q = slice_dist2(a.AT, it, x, a.v.x0, q);
+    } else if (v < gc + gr) {
+      const double *y = cand ? a.v.y : a.v.ybar;
+      for (int it = (v - gc) * W + w; it < a.A.nslices; it += gr * W)
+        q = slice_dist2(a.A, it, y, a.v.y0, q);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_down_sync(kFull, q, o);
+    if (lane == 0) red[warp] = q;
+    __syncthreads();
+    if (lane == 0 && w == 0 && v < gc + gr) {
+      double s = 0.0;
+      for (int i = 0; i < W; ++i) s += red[g * W + i];
+      __stcg(out + v, s);
+    }
+    __syncthreads();
+  }
+}
+
+// The sum of entries [lo, hi) of part (of n), by the first kBlock threads; all
+// threads of the block call it.
+__device__ __forceinline__ double radius_total(const double *part, int n, int lo, int hi,
+                                               double *red) {
+  const int tid = (int)threadIdx.x;
+  if (tid < kBlock) {
+    double s = 0.0;
+    for (int p = tid; p < n; p += kBlock) s += p >= lo && p < hi ? __ldcg(part + p) : 0.0;
+    red[tid] = s;
+  }
+  __syncthreads();
+  for (int o = kBlock / 2; o > 0; o >>= 1) {
+    if (tid < o) red[tid] += red[tid + o];
+    __syncthreads();
+  }
+  const double r = red[0];
+  __syncthreads();
+  return r;
+}
+
+// A batch's problem (b_check_kernel, b_finalize_kernel): chunks of 8 slices.
+template <int NT>
+__device__ __forceinline__ double radius_batch(const SellMat &A, int s0, int s1, const double *z,
+                                               const double *z0, double *red) {
+  constexpr int W = NT / kWarp;
+  const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x >> 5;
+  const int nch = (s1 - s0 + kCheckChunk - 1) / kCheckChunk;
+  double acc = 0.0;
+  for (int c0 = 0; c0 < nch; c0 += kWarp) {
+    for (int c = c0 + warp; c < min(nch, c0 + kWarp); c += W) {
+      double q = 0.0;
+      const int e = min(s1, s0 + (c + 1) * kCheckChunk);
+      for (int s = s0 + c * kCheckChunk; s < e; ++s) q = slice_dist2(A, s, z, z0, q);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(kFull, q, o);
+      if (lane == 0) red[c - c0] = q;
+    }
+    __syncthreads();
+    if (c0 + lane < nch) acc += red[lane];
+    __syncthreads();
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+  return acc;
+}
+
+__device__ __forceinline__ const float *values(const SellMat &A, float) { return A.valf; }
+__device__ __forceinline__ const double *values(const SellMat &A, double) { return A.val; }
+
+// ------------------------------------------------------- state of a problem
+
+// The single problem's state (DevState), its weights and trace.
+struct SingleIO {
+  static constexpr bool kBatch = false;
+  DevState *st;
+  double *w, *trace;
+  unsigned gen = 0;
+  __device__ __forceinline__ bool running() const { return st->status == kRunning; }
+  __device__ __forceinline__ int iterations() const { return st->K; }
+  __device__ void load(Scalars &c) const {
+    c = Scalars{st->tau,    st->sigma,      st->omega,  st->norm_b, st->norm_c,
+                st->tol,    st->beta,       st->rho_stored, st->last_r, st->mix_s,
+                st->t0,     st->restarts,   st->tau0,   st->fixed_len,
+                st->K,      st->scheme,     1,          st->returned};
+  }
+  __device__ void expired() const { st->status = kStatusTimeout; }
+  __device__ void record(const Header &h, int64_t t) const {
+    st->bar_gen = gen;
+    st->iters += h.sc.K;
+    st->checks += 1;
+    for (int i = 0; i < 5; ++i) {
+      st->kkt_a[i] = h.kkt[0][i];
+      st->kkt_c[i] = h.kkt[1][i];
+    }
+    st->returned = h.returned;
+    if (h.status != kRunning) {
+      st->status = h.status;
+      return;
+    }
+    if (trace && st->trace_count < st->trace_cap) {
+      double *row = trace + 6 * st->trace_count;
+      row[0] = (double)st->iters;
+      row[1] = h.rho;
+      row[2] = (double)h.restart;
+      row[3] = h.kkt[0][4];
+      row[4] = h.kkt[1][4];
+      row[5] = h.r;
+    }
+    st->trace_count += 1;
+    st->last_rho = h.rho;
+    st->last_r = h.r;
+    st->use_cur = h.use_cur;
+    st->restart_now = h.restart;
+    st->t0 = h.restart ? 0 : t;
+    if (h.restart) {
+      st->rho_stored = h.rho;
+      st->restarts += 1;
+      st->mix_s = h.mix_s;
+    }
+  }
+};
+
+// A problem of a batch (BInst): counters, restart rule and iteration limit as
+// in the batch's check chain (b_pre_check, b_finalize, b_decide).
+struct BatchIO {
+  static constexpr bool kBatch = true;
+  BInst *B;
+  BGlobal *G;
+  __device__ __forceinline__ bool running() const { return B->status == kRunning; }
+  __device__ __forceinline__ int iterations() const { return G->Kb; }
+  __device__ void load(Scalars &c) const {
+    c = Scalars{B->tau,   B->sigma,     B->omega,      B->norm_b, B->norm_c,
+                G->tol,   G->beta,      B->rho_stored, B->last_r, B->mix_s,
+                B->t0,    B->restarts,  B->tau0,       B->fixed_len,
+                G->Kb,    G->scheme,    B->since + G->Kb >= B->K ? 1 : 0, B->returned};
+  }
+  __device__ void expired() const {}
+  __device__ void record(const Header &h, int64_t t) const {
+    B->iters += h.sc.K;
+    B->since += h.sc.K;
+    B->due = h.sc.due;
+    B->restart_now = 0;
+    B->use_cur = 0;
+    if (h.sc.due) {
+      B->checks += 1;
+      for (int i = 0; i < 5; ++i) {
+        B->kkt_a[i] = h.kkt[0][i];
+        B->kkt_c[i] = h.kkt[1][i];
+      }
+      B->returned = h.returned;
+      if (h.status != kRunning) {
+        B->status = h.status;
+        return;
+      }
+      B->last_rho = h.rho;
+      B->last_r = h.r;
+      B->use_cur = h.use_cur;
+      B->restart_now = h.restart;
+      B->since = 0;
+    }
+    B->t0 = h.restart ? 0 : t;
+    if (h.restart) {
+      B->rho_stored = h.rho;
+      B->restarts += 1;
+      B->mix_s = h.mix_s;
+    }
+    if (B->iters >= B->iter_cap) B->status = kStatusIterLimit;  // the check's restart still happens
+    else atomicAdd(&G->running, 1);
+  }
+};
+
+// ------------------------------------------------------------------ the block
+//
+// K iterations and, when due, the check of one problem by the blocks of one
+// group.  T: float for mixed precision.  RES: the block's slices stay in shared
+// memory (else they are read from global memory in every pass).
+template <typename T, int NT, bool RES, class IO, class Link>
+__device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArgs &a,
+                                          const Share &sh, IO &io, Link &link) {
   constexpr bool MIX = sizeof(T) == 4;
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int P = (int)gridDim.x, blk = (int)blockIdx.x, tid = (int)threadIdx.x;
+  constexpr bool SHIFT = Link::kCluster && !RES;  // resident indices count from the problem's first
+  constexpr int W = NT / kWarp;
+  const int P = sh.P, tid = (int)threadIdx.x;
   const int lane = tid & (kWarp - 1), warp = tid >> 5;
-  DevState *st = a.st;
-  if (st->status != kRunning) return;
-  const int K = st->K;
-  const int nc = (a.AT.nslices - blk + P - 1) / P, nr = (a.A.nslices - blk + P - 1) / P;
+  const int nc = sh.nc, nr = sh.nr, K = io.iterations();
 
   // ---- layout of shared memory
   Sm<T> S;
   unsigned char *p = smem;
   S.h = (Header *)carve(p, sizeof(Header));
+  if (Link::kCluster) {  // at the same place in every block: owners store into all of them
+    S.ex = (T *)carve(p, sizeof(T) * sh.ncol);
+    S.ey = (T *)carve(p, sizeof(T) * sh.nrow);
+  }
   S.cs = (LSlice *)carve(p, sizeof(LSlice) * nc);
   S.rs = (LSlice *)carve(p, sizeof(LSlice) * nr);
-  S.red = (double *)carve(p, sizeof(double) * kRW * 32);
+  S.red = (double *)carve(p, sizeof(double) * W * 32);
   S.tot = (double *)carve(p, sizeof(double) * 32);
   S.nw = (double *)carve(p, sizeof(double) * 8);
   S.w = (double *)carve(p, sizeof(double) * K);
-  if (warp == 0) build_slices(a.AT, blk, P, S.cs, &S.h->ncl, &S.h->nce);
-  else if (warp == 1) build_slices(a.A, blk, P, S.rs, &S.h->nrl, &S.h->nre);
-  if (warp == 2) {
-    const double sw = sqrt(st->omega);
-    if (lane == 0) {
-      S.h->dead = 0;
-      S.h->sw = sw;
-      S.h->isw = 1.0 / sw;
-      S.h->inv = MIX ? 1.0 / st->mix_s : 1.0;
-    }
+  if (warp == 0)
+    build_slices<RES>(a.AT, sh.c0, nc, sh.stride, sh.cfirst, S.cs, &S.h->ncl, &S.h->nce);
+  else if (warp == 1)
+    build_slices<RES>(a.A, sh.r0, nr, sh.stride, sh.rfirst, S.rs, &S.h->nrl, &S.h->nre);
+  else if (warp == 2 && lane == 0) {
+    Scalars sc;
+    io.load(sc);
+    S.h->sc = sc;
+    S.h->dead = 0;
+    const double sw = sqrt(sc.omega);
+    S.h->sw = sw;
+    S.h->isw = 1.0 / sw;
+    S.h->inv = MIX ? 1.0 / sc.mix_s : 1.0;
   }
-  for (int k = tid; k < K; k += kRT) S.w[k] = a.w[k];
   __syncthreads();
   const int ncl = S.h->ncl, nrl = S.h->nrl;
+  for (int k = tid; k < K; k += NT) S.w[k] = 1.0 / (double)(S.h->sc.t0 + k + 1);
   S.crow = (int32_t *)carve(p, 4 * (size_t)ncl);
   S.rrow = (int32_t *)carve(p, 4 * (size_t)nrl);
-  S.cs0 = (double *)carve(p, 8 * (size_t)ncl);
-  S.cs1 = (double *)carve(p, 8 * (size_t)ncl);
-  S.rs0 = (double *)carve(p, 8 * (size_t)nrl);
-  S.rs1 = (double *)carve(p, 8 * (size_t)nrl);
   S.c = (T *)carve(p, sizeof(T) * ncl);
   S.x = (T *)carve(p, sizeof(T) * ncl);
   S.xb = (double *)carve(p, 8 * (size_t)ncl);
@@ -386,54 +711,74 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
     S.uf = (float *)carve(p, 4 * (size_t)ncl);
     S.lo = (float *)carve(p, 4 * (size_t)nrl);
     S.hi = (float *)carve(p, 4 * (size_t)nrl);
+    S.cs0 = (double *)carve(p, 8 * (size_t)ncl);
+    S.cs1 = (double *)carve(p, 8 * (size_t)ncl);
+    S.rs0 = (double *)carve(p, 8 * (size_t)nrl);
+    S.rs1 = (double *)carve(p, 8 * (size_t)nrl);
   } else {
     S.lk = (long long *)carve(p, 8 * (size_t)ncl);
     S.uk = (long long *)carve(p, 8 * (size_t)ncl);
     S.rt = (int32_t *)carve(p, 4 * (size_t)nrl);
+    // the check comes after the state has gone back to global memory
+    S.cs0 = S.xb;
+    S.cs1 = S.c;
+    S.rs0 = S.yb;
+    S.rs1 = S.b;
   }
-  S.cidx = (int32_t *)carve(p, 4 * (size_t)S.h->nce);
-  S.cval = (T *)carve(p, sizeof(T) * S.h->nce);
-  S.ridx = (int32_t *)carve(p, 4 * (size_t)S.h->nre);
-  S.rval = (T *)carve(p, sizeof(T) * S.h->nre);
+  const int32_t *cidx, *ridx;  // indexed by LSlice::soff
+  const T *cval, *rval;
+  if constexpr (RES) {
+    S.cidx = (int32_t *)carve(p, 4 * (size_t)S.h->nce);
+    S.cval = (T *)carve(p, sizeof(T) * S.h->nce);
+    S.ridx = (int32_t *)carve(p, 4 * (size_t)S.h->nre);
+    S.rval = (T *)carve(p, sizeof(T) * S.h->nre);
+    cidx = S.cidx;
+    cval = S.cval;
+    ridx = S.ridx;
+    rval = S.rval;
+  } else {
+    S.cidx = S.ridx = nullptr;
+    S.cval = S.rval = nullptr;
+    const int64_t oc = a.AT.info[sh.cfirst].off, orr = a.A.info[sh.rfirst].off;
+    cidx = a.AT.idx + oc;
+    cval = values(a.AT, T(0)) + oc;
+    ridx = a.A.idx + orr;
+    rval = values(a.A, T(0)) + orr;
+  }
 
   // ---- owned state
-  const T *gvc, *gvr;
-  if constexpr (MIX) {
-    gvc = a.AT.valf;
-    gvr = a.A.valf;
-  } else {
-    gvc = a.AT.val;
-    gvr = a.A.val;
-  }
-  load_slices<T>(a.AT, gvc, S.cs, nc, S.crow, S.cidx, S.cval);
-  load_slices<T>(a.A, gvr, S.rs, nr, S.rrow, S.ridx, S.rval);
+  load_slices<T, NT, RES>(a.AT, values(a.AT, T(0)), S.cs, nc, sh.row0, S.crow, S.cidx, S.cval);
+  load_slices<T, NT, RES>(a.A, values(a.A, T(0)), S.rs, nr, sh.col0, S.rrow, S.ridx, S.rval);
   __syncthreads();
-  T *gx, *gy;  // the exchanged vectors
-  if constexpr (MIX) {
-    gx = a.mv.dxhat;
-    gy = a.mv.dy;
+  if constexpr (Link::kCluster) {
+    link.ex = S.ex;
+    link.ey = S.ey;
+    link.ax = (uint32_t)__cvta_generic_to_shared(S.ex);
+    link.ay = (uint32_t)__cvta_generic_to_shared(S.ey);
+    for (int i = tid; i < sh.nrow; i += NT) {
+      if constexpr (MIX) S.ey[i] = a.mv.dy[sh.row0 + i];
+      else S.ey[i] = a.v.y[sh.row0 + i];
+    }
   } else {
-    gx = a.v.xhat;
-    gy = a.v.y;
+    link.gen = io.st->bar_gen;
+    link.dead = &S.h->dead;
   }
-  for (int s = tid; s < nrl; s += kRT) {
+  for (int s = tid; s < nrl; s += NT) {
     const int i = S.rrow[s];
-    T y;
     if constexpr (MIX) {
-      y = a.mv.dy[i];
+      S.y[s] = a.mv.dy[i];
       S.b[s] = a.mv.bf[i];
       S.yb[s] = a.mv.dybar[i];
       S.lo[s] = a.mv.ylo[i];
       S.hi[s] = a.mv.yhi[i];
     } else {
-      y = a.v.y[i];
+      S.y[s] = a.v.y[i];
       S.b[s] = a.v.b[i];
       S.yb[s] = a.v.ybar[i];
       S.rt[s] = (int)a.v.row_type[i];
     }
-    S.y[s] = y;
   }
-  for (int s = tid; s < ncl; s += kRT) {
+  for (int s = tid; s < ncl; s += NT) {
     const int j = S.crow[s];
     if constexpr (MIX) {
       S.c[s] = a.mv.cf[j];
@@ -449,21 +794,23 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
       S.uk[s] = a.v.ubk[j];
     }
   }
-  const T tau = (T)st->tau, sigma = (T)st->sigma;
-  GridBar bar{a.bar, st->bar_gen, &S.h->dead};
-  __syncthreads();
+  const T tau = (T)S.h->sc.tau, sigma = (T)S.h->sc.sigma;
+  // a cluster's blocks store into one another's copies only once all of them
+  // have started and filled theirs
+  if (Link::kCluster) link.sync();
+  else __syncthreads();
 
   // ---- K iterations.  The averages, which nothing waits for, are updated
   // between a barrier's arrival and its wait.
   bool lost = false;
   for (int k = 0; k < K; ++k) {
     const double w = S.w[k];
-    for (int q = 0, i; (i = pick(q, warp)) < nc; ++q) {
+    for (int q = 0, i; (i = pick<NT>(q, warp)) < nc; ++q) {
       const LSlice sl = S.cs[i];
       const int lg = sl.lg(), r = lane >> lg, s = sl.slot0 + r;
       const bool owner = (lane & ((1 << lg) - 1)) == 0 && r < sl.rows();
-      const T neg_g = slice_sum<T>(owner ? -S.c[s] : T(0), S.cidx + sl.soff + lane,
-                                   S.cval + sl.soff + lane, sl.steps(), lg, gy);
+      const T neg_g = slice_sum<SHIFT>(owner ? -S.c[s] : T(0), cidx + sl.soff + lane,
+                                       cval + sl.soff + lane, sl.steps(), lg, link.y(), sh.row0);
       if (owner) {
         const T x = S.x[s];
         T xn;
@@ -476,25 +823,25 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
           key = key > uk ? uk : key;
           xn = __longlong_as_double(ord_key(key));
         }
-        gx[S.crow[s]] = fma_t(T(2), xn, -x);
+        link.put_x(S.crow[s], fma_t(T(2), xn, -x));
         S.x[s] = xn;
       }
     }
-    bar.arrive();
-    for (int s = tid; s < ncl; s += kRT) {
+    link.arrive();
+    for (int s = tid; s < ncl; s += NT) {
       const double xb = S.xb[s];
       S.xb[s] = fma(w, (double)S.x[s] - xb, xb);
     }
-    if (!bar.wait()) {
+    if (!link.wait()) {
       lost = true;
       break;
     }
-    for (int q = 0, i; (i = pick(q, warp)) < nr; ++q) {
+    for (int q = 0, i; (i = pick<NT>(q, warp)) < nr; ++q) {
       const LSlice sl = S.rs[i];
       const int lg = sl.lg(), r = lane >> lg, s = sl.slot0 + r;
       const bool owner = (lane & ((1 << lg) - 1)) == 0 && r < sl.rows();
-      const T res = slice_sum<T>(owner ? -S.b[s] : T(0), S.ridx + sl.soff + lane,
-                                 S.rval + sl.soff + lane, sl.steps(), lg, gx);
+      const T res = slice_sum<SHIFT>(owner ? -S.b[s] : T(0), ridx + sl.soff + lane,
+                                     rval + sl.soff + lane, sl.steps(), lg, link.x(), sh.col0);
       if (owner) {
         const T y = S.y[s];
         T yn;
@@ -507,25 +854,25 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
           else if (t == 2 && bits > 0) bits = 0;
           yn = __longlong_as_double(bits);
         }
-        gy[S.rrow[s]] = yn;
+        link.put_y(S.rrow[s], yn);
         S.y[s] = yn;
       }
     }
-    if (k + 1 < K) bar.arrive();  // the barrier after the publication covers the last pass
+    if (k + 1 < K) link.arrive();  // the barrier after the publication covers the last pass
     else __syncthreads();
-    for (int s = tid; s < nrl; s += kRT) {
+    for (int s = tid; s < nrl; s += NT) {
       const double yb = S.yb[s];
       S.yb[s] = fma(w, (double)S.y[s] - yb, yb);
     }
-    if (k + 1 < K && !bar.wait()) {
+    if (k + 1 < K && !link.wait()) {
       lost = true;
       break;
     }
   }
 
-  // ---- publish the FP64 iterate and average
+  // ---- publish the iterate and the average (in mixed precision also in FP64)
   const double inv = S.h->inv;
-  for (int s = tid; s < ncl; s += kRT) {
+  for (int s = tid; s < ncl; s += NT) {
     const int j = S.crow[s];
     if constexpr (MIX) {
       a.mv.dx[j] = S.x[s];
@@ -538,9 +885,10 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
       a.v.xbar[j] = S.xb[s];
     }
   }
-  for (int s = tid; s < nrl; s += kRT) {
+  for (int s = tid; s < nrl; s += NT) {
     const int i = S.rrow[s];
     if constexpr (MIX) {
+      a.mv.dy[i] = S.y[s];
       a.mv.dybar[i] = S.yb[s];
       const int t = a.v.row_type[i];
       const double lo = (t == 1) ? 0.0 : -INFINITY, hi = (t == 2) ? 0.0 : INFINITY;
@@ -548,34 +896,48 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
       a.v.y[i] = fmin(fmax(fma((double)S.y[s], inv, y0), lo), hi);
       a.v.ybar[i] = fmin(fmax(fma(S.yb[s], inv, y0), lo), hi);
     } else {
+      a.v.y[i] = S.y[s];
       a.v.ybar[i] = S.yb[s];
     }
   }
-  if (lost || !bar.sync()) {
-    if (tid == 0) st->status = kStatusTimeout;
+  if (lost || !link.sync()) {
+    if (tid == 0) io.expired();
+    return;
+  }
+  const int64_t t = S.h->sc.t0 + K;
+  if (!S.h->sc.due) {
+    if (sh.rank == 0 && tid == 0) {
+      S.h->restart = 0;
+      io.record(*S.h, t);
+    }
     return;
   }
 
   // ---- check: A^T [ybar, y], A [xbar, x] and their epilogues
-  const int scheme = st->scheme;
+  const int scheme = S.h->sc.scheme;
   const bool gap_a = scheme == kSchemeAdaptive || scheme == kSchemeFlexible;
   const bool gap_c = scheme == kSchemeFlexible;
-  const double om = st->omega;
   const GapOut go[2] = {GapOut{a.cs.keys[0], a.cs.d2[0], a.cs.g2[0], a.cs.gd[0]},
                         GapOut{a.cs.keys[1], a.cs.d2[1], a.cs.g2[1], a.cs.gd[1]}};
   {
     const double *sc = nullptr, *sr = nullptr;
-    if constexpr (!MIX) {
+    if constexpr (!MIX && RES) {
       sc = S.cval;
       sr = S.rval;
     }
-    check_sums(S.cs, nc, S.cidx, sc, a.AT, a.v.ybar, a.v.y, S.cs0, S.cs1);
-    check_sums(S.rs, nr, S.ridx, sr, a.A, a.v.xbar, a.v.x, S.rs0, S.rs1);
+    check_sums<NT, RES>(S.cs, nc, S.cidx, sc, a.AT, sh.row0, a.v.ybar, a.v.y, S.cs0, S.cs1);
+    check_sums<NT, RES>(S.rs, nr, S.ridx, sr, a.A, sh.col0, a.v.xbar, a.v.x, S.rs0, S.rs1);
   }
   __syncthreads();
   // owned columns, then (from a whole warp on) owned rows, one per thread
   const int rfirst = (ncl + kWarp - 1) & ~(kWarp - 1), nown = rfirst + nrl;
-  const int busy = min(kRW, (nown + kWarp - 1) / kWarp);
+  const int busy = min(W, (nown + kWarp - 1) / kWarp);
+  double *part = a.part + (size_t)P * kResPart * (blockIdx.x / P);
+  const int ncand = gap_c ? 2 : gap_a ? 1 : 0;
+  const int nrad = a.cs.cols_grid + a.cs.rows_grid;
+  if (MIX && !IO::kBatch)
+    for (int c = 0; c < ncand; ++c)
+      radius_parts<NT>(a, sh, S.red, c, a.rpart + (size_t)c * nrad);
   if (warp < busy) {
     CheckColsEpi ce{};
     CheckRowsEpi re{};
@@ -584,7 +946,7 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
     re.off = a.n;
 #pragma unroll
     for (int i = 0; i < NQ; ++i) ce.q[i] = 0.0;
-    for (int s = tid; s < ncl; s += kRT) {
+    for (int s = tid; s < ncl; s += NT) {
       const int j = S.crow[s];
       const CheckColsEpi::Pre pre{a.v.c[j], a.v.lb[j], a.v.ub[j], 0.0, 0.0, a.v.x0[j]};
       const bool lf = dbits(pre.lb) != kNegInfBits, uf = dbits(pre.ub) != kPosInfBits;
@@ -602,7 +964,7 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
     }
 #pragma unroll
     for (int i = 0; i < NQ; ++i) re.q[i] = ce.q[i];
-    for (int e = tid; e < nown; e += kRT) {
+    for (int e = tid; e < nown; e += NT) {
       if (e < rfirst) continue;
       const int s = e - rfirst, i = S.rrow[s];
       const CheckRowsEpi::Pre pre{a.v.b[i], 0.0, 0.0, a.v.y0[i], (int)a.v.row_type[i]};
@@ -618,7 +980,7 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
                    go[1]);
       if (!(finite_d(ax_a) && finite_d(ax_c) && finite_d(ya) && finite_d(yc))) re.q[Q_BAD] = 1.0;
     }
-    // block sums, then grid sums
+    // sums of the warp, of the block, of the group
     double u[16], v[4];
 #pragma unroll
     for (int i = 0; i < 16; ++i) u[i] = re.q[i];
@@ -634,39 +996,57 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
   if (tid < NQ) {
     double s = 0.0;
     for (int i = 0; i < busy; ++i) s += S.red[i * 32 + tid];
-    __stcg(a.part + (size_t)blk * kResPart + tid, s);
+    if (P > 1) __stcg(part + (size_t)sh.rank * kResPart + tid, s);
+    else S.tot[tid] = s;
   }
-  // the state that the decision needs, read before the last barrier that every
-  // block passes: block 0 writes it after that
-  const double norm_b = st->norm_b, norm_c = st->norm_c, tol = st->tol, last_r = st->last_r,
-               beta = st->beta, rho_stored = st->rho_stored, mix_old = st->mix_s;
-  const int64_t t0 = st->t0, restarts = st->restarts, tau0 = st->tau0, fixed_len = st->fixed_len;
-  const int was_returned = st->returned;
-  if (!bar.sync()) {
-    if (tid == 0) st->status = kStatusTimeout;
-    return;
-  }
-  for (int i = warp; i < NQ; i += kRW) {
-    const double s = sum_parts(a.part, kResPart, i, P);
-    if (lane == 0) S.tot[i] = s;
+  if (P > 1) {
+    if (!link.sync()) {
+      if (tid == 0) io.expired();
+      return;
+    }
+    for (int i = warp; i < NQ; i += W) {
+      const double s = sum_parts(part, kResPart, i, P);
+      if (lane == 0) S.tot[i] = s;
+    }
   }
   __syncthreads();
 
+  if constexpr (MIX) {
+    for (int c = 0; c < ncand; ++c) {
+      double rx, ry;
+      if constexpr (IO::kBatch) {
+        const BInst &B = *io.B;
+        rx = radius_batch<NT>(a.AT, B.cs0, B.cs1, c ? a.v.x : a.v.xbar, a.v.x0, S.red);
+        ry = radius_batch<NT>(a.A, B.rs0, B.rs1, c ? a.v.y : a.v.ybar, a.v.y0, S.red);
+      } else {
+        const double *rp = a.rpart + (size_t)c * nrad;
+        rx = radius_total(rp, nrad, 0, a.cs.cols_grid, S.red);
+        ry = radius_total(rp, nrad, a.cs.cols_grid, nrad, S.red);
+      }
+      if (tid == 0) {
+        S.tot[c ? Q_RRX_C : Q_RRX_A] = rx;
+        S.tot[c ? Q_RRY_C : Q_RRY_A] = ry;
+      }
+    }
+    __syncthreads();
+  }
+
   // ---- termination and search setup: lane 0 for the average, lane 1 for the
-  // current iterate; every block decides from the same sums, block 0 records
+  // current iterate; every block decides from the same sums, one records
   const double *tot = S.tot;
   if (warp == 0) {
+    const Scalars &sc = S.h->sc;
     const int c = lane & 1;
     double k5[5];
-    kkt_from(tot, Q_RP2_A + c, Q_RD2_A + c, Q_POBJ_A + c, Q_DOBJ_A + c, norm_b, norm_c, k5);
+    kkt_from(tot, Q_RP2_A + c, Q_RD2_A + c, Q_POBJ_A + c, Q_DOBJ_A + c, sc.norm_b, sc.norm_c, k5);
     const double rel = k5[4], rel_a = __shfl_sync(kFull, rel, 0), rel_c = __shfl_sync(kFull, rel, 1);
     int status = kRunning, returned = 0;
     if (tot[Q_BAD] > 0.0 || !isfinite(rel_a) || !isfinite(rel_c)) {
       status = kStatusNumerical;
-      returned = was_returned;
-    } else if (rel_a <= tol) {
+      returned = sc.returned;
+    } else if (rel_a <= sc.tol) {
       status = kStatusOK;
-    } else if (rel_c <= tol) {
+    } else if (rel_c <= sc.tol) {
       status = kStatusOK;
       returned = 1;
     } else {
@@ -675,6 +1055,7 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
     double r2 = 0.0, rho_r = 0.0;
     int done = 1;
     if (status == kRunning && (c ? gap_c : gap_a)) {
+      const double om = sc.omega;
       const double r = sqrt(om * tot[c ? Q_RRX_C : Q_RRX_A] + tot[c ? Q_RRY_C : Q_RRY_A] / om);
       r2 = r * r;
       done = (r == 0.0);
@@ -719,8 +1100,8 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
           u[2] += in || key == kNoKey ? 0.0 : g2;
           cnt += in ? 1 : 0;
         };
-        for (int s = tid; s < ncl; s += kRT) add(S.crow[s]);
-        for (int e = tid; e < nown; e += kRT)
+        for (int s = tid; s < ncl; s += NT) add(S.crow[s]);
+        for (int e = tid; e < nown; e += NT)
           if (e >= rfirst) add((int64_t)a.n + S.rrow[e - rfirst]);
         const double su = warp_sum_multi<4>(u);
         cnt = __reduce_add_sync(kFull, cnt);
@@ -729,19 +1110,22 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
     }
     __syncthreads();
     // two buffers in turn: a block may still read the last step's sums
-    double *np = a.npart + (size_t)(step & 1) * P * 8;
+    double *np = a.npart + (size_t)(blockIdx.x / P) * 2 * P * 8 + (size_t)(step & 1) * P * 8;
     if (tid < 8 && !(tid < 4 ? done0 : done1)) {
       double s = 0.0;
       for (int i = 0; i < busy; ++i) s += S.red[i * 32 + tid];
-      __stcg(np + (size_t)blk * 8 + tid, s);
+      if (P > 1) __stcg(np + (size_t)sh.rank * 8 + tid, s);
+      else S.nw[tid] = s;
     }
-    if (!bar.sync()) {
-      if (tid == 0) st->status = kStatusTimeout;
-      return;
-    }
-    if (warp < 8 && !(warp < 4 ? done0 : done1)) {
-      const double s = sum_parts(np, 8, warp, P);
-      if (lane == 0) S.nw[warp] = s;
+    if (P > 1) {
+      if (!link.sync()) {
+        if (tid == 0) io.expired();
+        return;
+      }
+      if (warp < 8 && !(warp < 4 ? done0 : done1)) {
+        const double s = sum_parts(np, 8, warp, P);
+        if (lane == 0) S.nw[warp] = s;
+      }
     }
     __syncthreads();
     if (warp == 0 && lane < 2 && !(lane ? done1 : done0)) {
@@ -765,12 +1149,11 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
   }
 
   // ---- restart decision (Eq. adaptive-restart-scheme / flexible / fixed)
-  const int status = S.h->status;
-  const int64_t t = t0 + K;
   if (tid == 0) {
-    double rho = NAN, r = last_r;
+    const Scalars &sc = S.h->sc;
+    double rho = NAN, r = sc.last_r;
     int use_cur = 0, restart = 0;
-    if (status == kRunning) {
+    if (S.h->status == kRunning) {
       if (gap_a) {
         r = sqrt(S.h->r2[0]);
         rho = S.h->r2[0] > 0.0 ? S.h->rho_r[0] / r : 0.0;
@@ -783,63 +1166,31 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
             r = rc;
           }
         }
-        restart = (restarts == 0) ? (t >= tau0) : (rho <= beta * rho_stored);
+        restart = (sc.restarts == 0) ? (t >= sc.tau0) : (rho <= sc.beta * sc.rho_stored);
       } else if (scheme == kSchemeFixed) {
-        restart = (t >= fixed_len);
+        restart = (t >= sc.fixed_len);
       }
     }
     S.h->rho = rho;
     S.h->r = r;
     S.h->use_cur = use_cur;
     S.h->restart = restart;
-    S.h->mix_s = (restart && MIX && r > 0.0 && isfinite(r)) ? fmin(1.0 / r, 1e12) : mix_old;
+    S.h->mix_s = (restart && MIX && r > 0.0 && isfinite(r)) ? fmin(1.0 / r, 1e12) : sc.mix_s;
+    if (sh.rank == 0) {
+      if constexpr (!Link::kCluster) io.gen = link.gen;
+      io.record(*S.h, t);
+    }
   }
   __syncthreads();
   const int use_cur = S.h->use_cur, restart = S.h->restart;
   const double mix_s = S.h->mix_s;
-  const int64_t t0n = restart ? 0 : t;
-  if (blk == 0) {
-    if (tid == 0) {
-      st->bar_gen = bar.gen;
-      st->iters += K;
-      st->checks += 1;
-      for (int i = 0; i < 5; ++i) {
-        st->kkt_a[i] = S.h->kkt[0][i];
-        st->kkt_c[i] = S.h->kkt[1][i];
-      }
-      st->returned = S.h->returned;
-      if (status != kRunning) {
-        st->status = status;
-      } else {
-        if (a.trace && st->trace_count < st->trace_cap) {
-          double *row = a.trace + 6 * st->trace_count;
-          row[0] = (double)st->iters;
-          row[1] = S.h->rho;
-          row[2] = (double)restart;
-          row[3] = S.h->kkt[0][4];
-          row[4] = S.h->kkt[1][4];
-          row[5] = S.h->r;
-        }
-        st->trace_count += 1;
-        st->last_rho = S.h->rho;
-        st->last_r = S.h->r;
-        st->use_cur = use_cur;
-        st->restart_now = restart;
-        st->t0 = t0n;
-        if (restart) {
-          st->rho_stored = S.h->rho;
-          st->restarts += 1;
-          st->mix_s = mix_s;
-        }
-      }
-    }
-    if (status == kRunning)
-      for (int k = tid; k < K; k += kRT) a.w[k] = 1.0 / (double)(t0n + k + 1);
-  }
-  if (status != kRunning || (!restart && !use_cur)) return;
+  if (S.h->status != kRunning) return;
+  if (sh.rank == 0 && a.w)  // the next block's weights, for iterations outside this kernel
+    for (int k = tid; k < K; k += NT) a.w[k] = 1.0 / (double)((restart ? 0 : t) + k + 1);
+  if (!restart && !use_cur) return;
 
   // ---- restart (or the flexible scheme's replacement of the average), owned part
-  for (int s = tid; s < ncl; s += kRT) {
+  for (int s = tid; s < ncl; s += NT) {
     const int j = S.crow[s];
     const double x = (use_cur ? a.v.x : a.v.xbar)[j];
     a.v.xbar[j] = x;
@@ -860,7 +1211,7 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
       }
     }
   }
-  for (int s = tid; s < nrl; s += kRT) {
+  for (int s = tid; s < nrl; s += NT) {
     const int i = S.rrow[s];
     const double y = (use_cur ? a.v.y : a.v.ybar)[i];
     a.v.ybar[i] = y;
@@ -884,19 +1235,93 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
   }
 }
 
+// One problem over the whole grid (cooperative launch).
+template <typename T>
+__global__ void __launch_bounds__(kGridThreads, 1)
+    resident_kernel(const __grid_constant__ ResidentArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  SingleIO io{a.st, a.w, a.trace};
+  if (!io.running()) return;
+  const int P = (int)gridDim.x, b = (int)blockIdx.x;
+  const Share sh{b, (a.AT.nslices - b + P - 1) / P, b, (a.A.nslices - b + P - 1) / P, P, 0, 0,
+                 0, a.n, 0, a.m, b, P};
+  GridLink<T> link{a.bar, 0u, nullptr, nullptr, nullptr};
+  if constexpr (sizeof(T) == 4) {
+    link.gx = a.mv.dxhat;
+    link.gy = a.mv.dy;
+  } else {
+    link.gx = a.v.xhat;
+    link.gy = a.v.y;
+  }
+  run_block<T, kGridThreads, true>(smem, a, sh, io, link);
+}
+
+// One problem per cluster of a.cluster blocks: the single problem, or the
+// problems of a batch.
+template <typename T, bool RES, class IO>
+__global__ void __launch_bounds__(kClusterThreads, RES ? 2 : 4)
+    cluster_kernel(const __grid_constant__ ResidentArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int C = a.cluster, rank = (int)blockIdx.x % C;
+  ClusterLink<T> link{};
+  link.C = C;
+  if constexpr (std::is_same<IO, SingleIO>::value) {
+    SingleIO io{a.st, a.w, a.trace};
+    if (!io.running()) return;
+    const Share sh{rank, (a.AT.nslices - rank + C - 1) / C, rank, (a.A.nslices - rank + C - 1) / C,
+                   C, 0, 0, 0, a.n, 0, a.m, rank, C};
+    run_block<T, kClusterThreads, RES>(smem, a, sh, io, link);
+  } else {
+    BatchIO io{a.inst + blockIdx.x / C, a.glob};
+    if (!io.running()) return;
+    const BInst &B = *io.B;
+    const Share sh{B.cs0 + rank, (B.cs1 - B.cs0 - rank + C - 1) / C,
+                   B.rs0 + rank, (B.rs1 - B.rs0 - rank + C - 1) / C,
+                   C, B.cs0, B.rs0, B.col0, B.ncol, B.row0, B.nrow, rank, C};
+    link.col0 = sh.col0;
+    link.row0 = sh.row0;
+    run_block<T, kClusterThreads, RES>(smem, a, sh, io, link);
+  }
+}
+
+template <typename F>
+bool set_smem(F *kernel, int bytes) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) ==
+      cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
+}
+
+// The cluster kernel of a precision, residency and kind of problem.
+using ClusterKernel = void (*)(ResidentArgs);
+ClusterKernel cluster_of(bool mixed, bool res, bool batch) {
+  static const ClusterKernel k[8] = {
+      cluster_kernel<double, false, SingleIO>, cluster_kernel<double, false, BatchIO>,
+      cluster_kernel<double, true, SingleIO>,  cluster_kernel<double, true, BatchIO>,
+      cluster_kernel<float, false, SingleIO>,  cluster_kernel<float, false, BatchIO>,
+      cluster_kernel<float, true, SingleIO>,   cluster_kernel<float, true, BatchIO>};
+  return k[(mixed ? 4 : 0) + (res ? 2 : 0) + (batch ? 1 : 0)];
+}
+
 }  // namespace
 
-// Bytes of shared memory of a block that owns nc + nr slices with ncl columns and nrl rows,
-// without resident elements (the carving of resident_kernel).
-size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed) {
+// Bytes of shared memory of a block that owns nc + nr slices with ncl columns and nrl rows and
+// (cluster kernel) copies of ncol and nrow exchanged elements, without resident elements (the
+// carving of run_block).
+size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed, int ncol,
+                            int nrow) {
   const size_t lists = sizeof(LSlice) * ((size_t)nc + nr);
   const size_t state = mixed ? col_bytes<float>() * ncl + row_bytes<float>() * nrl
                              : col_bytes<double>() * ncl + row_bytes<double>() * nrl;
-  return sizeof(Header) + lists + state + sizeof(double) * (kRW * 32 + 40 + (size_t)K) + 16 * 26;
+  const size_t copies = (mixed ? 4 : 8) * ((size_t)ncol + nrow);
+  const int warps = (ncol > 0 ? kClusterThreads : kGridThreads) / kWarp;
+  return sizeof(Header) + lists + state + copies + sizeof(double) * (warps * 32 + 40 + (size_t)K) +
+         16 * 28;
 }
 
-// Largest dynamic shared memory of the kernel on the current device; 0 when it cannot launch
-// cooperatively.
+// Largest dynamic shared memory of the kernels on the current device; 0 when it cannot launch
+// them (no cooperative launch).
 size_t resident_smem_limit(int device, bool mixed) {
   int coop = 0, optin = 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess ||
@@ -906,25 +1331,20 @@ size_t resident_smem_limit(int device, bool mixed) {
     cudaGetLastError();
     return 0;
   }
-  const cudaError_t e =
-      mixed ? cudaFuncSetAttribute(resident_kernel<float>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, optin)
-            : cudaFuncSetAttribute(resident_kernel<double>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
+  if (!(mixed ? set_smem(resident_kernel<float>, optin) : set_smem(resident_kernel<double>, optin)))
     return 0;
-  }
+  for (int i = 0; i < 4; ++i)
+    if (!set_smem(cluster_of(mixed, i & 1, i & 2), optin)) return 0;
   return (size_t)optin;
 }
 
 // Whether P blocks with smem bytes each can be resident at once.
 bool resident_fits(int P, int nsm, size_t smem, bool mixed) {
   int per_sm = 0;
-  const cudaError_t e =
-      mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, resident_kernel<float>, kRT, smem)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, resident_kernel<double>, kRT,
-                                                            smem);
+  const cudaError_t e = mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                                    &per_sm, resident_kernel<float>, kGridThreads, smem)
+                              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                                    &per_sm, resident_kernel<double>, kGridThreads, smem);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -936,7 +1356,7 @@ cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixe
                             cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)P);
-  cfg.blockDim = dim3(kRT);
+  cfg.blockDim = dim3(kGridThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -946,6 +1366,42 @@ cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixe
   cfg.numAttrs = 1;
   return mixed ? cudaLaunchKernelEx(&cfg, resident_kernel<float>, a)
                : cudaLaunchKernelEx(&cfg, resident_kernel<double>, a);
+}
+
+namespace {
+cudaLaunchConfig_t cluster_config(int problems, int C, size_t smem, cudaLaunchAttribute *at) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(problems * C));
+  cfg.blockDim = dim3(kClusterThreads);
+  cfg.dynamicSmemBytes = smem;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+}  // namespace
+
+// Whether the device can hold a cluster of C blocks with smem bytes each.
+bool cluster_fits(int C, size_t smem, bool mixed, bool res, bool batch) {
+  cudaLaunchAttribute at[1];
+  cudaLaunchConfig_t cfg = cluster_config(1, C, smem, at);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, cluster_of(mixed, res, batch), &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return n > 0;
+}
+
+cudaError_t launch_cluster(const ResidentArgs &a, int problems, size_t smem, bool mixed, bool res,
+                           cudaStream_t s) {
+  cudaLaunchAttribute at[1];
+  cudaLaunchConfig_t cfg = cluster_config(problems, a.cluster, smem, at);
+  cfg.stream = s;
+  return cudaLaunchKernelEx(&cfg, cluster_of(mixed, res, a.inst != nullptr), a);
 }
 
 }  // namespace lpg

@@ -1,7 +1,9 @@
 """The resident kernel (autotune = 1, LPs that fit on the SMs) against the
-per-pass kernels (autotune = 0): the same lanes, chains and butterflies, so the
-iterates agree bit for bit; the check's sums are reduced in another order, so
-its gaps and residuals agree to rounding and the restart decisions are equal."""
+per-pass kernels (autotune = 0): the same lanes, chains and butterflies (and, in
+mixed precision, the same order of the radius that scales the next correction),
+so the iterates agree bit for bit; the check's other sums are reduced in another
+order, so its gaps and residuals agree to rounding and the restart decisions are
+equal."""
 import dataclasses
 
 import numpy as np
@@ -53,13 +55,8 @@ def test_same_iterates_as_the_per_pass_kernels(lpm, name, precision):
     s0, b, t0, i0 = run(lpm, data, 0, **opts)
     assert i1.graph_kernels == 1 and i0.graph_kernels > 48
     assert (s1, i1.iters, i1.restarts, i1.returned) == (s0, i0.iters, i0.restarts, i0.returned)
-    if precision == 0:  # the correction's data carry the check's rounding in mixed precision
-        for k in a:
-            np.testing.assert_array_equal(a[k], b[k], err_msg=k)
-    else:
-        for k in a:
-            np.testing.assert_allclose(a[k], b[k], rtol=0, err_msg=k,
-                                       atol=1e-6 * max(1.0, np.abs(b[k]).max(initial=0.0)))
+    for k in a:
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
     np.testing.assert_array_equal(t1[:, [0, 2]], t0[:, [0, 2]])
     if precision == 0:
         # a gap sums n + m positive terms in another order: n eps relative, and residuals
@@ -105,3 +102,56 @@ def test_converges_and_repeats(lpm):
     np.testing.assert_array_equal(outs[0][0], outs[1][0])
     np.testing.assert_array_equal(outs[0][1], outs[1][1])
     assert abs(np.dot(data.c, outs[0][0]) - data.obj_star) <= 1e-6 * (1 + abs(data.obj_star))
+
+
+def batch_run(lpm, probs, autotune, **opts):
+    with lpm.LPBatch(probs, autotune=autotune, eta=0.05, **opts) as g:
+        status = g.solve(1e-300)
+        return status, g.state(), g.info()[1]
+
+
+BATCHES = {  # clusters of 8, 2 and 1 blocks, matrix inside; streamed, several blocks per SM
+    "3_uneven": lambda: [lpgen.tiny_standard_form(1, m=31, n=33, per_col=3), lpgen.adversarial(7),
+                         lpgen.large_mixed(3, m=199, n=701)],
+    "70": lambda: [lpgen.tiny_standard_form(k, m=90 + k, n=200, per_col=4) for k in range(70)],
+    "160": lambda: [lpgen.adversarial(k, m=20 + k % 7, n=41) for k in range(160)],
+    "640": lambda: [lpgen.tiny_standard_form(k, m=60, n=121, per_col=4) for k in range(640)],
+}
+
+
+@pytest.mark.parametrize("name", list(BATCHES))
+@pytest.mark.parametrize("precision", [0, 1])
+def test_batch_same_iterates_as_the_per_pass_kernels(lpm, name, precision):
+    probs = BATCHES[name]()
+    opts = dict(check_every=16, max_iter=16 * 9, precision=precision)
+    s1, a, p1 = batch_run(lpm, probs, 1, **opts)
+    s0, b, p0 = batch_run(lpm, probs, 0, **opts)
+    assert s1 == s0
+    for k in a:
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    for u, v in zip(p1, p0):
+        for k in ("iters", "restarts", "checks", "status", "returned"):
+            assert u[k] == v[k], k
+        if precision == 0:
+            np.testing.assert_allclose(u["kkt_avg"], v["kkt_avg"], rtol=1e-9, atol=1e-11)
+            np.testing.assert_allclose(u["rho_stored"], v["rho_stored"], rtol=1e-9, atol=1e-11)
+
+
+def test_batch_check_periods_and_schemes(lpm):
+    """Problems due at different blocks, flexible and fixed restarts, and an
+    iteration limit that falls between two checks."""
+    probs = [lpgen.large_mixed(k, m=120 + 10 * k, n=400) for k in range(5)]
+    for scheme in ("FLEXIBLE", "FIXED", "NONE"):
+        got = []
+        for autotune in (1, 0):
+            with lpm.LPBatch(probs, autotune=autotune, eta=0.05, check_every=16, fixed_len=48,
+                             max_iter=16 * 11,
+                             restart_scheme=getattr(lpm, "LP_RESTART_" + scheme)) as g:
+                g.set_check_every([16, 32, 48, 64, 16])
+                g.solve(1e-300)
+                got.append((g.state(), g.info()[1]))
+        for k in got[0][0]:
+            np.testing.assert_array_equal(got[0][0][k], got[1][0][k], err_msg=f"{scheme} {k}")
+        for u, v in zip(got[0][1], got[1][1]):
+            for k in ("iters", "restarts", "checks", "status", "returned"):
+                assert u[k] == v[k], (scheme, k)
