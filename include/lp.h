@@ -101,9 +101,12 @@ typedef struct {
   int32_t single_lane_max; /* rows of at most this many elements get one lane each (64) */
   int32_t spmv_mode;      /* reserved, must be 0 */
   int32_t precision;      /* LP_PRECISION_FP64 (default) or LP_PRECISION_MIXED */
-  int32_t lane_auto;      /* > 0: per matrix, halve single_lane_max and lane_steps until the
-                             layout has at least lane_auto x (SM count) slices (warps), in FP64
-                             not below 8 elements per lane; 0: use the given lane policy as is (32) */
+  int32_t lane_auto;      /* > 0: per matrix, choose the lane policy from the given one: in mixed
+                             precision single_lane_max and lane_steps are halved until the layout
+                             has at least lane_auto x (SM count) slices (warps); in FP64 the
+                             halvings (not below 8) with the smallest modelled time of a pass are
+                             taken (FP64 issue against a lane's chain of gathers); 0: use the
+                             given lane policy as is (32) */
   int32_t autotune;       /* 1: at lp_create, choose how the iterations run: an LP that fits into
                              the SMs' shared memory (without split rows, check_every <= 1024) runs
                              K iterations and the check in one launch; for others every

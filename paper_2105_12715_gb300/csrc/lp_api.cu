@@ -364,13 +364,15 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
 }
 
 // Kernel-variant tuner (lp_options.autotune): on this problem, times every
-// unroll variant of the column pass, then of the row pass (three rounds, each
-// a warm-up and three timed launches per variant, CUDA events on the stream)
-// and keeps the fastest.  Every variant sums each row in the same order, so the choice
+// unroll variant of the column pass, then of the row pass (a warm-up and two
+// timed launches per variant, CUDA events on the stream, and a second round for
+// those within 5% of the fastest) and keeps the fastest.  Every variant sums each row in the same order, so the choice
 // changes speed, not results.  The launches advance the iterate: the caller
 // resets the state afterwards.
 lp_status tune_variants(lp_problem *h, cudaStream_t s) {
-  constexpr int kCands = 4, kRounds = 3, kReps = 3;
+  // (48 to 96 launches took 3.7 ms of a 20 ms lp_create at 100k x 500k)
+  constexpr int kCands = 4, kRounds = 2, kReps = 2;
+  constexpr float kOut = 1.05f;  // slower than this by more: not timed again
   const int cands[kCands] = {-2, -4, 2, 4};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   LP_CU(cudaEventCreate(&e0));
@@ -385,6 +387,7 @@ lp_status tune_variants(lp_problem *h, cudaStream_t s) {
     for (int round = 0; round < kRounds && st == LP_OK; ++round) {
       for (int i = 0; i < kCands; ++i) {
         const int ci = (i + round) % kCands;
+        if (best[ci] > kOut * *std::min_element(best, best + kCands) && round > 0) continue;
         u = cands[ci];
         for (int r = 0; r <= kReps; ++r) {
           if (r == 1) cudaEventRecord(e0, s);
@@ -487,8 +490,12 @@ lp_status host_layout(lp_problem *h, const int32_t *row_ptr, const int32_t *col_
   HostSell HA, HAT;
   const LanePolicy policy{opt.long_row_threshold, opt.lane_steps, opt.single_lane_max};
   const int64_t target = (int64_t)opt.lane_auto * h->nsm;
-  const LanePolicy pa = choose_policy(rp, perm_y, policy, target, policy_floor(h->mixed));
-  const LanePolicy pat = choose_policy(cp, perm_x, policy, target, policy_floor(h->mixed));
+  const LanePolicy pa = choose_lanes(policy, target, h->mixed, [&](const LanePolicy &p) {
+    return layout_work(rp, perm_y, p);
+  });
+  const LanePolicy pat = choose_lanes(policy, target, h->mixed, [&](const LanePolicy &p) {
+    return layout_work(cp, perm_x, p);
+  });
   const int32_t split_len = opt.split_row_len;
   build_sell(m, n, rp, hci, hv, perm_y, inv_x, pa, HA, {}, split_len);
   build_sell(n, m, cp, ri.data(), cv.data(), perm_x, inv_y, pat, HAT, {}, split_len);
@@ -702,7 +709,7 @@ lp_status device_layout(lp_problem *h, const int32_t *row_ptr, const int32_t *co
   LP_CU(cudaMemcpyAsync(hc.data(), hist_c, sizeof(int64_t) * hc.size(), cudaMemcpyDeviceToHost, s));
   LP_CU(cudaStreamSynchronize(s));
 
-  // lane policy (the host layout's choose_policy, from the length histogram)
+  // lane policy (choose_lanes, as for the host layout, from the length histogram)
   // and the runs of equal lane count in the sorted order
   // (the lane count is nondecreasing in the length, so each of the at most 6
   // lane counts forms one run; false if that ever failed)
@@ -733,15 +740,30 @@ lp_status device_layout(lp_problem *h, const int32_t *row_ptr, const int32_t *co
     if (warp_rows) *warp_rows = wr;
     return true;
   };
-  auto choose = [&](const std::vector<int64_t> &hist, LanePolicy p) {
-    const int64_t target = (int64_t)opt.lane_auto * nsm;
-    if (target <= 0) return p;
-    int64_t ns = 0;
-    for (;;) {
-      if (!runs_of(hist, p, nullptr, &ns, nullptr)) break;
-      if (ns >= target || !more_lanes(p, policy_floor(h->mixed))) break;
+  // the same work as layout_work's: of a run's rows, longest first, every
+  // (32 >> lg)-th opens a slice
+  auto hist_work = [](const std::vector<int64_t> &hist, const LanePolicy &p) {
+    LayoutWork w;
+    int run_lg = -1;
+    int64_t pos = 0;  // rows of the current run before this length
+    for (int64_t len = (int64_t)hist.size() - 1; len >= 0; --len) {
+      const int64_t rows = hist[(size_t)len];
+      if (rows == 0) continue;
+      const int lg = lanes_log2(len, p);
+      if (lg != run_lg) {
+        run_lg = lg;
+        pos = 0;
+      }
+      const int64_t cap = kWarp >> lg;
+      const int64_t opened = (pos + rows + cap - 1) / cap - (pos + cap - 1) / cap;
+      if (opened > 0) w.add(len, lg, p, opened);
+      pos += rows;
     }
-    return p;
+    return w;
+  };
+  auto choose = [&](const std::vector<int64_t> &hist, const LanePolicy &p) {
+    return choose_lanes(p, (int64_t)opt.lane_auto * nsm, h->mixed,
+                        [&](const LanePolicy &q) { return hist_work(hist, q); });
   };
   const LanePolicy policy{opt.long_row_threshold, opt.lane_steps, opt.single_lane_max};
   const int32_t split_len = opt.split_row_len;
@@ -1012,9 +1034,11 @@ lp_status lp_create(int32_t m, int32_t n, int64_t nnz, const int32_t *row_ptr,
     LP_CU(cudaGetLastError());
     if (opt.sigma_method == LP_SIGMA_LANCZOS) {
       // three rotating n-vectors: v_{k-1}, v_k and w (which becomes v_{k+1})
-      LanczosT T{nullptr, nullptr, std::min<int32_t>(opt.power_iters, kLanczosMax)};
+      LanczosT T{};
+      T.cap = std::min<int32_t>(opt.power_iters, kLanczosMax);
+      const int64_t parts = lanczos_parts(h->A, h->AT);
       double *coef = nullptr;
-      if (cudaMalloc(&coef, sizeof(double) * 2 * T.cap) != cudaSuccess) {
+      if (cudaMalloc(&coef, sizeof(double) * (3 * (int64_t)T.cap + parts + 1)) != cudaSuccess) {
         cudaGetLastError();
         return fail(LP_ERR_OOM, "cudaMalloc of the Lanczos coefficients failed");
       }
@@ -1023,18 +1047,36 @@ lp_status lp_create(int32_t m, int32_t n, int64_t nnz, const int32_t *row_ptr,
         ~Free() { cudaFree(p); }
       } free_coef{coef};
       T.alpha = coef;
-      T.beta = coef + T.cap;
+      T.beta = T.alpha + T.cap;
+      T.inv = T.beta + T.cap;
+      T.parts = T.inv + T.cap;
+      T.arrived = reinterpret_cast<unsigned int *>(T.parts + parts);
+      LP_CU(cudaMemsetAsync(T.arrived, 0, sizeof(unsigned int), s));
       double *P[3] = {pv, pw, h->v.xbar};
+      // The Ritz values are computed on the handle's own stream while the next
+      // steps run; the host enqueues one chunk of steps ahead of the flag it reads.
+      cudaStream_t side = h->cap_stream;
+      constexpr int kChunk = 2 * kLanczosEval;
+      int chunk = 0;
       for (int k = 0; k < T.cap; ++k) {
         launch_lanczos_step(h->A, h->AT, P[k % 3], pav, P[(k + 1) % 3], P[(k + 2) % 3], h->st, T,
-                            k, (k + 1) % 4 == 0, cs.partials, cs.pstride, rgrid, n, s);
-        if ((k + 1) % 16 != 0 && k + 1 != T.cap) continue;
+                            k, s);
+        if ((k + 1) % kLanczosEval != 0 && k + 1 != T.cap) continue;
+        LP_CU(cudaEventRecord(h->ev[0], s));
+        LP_CU(cudaStreamWaitEvent(side, h->ev[0], 0));
+        launch_lanczos_ritz(h->st, T, k, side);
         LP_CU(cudaGetLastError());
-        int32_t done = 0;
-        LP_CU(cudaMemcpyAsync(&done, &h->st->pw_done, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        LP_CU(cudaStreamSynchronize(s));
-        if (done) break;
+        if ((k + 1) % kChunk != 0) continue;
+        if (chunk > 0) {
+          LP_CU(cudaEventSynchronize(h->ev[1]));
+          if (h->h_status[0]) break;
+        }
+        LP_CU(cudaMemcpyAsync(&h->h_status[0], &h->st->pw_done, sizeof(int32_t),
+                              cudaMemcpyDeviceToHost, side));
+        LP_CU(cudaEventRecord(h->ev[1], side));
+        ++chunk;
       }
+      LP_CU(cudaStreamSynchronize(side));
       LP_CU(cudaStreamSynchronize(s));
     } else {
       const int chunk = 25;

@@ -1041,7 +1041,7 @@ __global__ void __launch_bounds__(kBlock) b_lanczos_kernel(BInst *I, BGlobal *G,
   __syncthreads();
   const bool last = (k + 1 >= cap) || !(bk > 0.0);
   if ((evaluate || last) && threadIdx.x < kWarp) {
-    const double theta = tridiag_top_eig(al, be, k + 1);
+    const double theta = tridiag_top_eig(al, be, k + 1, B.pw_iters > 0 ? B.pw_est : 0.0);
     if (threadIdx.x == 0) {
       const int conv = (B.pw_iters > 0 && fabs(theta - B.pw_est) <= G->pw_tol * theta);
       B.pw_est = theta;
@@ -1776,10 +1776,13 @@ lp_status lp_batch_create(int32_t count, const int32_t *host_row_start,
   HostSell HA, HAT;
   const LanePolicy policy{opt.long_row_threshold, opt.lane_steps, opt.single_lane_max};
   const int64_t target = (int64_t)opt.lane_auto * h->nsm;
-  const LanePolicy pa = choose_policy(rp, perm_y, policy, target,
-                                         policy_floor(opt.precision == LP_PRECISION_MIXED), brk_rows);
-  const LanePolicy pat = choose_policy(cp, perm_x, policy, target,
-                                          policy_floor(opt.precision == LP_PRECISION_MIXED), brk_cols);
+  const bool fp32 = opt.precision == LP_PRECISION_MIXED;
+  const LanePolicy pa = choose_lanes(policy, target, fp32, [&](const LanePolicy &p) {
+    return layout_work(rp, perm_y, p, brk_rows);
+  });
+  const LanePolicy pat = choose_lanes(policy, target, fp32, [&](const LanePolicy &p) {
+    return layout_work(cp, perm_x, p, brk_cols);
+  });
   build_sell(m, n, rp, hci, hv, perm_y, inv_x, pa, HA, brk_rows);
   build_sell(n, m, cp, ri.data(), cv.data(), perm_x, inv_y, pat, HAT, brk_cols);
 

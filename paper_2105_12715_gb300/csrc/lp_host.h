@@ -214,55 +214,83 @@ inline int32_t slice_limit(const std::vector<int32_t> &breaks, size_t *bi, int32
   return *bi < breaks.size() ? std::min(breaks[*bi], nrows) : nrows;
 }
 
-// Number of slices the layout of rows perm[0..) (longest first within each
-// segment between breaks) would have.
-inline int64_t count_slices(const std::vector<int64_t> &ptr, const std::vector<int32_t> &perm,
-                            const LanePolicy &p, const std::vector<int32_t> &breaks = {}) {
+// Work of a layout, from its slices: their number, the FP64 instructions that a
+// warp issues for them, and the longest chain of steps of a lane (a split row's
+// chunk takes at most lane_steps of the default policy).
+struct LayoutWork {
+  int64_t slices = 0, ops = 0, chain = 0;
+  void add(int64_t len, int lg, const LanePolicy &p, int64_t times) {
+    const int64_t steps = (len + (int64_t(1) << lg) - 1) >> lg;
+    slices += times;
+    ops += times * (steps + lg + 4);  // products, butterfly, epilogue
+    chain = std::max(chain, len >= p.warp_threshold ? std::min<int64_t>(steps, 16) : steps);
+  }
+  // FP64 pass in us (GB300; 14 LPs of 40k to 200k rows, rows of 12 and of 50
+  // elements, lengths 2 to 200: within 20%): issue of the FP64 instructions, or one
+  // lane's chain of gathers when too few warps hide it.
+  double fp64_us() const {
+    return std::max(3.0 + 0.113e-3 * (double)ops, 2.0 + 0.35 * (double)chain);
+  }
+};
+
+// The layout's work for rows perm[0..) (longest first within each segment
+// between breaks).
+inline LayoutWork layout_work(const std::vector<int64_t> &ptr, const std::vector<int32_t> &perm,
+                              const LanePolicy &p, const std::vector<int32_t> &breaks = {}) {
   const int32_t nrows = (int32_t)perm.size();
-  int64_t ns = 0;
+  LayoutWork w;
   int32_t r = 0;
   size_t bi = 0;
   while (r < nrows) {
     const int32_t lim = slice_limit(breaks, &bi, r, nrows);
-    const int lg = lanes_log2(ptr[perm[r] + 1] - ptr[perm[r]], p);
+    const int64_t len = ptr[perm[r] + 1] - ptr[perm[r]];
+    const int lg = lanes_log2(len, p);
     const int cap = kWarp >> lg;
     int32_t q = r;
     while (q < lim && q - r < cap && lanes_log2(ptr[perm[q] + 1] - ptr[perm[q]], p) == lg) ++q;
-    ++ns;
+    w.add(len, lg, p, 1);
     r = q;
   }
-  return ns;
+  return w;
 }
 
-// Gives rows more lanes: halves single_max and lane_steps, each down to
-// floor_steps; false once neither can shrink.
-inline bool more_lanes(LanePolicy &p, int32_t floor_steps) {
-  const int32_t sm = p.single_max > floor_steps ? std::max(floor_steps, p.single_max / 2) : p.single_max;
-  const int32_t ls = p.lane_steps > floor_steps ? std::max(floor_steps, p.lane_steps / 2) : p.lane_steps;
-  if (sm == p.single_max && ls == p.lane_steps) return false;
-  p.single_max = sm;
-  p.lane_steps = ls;
-  return true;
-}
-// Fewest elements per lane that more_lanes goes down to.  FP64: 8.  Every extra
-// factor of two in lanes costs each row a butterfly step, an FP64 addition of
-// the whole warp, and GB300's FP64 pipe (2 per cycle per SM) is what a small LP
-// runs out of first (5k x 25k, resident kernel, 64 iterations and a check: 0.52 ms
-// with 8, 0.73 with 4, 0.53 with 16).  FP32 additions cost a 32nd of that: down to 1.
-inline int32_t policy_floor(bool mixed) { return mixed ? 1 : 8; }
-
-// Launch-shape tuning by a model: a pass runs one warp per slice, and
-// fewer slices than `target` warps leave SMs idle while each warp walks a
-// long chain of dependent gathers.  Starting from the given policy, give
-// rows more lanes (halving single_max and lane_steps) until the layout
-// has at least `target` slices or rows get floor_steps elements per lane.
-inline LanePolicy choose_policy(const std::vector<int64_t> &ptr, const std::vector<int32_t> &perm,
-                                LanePolicy p, int64_t target, int32_t floor_steps,
-                                const std::vector<int32_t> &breaks = {}) {
+// Launch-shape tuning by a model, starting from the given policy (target > 0).
+//   FP32: a pass runs one warp per slice, and fewer slices than `target` warps
+// leave SMs idle while each warp walks a long chain of dependent gathers: rows
+// get more lanes (single_max and lane_steps halved) until the layout has
+// `target` slices or rows get one element per lane.
+//   FP64: every factor of two in lanes costs each row a butterfly step, an FP64
+// addition of the whole warp, and GB300's FP64 pipe (2 per cycle per SM) is what
+// a pass runs out of first, so the policy with the smallest LayoutWork::fp64_us()
+// among single_max halved up to three times and lane_steps halved up to once, not
+// below 8, is taken (100k x 500k, rows of 50: 23.5 us per row pass with one lane
+// per row, 38.2 with the 8 lanes that `target` asks for; 40k rows: 13.8 with 4
+// lanes, 16.5 with 8, 17.3 with 1).  work(p) gives the layout's work under p.
+template <class F>
+inline LanePolicy choose_lanes(LanePolicy p, int64_t target, bool mixed, F work) {
   if (target <= 0) return p;
-  while (count_slices(ptr, perm, p, breaks) < target && more_lanes(p, floor_steps)) {
+  if (mixed) {
+    while (work(p).slices < target && (p.single_max > 1 || p.lane_steps > 1)) {
+      p.single_max = p.single_max / 2;
+      p.lane_steps = std::max(1, p.lane_steps / 2);
+    }
+    return p;
   }
-  return p;
+  constexpr int32_t kFloor = 8;
+  LanePolicy best = p;
+  double cost = work(p).fp64_us();
+  for (int ls = 0; ls < 2; ++ls)
+    for (int sm = 0; sm < 4; ++sm) {
+      LanePolicy q = p;
+      q.lane_steps = std::max(std::min(p.lane_steps, kFloor), p.lane_steps >> ls);
+      q.single_max = std::max(std::min(p.single_max, kFloor), p.single_max >> sm);
+      const double c = work(q).fp64_us();
+      if (c < cost) {
+        cost = c;
+        best = q;
+      }
+    }
+  return best;
 }
 
 // Sliced layout (see SellMat) of the operator whose row r (permuted order)

@@ -113,7 +113,7 @@ struct DevState {
   int32_t pw_done;
   int32_t pw_iters;
   int32_t pw_max;
-  int32_t pad2;
+  int32_t pw_stop;  // Lanczos: pw_done as the last step saw it
   double pw_tol;
   // cross-block reductions (last-block pattern; counters return to 0)
   double tot[NQ];
@@ -156,12 +156,15 @@ struct AdjVecs {
 };
 
 // Coefficients of the Lanczos tridiagonal matrix (sigma_max estimate):
-// alpha[0..cap-1] on the diagonal, beta[0..cap-1] below it.
+// alpha[0..cap-1] on the diagonal, beta[0..cap-1] below it, inv = 1 / beta; block
+// partials of a step's reduction and their arrival counter (zero between steps).
 struct LanczosT {
-  double *alpha, *beta;
+  double *alpha, *beta, *inv, *parts;
+  unsigned int *arrived;
   int32_t cap;
 };
 constexpr int kLanczosMax = 1024;  // longest Lanczos run (steps)
+constexpr int kLanczosEval = 4;    // steps between evaluations of the Ritz value
 
 // Scratch of the check and of the multiplier search.
 struct CheckScratch {
@@ -328,8 +331,9 @@ void launch_power_iteration_step(const SellMat &A, const SellMat &AT,
                                  int grid, int n, int m, cudaStream_t s);
 void launch_lanczos_step(const SellMat &A, const SellMat &AT, const double *v, double *av,
                          double *w, const double *vprev, DevState *st, const LanczosT &T, int k,
-                         bool evaluate, double *partials, int pstride, int grid, int n,
                          cudaStream_t s);
+int64_t lanczos_parts(const SellMat &A, const SellMat &AT);
+void launch_lanczos_ritz(DevState *st, const LanczosT &T, int k, cudaStream_t s);
 void launch_start_vector(const int32_t *perm, double *v, int n, double *partials, int pstride,
                          int grid, cudaStream_t s);
 void launch_gather(double *out, const double *in, const int32_t *perm, int64_t n,

@@ -57,7 +57,7 @@ template <bool SPLIT = false>
 __global__ void __launch_bounds__(kBlock) spmv_kernel(SellMat A, const double *__restrict__ v,
                                                       StoreEpi epi, const DevState *st) {
   if (st && (st->status != kRunning || st->pw_done)) return;
-  process_all<1, kUnroll, false, false, SPLIT>(A, v, (const double *)nullptr, epi);
+  process_all<1, 2, true, false, SPLIT>(A, v, (const double *)nullptr, epi);
 }
 
 template <int U, bool PIPE, bool SPLIT = false>
@@ -800,70 +800,120 @@ __global__ void power_scale_kernel(double *v, const double *w, int64_t n, const 
 // sigma_max(A)^2 is the largest eigenvalue of A^T A; the Lanczos process on
 // A^T A estimates it by the largest eigenvalue (Ritz value) of the
 // tridiagonal matrix it builds, in far fewer products than the power
-// iteration.  Step k, with w = A^T A v_k from two SpMVs:
-//   alpha_k = v_k . w,  w <- w - alpha_k v_k - beta_{k-1} v_{k-1},
-//   beta_k = ||w||,     v_{k+1} = w / beta_k.
-// The Ritz value is evaluated every few steps; the run stops when it changes
-// by at most pw_tol relative to the previous evaluation, at beta_k = 0 (an
-// invariant subspace: the Ritz value is exact) or at the step cap.  Every
-// block re-sums the block partials of a reduction in the same fixed order,
-// so all blocks see the same alpha_k and beta_k.
-__global__ void __launch_bounds__(kBlock) lz_dot_kernel(const double *__restrict__ v,
-                                                        const double *__restrict__ w, int64_t n,
-                                                        double *partials, int pstride,
-                                                        const DevState *st) {
-  if (st->pw_done) return;
-  double q[1] = {0.0};
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    q[0] += v[i] * w[i];
-  block_reduce_store<1>(q, partials, pstride, (int)blockIdx.x);
-}
-
-__global__ void __launch_bounds__(kBlock) lz_update_kernel(double *w, const double *v,
-                                                           const double *vprev, int64_t n,
-                                                           double *partials, int pstride,
-                                                           int nparts, const DevState *st,
-                                                           LanczosT T, int k) {
-  if (st->pw_done) return;
-  __shared__ double red[kBlock];
-  const double alpha = sum_fixed(partials, nparts, red);
-  if (blockIdx.x == 0 && threadIdx.x == 0) T.alpha[k] = alpha;
-  const double bprev = k > 0 ? T.beta[k - 1] : 0.0;
-  double q[1] = {0.0};
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    double r = w[i] - alpha * v[i];
-    if (k > 0) r -= bprev * vprev[i];
-    w[i] = r;
-    q[0] += r * r;
+// iteration.  Step k, with the unnormalized residuals w_k (v_k = w_{k-1} / beta_{k-1},
+// v_0 the start vector), in two launches:
+//   rows:  z = A v_k,  alpha_k = ||z||^2  (= v_k . A^T A v_k),
+//   cols:  w_k = A^T z - alpha_k v_k - beta_{k-1} v_{k-1},  beta_k = ||w_k||.
+// The reductions ride in the products' epilogues (one block partial each, in a
+// fixed order, summed by the last block to finish), and the normalizations in
+// the scalars: separate dot, update and scale kernels cost another 45 us per
+// step beside two products of 32 us at 100k x 500k, most of it FP64 divisions
+// and every block summing all partials again.
+// The Ritz value is evaluated every kLanczosEval steps; the run stops when it
+// changes by at most pw_tol relative to the previous evaluation, at beta_k = 0 (an
+// invariant subspace: the Ritz value is exact) or at the step cap.
+struct LzEpi {
+  double *out;
+  const double *v = nullptr, *vprev = nullptr;  // cols: w_{k-1}, w_{k-2}
+  double sv = 0.0, sp = 0.0;  // rows: sv scales the sum; cols: multiples subtracted
+  double q = 0.0;
+  // split rows: see process_split_item
+  static constexpr bool kSplitSlots = true;
+  double *split_slots = nullptr;
+  __device__ __forceinline__ void zero_split_slot(int item) const { split_slots[item] = 0.0; }
+  __device__ __forceinline__ void flush_split_slot(int first) {
+    split_slots[first] = q;
+    q = 0.0;
   }
-  block_reduce_store<1>(q, partials + pstride, pstride, (int)blockIdx.x);
-}
+  struct Pre { double v, p; };
+  __device__ __forceinline__ Pre load(int r) const {
+    return {v ? v[r] : 0.0, vprev ? vprev[r] : 0.0};
+  }
+  __device__ __forceinline__ double init(const Pre &) const { return 0.0; }
+  __device__ __forceinline__ void store(int r, double a, double, const Pre &p) {
+    const double t = v ? fma(-sp, p.p, fma(-sv, p.v, a)) : a * sv;
+    out[r] = t;
+    q = fma(t, t, q);
+  }
+};
 
-__global__ void __launch_bounds__(kBlock) lz_scale_kernel(double *w, int64_t n,
-                                                          const double *partials, int pstride,
-                                                          int nparts, const DevState *st,
-                                                          LanczosT T, int k) {
-  if (st->pw_done) return;
+template <bool COLS, bool SPLIT>
+__global__ void __launch_bounds__(kBlock) lz_step_kernel(SellMat A, const double *__restrict__ x,
+                                                         LzEpi epi, DevState *st, LanczosT T,
+                                                         int k) {
+  pdl_enter();
+  if (st->pw_stop) return;
+  const double i1 = k > 0 ? T.inv[k - 1] : 1.0;  // v_k = w_{k-1} i1
+  if (COLS) {
+    epi.sv = T.alpha[k] * i1;
+    epi.sp = k > 0 ? T.beta[k - 1] * (k > 1 ? T.inv[k - 2] : 1.0) : 0.0;
+  } else {
+    epi.sv = i1;
+  }
+  process_all<1, 2, true, false, SPLIT>(A, x, (const double *)nullptr, epi);
+  __shared__ bool last;
   __shared__ double red[kBlock];
-  const double beta = sqrt(sum_fixed(partials + pstride, nparts, red));
-  if (blockIdx.x == 0 && threadIdx.x == 0) T.beta[k] = beta;
-  if (!(beta > 0.0)) return;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    w[i] = w[i] / beta;
+  // only the rows' first lanes hold terms: butterfly steps that would add zeros
+  // everywhere are left out (with 8 lanes per row 3 of 5)
+  double q = epi.q;
+  const unsigned terms = __ballot_sync(kFull, nonzero_d(q));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    constexpr unsigned kBit[5] = {0xaaaaaaaau, 0xccccccccu, 0xf0f0f0f0u, 0xff00ff00u, 0xffff0000u};
+    const int b = o == 16 ? 4 : o == 8 ? 3 : o == 4 ? 2 : o == 2 ? 1 : 0;
+    if (terms & kBit[b]) q += __shfl_down_sync(kFull, q, o);
+  }
+  if ((threadIdx.x & (kWarp - 1)) == 0) red[threadIdx.x >> 5] = q;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int i = 0; i < kWarpsPerBlock; ++i) t += red[i];
+    __stcg(T.parts + blockIdx.x, t);
+    __threadfence();
+    last = atomicAdd(T.arrived, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double s = 0.0;  // the blocks, then (SPLIT) the chunk slices' slots
+  const int parts = (int)gridDim.x + A.nsplit;
+  for (int i = threadIdx.x; i < parts; i += kBlock) s += __ldcg(T.parts + i);
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = kBlock / 2; o > 0; o >>= 1) {
+    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x != 0) return;
+  *T.arrived = 0u;
+  if (COLS) {
+    const double beta = sqrt(red[0]);
+    T.beta[k] = beta;
+    T.inv[k] = beta > 0.0 ? 1.0 / beta : 0.0;
+    // the next steps' blocks all see the same flag
+    st->pw_stop = *(volatile int32_t *)&st->pw_done;
+  } else {
+    T.alpha[k] = red[0];
+  }
 }
 
-// One warp.  After step k: the Ritz value of the (k+1) x (k+1) matrix.
-__global__ void lz_ritz_kernel(DevState *st, LanczosT T, int k, int evaluate) {
+// One warp.  After step k (of every kLanczosEval-th): the Ritz value of the
+// (k+1) x (k+1) matrix, or of the smaller one that ends at the first beta = 0
+// since the last evaluation.  It runs on a stream of its own beside the next
+// steps (a chain of FP64 divisions, 50 to 200 us), which it stops through
+// pw_done; they change nothing it reads.
+__global__ void lz_ritz_kernel(DevState *st, LanczosT T, int k) {
   if (st->pw_done) return;
-  const double beta = T.beta[k];
-  const bool last = (k + 1 >= T.cap) || !(beta > 0.0);
-  if (!evaluate && !last) return;
-  const double theta = tridiag_top_eig(T.alpha, T.beta, k + 1);
+  bool last = k + 1 >= T.cap;
+  for (int j = max(0, k + 1 - kLanczosEval); j <= k; ++j)
+    if (!(T.beta[j] > 0.0)) {
+      k = j;
+      last = true;
+    }
+  const bool first = st->pw_iters == 0;
+  const double theta = tridiag_top_eig(T.alpha, T.beta, k + 1, first ? 0.0 : st->pw_est);
   if (threadIdx.x == 0) {
-    const int conv = (st->pw_iters > 0 && fabs(theta - st->pw_est) <= st->pw_tol * theta);
+    const int conv = (!first && fabs(theta - st->pw_est) <= st->pw_tol * theta);
     st->pw_est = theta;
     st->pw_iters = k + 1;
     if (conv || last) st->pw_done = 1;
@@ -1268,16 +1318,37 @@ void launch_power_iteration_step(const SellMat &A, const SellMat &AT, double *v,
   power_scale_kernel<<<grid_for(n, num_sms()), kBlock, 0, s>>>(v, w, n, st);
 }
 
+namespace {
+template <bool COLS>
+void lz_launch(const SellMat &A, const double *x, LzEpi epi, DevState *st, const LanczosT &T, int k,
+               cudaStream_t s) {
+  const int g = split_grid(A) + item_grid(A);
+  epi.split_slots = T.parts + g;
+  if (A.nsplit > 0) launch_pdl(lz_step_kernel<COLS, true>, g, kBlock, s, A, x, epi, st, T, k);
+  else launch_pdl(lz_step_kernel<COLS, false>, g, kBlock, s, A, x, epi, st, T, k);
+}
+}  // namespace
+
+// Entries of LanczosT::parts that the steps on A and A^T need.
+int64_t lanczos_parts(const SellMat &A, const SellMat &AT) {
+  return std::max((int64_t)split_grid(A) + item_grid(A) + A.nsplit,
+                  (int64_t)split_grid(AT) + item_grid(AT) + AT.nsplit);
+}
+
 void launch_lanczos_step(const SellMat &A, const SellMat &AT, const double *v, double *av,
                          double *w, const double *vprev, DevState *st, const LanczosT &T, int k,
-                         bool evaluate, double *partials, int pstride, int grid, int n,
                          cudaStream_t s) {
-  launch_spmv(A, v, av, s, st);
-  launch_spmv(AT, av, w, s, st);
-  lz_dot_kernel<<<grid, kBlock, 0, s>>>(v, w, n, partials, pstride, st);
-  lz_update_kernel<<<grid, kBlock, 0, s>>>(w, v, vprev, n, partials, pstride, grid, st, T, k);
-  lz_scale_kernel<<<grid, kBlock, 0, s>>>(w, n, partials, pstride, grid, st, T, k);
-  lz_ritz_kernel<<<1, kWarp, 0, s>>>(st, T, k, evaluate ? 1 : 0);
+  LzEpi rows{}, cols{};
+  rows.out = av;
+  cols.out = w;
+  cols.v = v;
+  cols.vprev = k > 0 ? vprev : nullptr;
+  lz_launch<false>(A, v, rows, st, T, k, s);
+  lz_launch<true>(AT, av, cols, st, T, k, s);
+}
+
+void launch_lanczos_ritz(DevState *st, const LanczosT &T, int k, cudaStream_t s) {
+  lz_ritz_kernel<<<1, kWarp, 0, s>>>(st, T, k);
 }
 
 void launch_start_vector(const int32_t *perm, double *v, int n, double *partials, int pstride,

@@ -1,7 +1,7 @@
 // Device-side construction of the library's layout (setup step of Section 7's
 // method: the CSC copy of A, the length-sorted row and column orders and the
 // two lane-grouped slice layouts), the same arrays, bit for bit, as the host
-// construction in lp_host.h (build_csc, sort_by_length_desc, choose_policy,
+// construction in lp_host.h (build_csc, sort_by_length_desc, choose_lanes,
 // build_sell), so that both give identical iterates.  Every step is
 // deterministic: integer histograms and scans, and stable sorts.
 //
@@ -260,24 +260,43 @@ __global__ void __launch_bounds__(kLayBlock) lay_dup_kernel(const uint32_t *__re
 // ------------------------------------------------------------ orders
 
 // len[i] = ptr[i + 1] - ptr[i]; key[i] = mx - len[i] once mx is known (second call).
+// Lengths below kLenBins are counted in shared memory first, and the maximum is
+// taken per warp: most rows share a few lengths, and 500,000 columns updating
+// the same global counters one by one took 500 us.
+constexpr int kLenBins = 1024;
 template <class P>
 __global__ void __launch_bounds__(kLayBlock) lay_len_kernel(const P *__restrict__ ptr,
                                                             int32_t count, int64_t *mx,
                                                             uint32_t *key, int64_t mxv,
                                                             int64_t *hist) {
+  __shared__ unsigned bins[kLenBins];
+  if (key) {
+    for (int b = threadIdx.x; b < kLenBins; b += blockDim.x) bins[b] = 0u;
+    __syncthreads();
+  }
   int64_t local = 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t len = (int64_t)ptr[i + 1] - (int64_t)ptr[i];
     if (key) {
       key[i] = (uint32_t)(mxv - len);
-      atomicAdd(reinterpret_cast<unsigned long long *>(&hist[len]), 1ull);
+      if (len < kLenBins) atomicAdd(&bins[len], 1u);
+      else atomicAdd(reinterpret_cast<unsigned long long *>(&hist[len]), 1ull);
     } else {
       local = len > local ? len : local;
     }
   }
-  if (!key && local > 0) atomicMax(reinterpret_cast<unsigned long long *>(mx),
-                                   (unsigned long long)local);
+  if (key) {
+    __syncthreads();
+    for (int b = threadIdx.x; b < kLenBins; b += blockDim.x)
+      if (bins[b] > 0u)
+        atomicAdd(reinterpret_cast<unsigned long long *>(&hist[b]), (unsigned long long)bins[b]);
+  }
+  if (!key) {  // lengths are below 2^31: one global maximum per warp
+    const unsigned most = __reduce_max_sync(0xffffffffu, (unsigned)local);
+    if ((threadIdx.x & 31) == 0 && most > 0u)
+      atomicMax(reinterpret_cast<unsigned long long *>(mx), (unsigned long long)most);
+  }
 }
 
 __global__ void __launch_bounds__(kLayBlock) lay_inverse_kernel(const int32_t *__restrict__ perm,

@@ -719,9 +719,13 @@ __device__ __forceinline__ double scan256(double v, double *warp_tot) {
 // warp: each round, lane l counts the eigenvalues below the l-th of 32
 // interior points of the bracket [lo, hi] and the bracket shrinks to the
 // interval where the count first reaches k.  lo starts at the largest
-// diagonal entry (a lower bound on the largest eigenvalue), hi at the
-// largest Gershgorin row bound (an upper bound).  Returns the bracket's
-// midpoint (exactly lo when lo = hi, e.g. a 1 x 1 or zero matrix).
+// diagonal entry (a lower bound on the largest eigenvalue) or at `below`, the
+// estimate of a smaller T_j (another one, by interlacing), hi at the largest
+// Gershgorin row bound (an upper bound).  The points of the first round lie
+// at lo + (hi - lo) / 2^32 .. 2^1: once the process converges the eigenvalue
+// is that close to `below`, and 5 rounds do instead of 11 (a round is a chain
+// of k FP64 divisions, 1,000 cycles each).  Returns the bracket's midpoint
+// (exactly lo when lo = hi, e.g. a 1 x 1 or zero matrix).
 __device__ __forceinline__ int sturm_count_below(const double *a, const double *b, int k,
                                                  double x, double pivmin) {
   int c = 0;
@@ -734,7 +738,7 @@ __device__ __forceinline__ int sturm_count_below(const double *a, const double *
   return c;
 }
 
-__device__ double tridiag_top_eig(const double *a, const double *b, int k) {
+__device__ double tridiag_top_eig(const double *a, const double *b, int k, double below) {
   const int lane = threadIdx.x & (kWarp - 1);
   double lo = -INFINITY, hi = -INFINITY, bmax2 = 0.0;
   for (int i = lane; i < k; i += kWarp) {
@@ -748,22 +752,23 @@ __device__ double tridiag_top_eig(const double *a, const double *b, int k) {
     hi = fmax(hi, __shfl_xor_sync(kFull, hi, o));
     bmax2 = fmax(bmax2, __shfl_xor_sync(kFull, bmax2, o));
   }
+  lo = fmax(lo, below);
+  hi = fmax(hi, lo);
   // the largest eigenvalue lies in [lo, hi]; when no point of a round has all
   // k eigenvalues below it, it lies above the last point
   const double pivmin = 2.2250738585072014e-308 * fmax(1.0, bmax2);
   for (int round = 0; round < 24 && hi - lo > 2.0 * 2.220446049250313e-16 * fmax(fabs(lo), fabs(hi));
        ++round) {
-    const double w = (hi - lo) / 33.0;
-    const double x = lo + w * (double)(lane + 1);
+    // 2^(lane - 32) of the bracket, then the 32 points of an even division
+    const double x = round == 0
+                         ? fma(hi - lo, __longlong_as_double((long long)(1023 - 32 + lane) << 52), lo)
+                         : fma((hi - lo) / 33.0, (double)(lane + 1), lo);
     const unsigned all = __ballot_sync(kFull, sturm_count_below(a, b, k, x, pivmin) >= k);
-    if (all == 0u) {
-      lo = lo + w * 32.0;
-    } else {
-      const int f = __ffs(all) - 1;
-      const double nlo = lo + w * (double)f, nhi = lo + w * (double)(f + 1);
-      lo = nlo;
-      hi = nhi;
-    }
+    const int f = all ? __ffs(all) - 1 : kWarp;  // first point with all k eigenvalues below it
+    const double under = __shfl_sync(kFull, x, f > 0 ? f - 1 : 0);
+    const double over = __shfl_sync(kFull, x, f & (kWarp - 1));
+    if (f > 0) lo = under;
+    if (f < kWarp) hi = over;
   }
   return 0.5 * (lo + hi);
 }
