@@ -57,6 +57,9 @@ struct lp_problem {
   std::vector<int64_t> ckpt_t0;        // inner iteration count at each block start
   std::vector<int8_t> ckpt_restart;    // restart decision of each block's check
   int64_t rec_blocks = 0;
+  int64_t *rec_t0 = nullptr;           // device copies of the two, and [blocks] outer counts
+  int8_t *rec_rs = nullptr;
+  int32_t *rec_flag = nullptr;         // a recorded solve stopped / an adjoint's wait ran out
   AdjVecs adj{};
   uint8_t *mask_x = nullptr, *mask_y = nullptr;  // [K][n], [K][m]
   DevState *st = nullptr;
@@ -87,9 +90,12 @@ struct lp_problem {
   ResidentArgs res{};                 // resident kernel (lp_resident.cu), when res_blocks > 0
   int res_blocks = 0;
   size_t res_smem = 0;
+  size_t adj_smem = 0;                // adjoint kernel on the same blocks (0: the per-pass kernels)
 
   ~lp_problem() {
     if (ckpt) cudaFree(ckpt);
+    if (rec_t0) cudaFree(rec_t0);
+    if (rec_rs) cudaFree(rec_rs);
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
     for (auto &e : ev)
@@ -305,7 +311,7 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
   LP_CU(cudaStreamSynchronize(s));
   const int most = std::max(h->AT.nslices, h->A.nslices);
   // shared memory of the largest of P blocks; block b owns the slices b, b + P, ...
-  auto block_bytes = [&](int P, bool cluster) {
+  auto block_bytes = [&](int P, bool cluster, bool adjoint) {
     size_t smem = 0;
     for (int b = 0; b < P; ++b) {
       int cols = 0, rows = 0;
@@ -319,9 +325,10 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
         elems += (ir[i].len_g >> 3) * kWarp;
       }
       const int nc = (h->AT.nslices - b + P - 1) / P, nr = (h->A.nslices - b + P - 1) / P;
-      smem = std::max(smem, resident_fixed_bytes(nc, nr, cols, rows, opt.check_every, h->mixed,
-                                                 cluster ? h->n : 0, cluster ? h->m : 0) +
-                                (size_t)(elems * elem));
+      const int cx = cluster ? h->n : 0, cy = cluster ? h->m : 0, K = opt.check_every;
+      const size_t fixed = adjoint ? adjoint_fixed_bytes(nc, nr, cols, rows, K, cx, cy)
+                                   : resident_fixed_bytes(nc, nr, cols, rows, K, h->mixed, cx, cy);
+      smem = std::max(smem, fixed + (size_t)(elems * elem));
     }
     return smem;
   };
@@ -330,14 +337,14 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
   if ((int64_t)h->n + h->m <= kClusterElems) {
     for (int C = kClusterBlocks; C >= 1 && !cluster; C /= 2) {
       if (C > 1 && C > most) continue;
-      smem = block_bytes(C, true);
+      smem = block_bytes(C, true, false);
       if (smem <= limit && cluster_fits(C, smem, h->mixed, true, false)) cluster = C;
     }
     P = cluster;
   }
   if (!cluster) {
     P = std::max(1, std::min(h->nsm, (most + kSlicesPerBlock - 1) / kSlicesPerBlock));
-    smem = block_bytes(P, false);
+    smem = block_bytes(P, false, false);
     if (smem > limit || !resident_fits(P, h->nsm, smem, h->mixed)) return LP_OK;
   }
   lp_status e;
@@ -348,6 +355,10 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
       (e = h->alloc(&h->res.rpart, (int64_t)2 * (h->cs.cols_grid + h->cs.rows_grid))) != LP_OK)
     return e;
   h->res.cluster = cluster;
+  if (!h->mixed) {
+    const size_t bytes = block_bytes(P, cluster > 0, true);
+    if (bytes <= limit && adjoint_fits(P, h->nsm, cluster, bytes)) h->adj_smem = bytes;
+  }
   h->res.A = h->A;
   h->res.AT = h->AT;
   h->res.v = h->v;
@@ -852,6 +863,55 @@ lp_status device_layout(lp_problem *h, const int32_t *row_ptr, const int32_t *co
   h->perm_x = perm_x;
   h->perm_y = perm_y;
   LP_CU(cudaStreamSynchronize(s));  // scratch is freed on return
+  return LP_OK;
+}
+
+// lp_backward's recurrence, launched pass by pass.
+lp_status backward_by_passes(lp_problem *h, cudaStream_t s) {
+  const int n = h->n, m = h->m, K = h->opt.check_every;
+  const int64_t slot = 2 * (int64_t)n + 2 * (int64_t)m;
+  DevState hs{};
+  LP_CU(cudaMemcpyAsync(&hs, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+  LP_CU(cudaStreamSynchronize(s));
+  const double tau = hs.tau, sigma = hs.sigma;
+  for (int64_t b = h->rec_blocks - 1; b >= 0; --b) {
+    // recompute the block's forward steps with their masks
+    const double *c = h->ckpt + b * slot;
+    LP_CU(cudaMemcpyAsync(h->v.x, c, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+    LP_CU(cudaMemcpyAsync(h->v.y, c + n, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+    LP_CU(cudaMemcpyAsync(h->v.xbar, c + n + m, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+    LP_CU(cudaMemcpyAsync(h->v.ybar, c + 2 * n + m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+    const int64_t t0 = h->ckpt_t0[b];
+    auto wk = [&](int k) { return 1.0 / (double)(t0 + k + 1); };
+    for (int k = 0; k < K; ++k)
+      launch_forward_masked(h->A, h->AT, h->v, tau, sigma, wk(k), h->mask_x + (int64_t)k * n,
+                            h->mask_y + (int64_t)k * m, s);
+    // reverse through the block
+    launch_adjoint_block_start(h->adj, h->mask_y + (int64_t)(K - 1) * m, h->ckpt_restart[b],
+                               sigma, wk(K - 1), n, m, s);
+    for (int k = K - 1; k >= 0; --k)
+      launch_adjoint_step(h->A, h->AT, h->adj, h->mask_x + (int64_t)k * n,
+                          k > 0 ? h->mask_y + (int64_t)(k - 1) * m : nullptr, tau, sigma, wk(k),
+                          k > 0 ? wk(k - 1) : 0.0, k > 0 ? 1 : 0, s);
+    LP_CU(cudaGetLastError());
+  }
+  // restore the final state of the recorded solve: replay the last block
+  {
+    const int64_t b = h->rec_blocks - 1;
+    const double *c = h->ckpt + b * slot;
+    LP_CU(cudaMemcpyAsync(h->v.x, c, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+    LP_CU(cudaMemcpyAsync(h->v.y, c + n, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+    LP_CU(cudaMemcpyAsync(h->v.xbar, c + n + m, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+    LP_CU(cudaMemcpyAsync(h->v.ybar, c + 2 * n + m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+    const int64_t t0 = h->ckpt_t0[b];
+    for (int k = 0; k < K; ++k)
+      launch_forward_masked(h->A, h->AT, h->v, tau, sigma, 1.0 / (double)(t0 + k + 1),
+                            h->mask_x + (int64_t)k * n, h->mask_y + (int64_t)k * m, s);
+    if (h->ckpt_restart[b]) {  // the recorded check restarted: z <- zbar
+      LP_CU(cudaMemcpyAsync(h->v.x, h->v.xbar, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+      LP_CU(cudaMemcpyAsync(h->v.y, h->v.ybar, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+    }
+  }
   return LP_OK;
 }
 }  // namespace
@@ -1465,9 +1525,15 @@ lp_status lp_solve_recorded(lp_handle h, int64_t iters, void *cuda_stream) {
     for (double **p : ys)
       if ((e = h->alloc(p, m)) != LP_OK) return e;
   }
-  h->ckpt_t0.assign(blocks, 0);
-  h->ckpt_restart.assign(blocks, 0);
+  if (h->rec_t0) cudaFree(h->rec_t0);
+  if (h->rec_rs) cudaFree(h->rec_rs);
+  h->rec_t0 = nullptr;
+  h->rec_rs = nullptr;
   h->rec_blocks = 0;
+  LP_CU(cudaMalloc(&h->rec_t0, sizeof(int64_t) * (blocks + 1)));
+  LP_CU(cudaMalloc(&h->rec_rs, sizeof(int8_t) * blocks));
+  if (!h->rec_flag && (e = h->alloc(&h->rec_flag, 2)) != LP_OK) return e;
+  LP_CU(cudaMemsetAsync(h->rec_flag, 0, sizeof(int32_t), s));
   if ((e = set_run_params(h, 1e-300, s)) != LP_OK) return e;
   for (int64_t b = 0; b < blocks; ++b) {
     double *c = h->ckpt + b * slot;
@@ -1475,17 +1541,21 @@ lp_status lp_solve_recorded(lp_handle h, int64_t iters, void *cuda_stream) {
     LP_CU(cudaMemcpyAsync(c + n, h->v.y, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
     LP_CU(cudaMemcpyAsync(c + n + m, h->v.xbar, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     LP_CU(cudaMemcpyAsync(c + 2 * n + m, h->v.ybar, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    DevState hs{};
-    LP_CU(cudaMemcpyAsync(&hs, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
-    LP_CU(cudaStreamSynchronize(s));
-    if (hs.status != kRunning) return fail(LP_ERR_NUMERICAL, "solve stopped during recording");
-    h->ckpt_t0[b] = hs.t0;
-    const int64_t restarts_before = hs.restarts;
+    launch_record(h->st, h->rec_t0 + b, h->rec_t0 + blocks, nullptr, h->rec_flag, s);
     LP_CU(cudaGraphLaunch(h->exec, s));
-    LP_CU(cudaMemcpyAsync(&hs, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
-    LP_CU(cudaStreamSynchronize(s));
-    h->ckpt_restart[b] = (hs.restarts > restarts_before) ? 1 : 0;
+    // a stop in the last block's check does not spoil the recording
+    launch_record(h->st, nullptr, h->rec_t0 + blocks, h->rec_rs + b,
+                  b + 1 < blocks ? h->rec_flag : h->rec_flag + 1, s);
   }
+  LP_CU(cudaGetLastError());
+  h->ckpt_t0.assign(blocks, 0);
+  h->ckpt_restart.assign(blocks, 0);
+  int32_t stopped = 0;
+  LP_CU(cudaMemcpyAsync(h->ckpt_t0.data(), h->rec_t0, sizeof(int64_t) * blocks, cudaMemcpyDeviceToHost, s));
+  LP_CU(cudaMemcpyAsync(h->ckpt_restart.data(), h->rec_rs, sizeof(int8_t) * blocks, cudaMemcpyDeviceToHost, s));
+  LP_CU(cudaMemcpyAsync(&stopped, h->rec_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  LP_CU(cudaStreamSynchronize(s));
+  if (stopped) return fail(LP_ERR_NUMERICAL, "solve stopped during recording");
   h->rec_blocks = blocks;
   h->solved = true;
   return LP_OK;
@@ -1501,10 +1571,6 @@ lp_status lp_backward(lp_handle h, const double *dl_dx, const double *dl_dy, dou
   h->use_stream(s);
   const int n = h->n, m = h->m, K = h->opt.check_every;
   const int64_t slot = 2 * (int64_t)n + 2 * (int64_t)m;
-  DevState hs{};
-  LP_CU(cudaMemcpyAsync(&hs, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
-  LP_CU(cudaStreamSynchronize(s));
-  const double tau = hs.tau, sigma = hs.sigma;
   // adjoint seeds: gradients of the loss with respect to the final averages
   launch_fill(h->adj.ax, 0.0, n, s);
   launch_fill(h->adj.ac, 0.0, n, s);
@@ -1522,43 +1588,32 @@ lp_status lp_backward(lp_handle h, const double *dl_dx, const double *dl_dy, dou
   } else {
     launch_fill(h->adj.ayb, 0.0, m, s);
   }
-  for (int64_t b = h->rec_blocks - 1; b >= 0; --b) {
-    // recompute the block's forward steps with their masks
-    const double *c = h->ckpt + b * slot;
-    LP_CU(cudaMemcpyAsync(h->v.x, c, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-    LP_CU(cudaMemcpyAsync(h->v.y, c + n, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    LP_CU(cudaMemcpyAsync(h->v.xbar, c + n + m, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-    LP_CU(cudaMemcpyAsync(h->v.ybar, c + 2 * n + m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    const int64_t t0 = h->ckpt_t0[b];
-    auto wk = [&](int k) { return 1.0 / (double)(t0 + k + 1); };
-    for (int k = 0; k < K; ++k)
-      launch_forward_masked(h->A, h->AT, h->v, tau, sigma, wk(k), h->mask_x + (int64_t)k * n,
-                            h->mask_y + (int64_t)k * m, s);
-    // reverse through the block
-    launch_adjoint_block_start(h->adj, h->mask_y + (int64_t)(K - 1) * m, h->ckpt_restart[b],
-                               sigma, wk(K - 1), n, m, s);
-    for (int k = K - 1; k >= 0; --k)
-      launch_adjoint_step(h->A, h->AT, h->adj, h->mask_x + (int64_t)k * n,
-                          k > 0 ? h->mask_y + (int64_t)(k - 1) * m : nullptr, tau, sigma, wk(k),
-                          k > 0 ? wk(k - 1) : 0.0, k > 0 ? 1 : 0, s);
-    LP_CU(cudaGetLastError());
+  int32_t expired = 0;
+  bool launched = false;
+  if (h->res_blocks > 0 && h->adj_smem > 0) {  // one launch for all blocks
+    AdjointArgs q{};
+    q.r = h->res;
+    q.adj = h->adj;
+    q.ckpt = h->ckpt;
+    q.slot = slot;
+    q.blocks = h->rec_blocks;
+    q.mstride = m;
+    q.t0 = h->rec_t0;
+    q.restarted = h->rec_rs;
+    q.mask_x = h->mask_x;
+    q.mask_y = h->mask_y;
+    q.expired = h->rec_flag;
+    q.K = K;
+    q.count = 1;
+    LP_CU(cudaMemsetAsync(h->rec_flag, 0, sizeof(int32_t), s));
+    LP_CU(cudaMemsetAsync(h->res.bar, 0, sizeof(unsigned) * kResBarLines * 32, s));
+    launched = launch_adjoint(q, h->res_blocks, h->adj_smem, s) == cudaSuccess;
+    if (!launched) cudaGetLastError();
+    LP_CU(cudaMemcpyAsync(&expired, h->rec_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   }
-  // restore the final state of the recorded solve: replay the last block
-  {
-    const int64_t b = h->rec_blocks - 1;
-    const double *c = h->ckpt + b * slot;
-    LP_CU(cudaMemcpyAsync(h->v.x, c, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-    LP_CU(cudaMemcpyAsync(h->v.y, c + n, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    LP_CU(cudaMemcpyAsync(h->v.xbar, c + n + m, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-    LP_CU(cudaMemcpyAsync(h->v.ybar, c + 2 * n + m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    const int64_t t0 = h->ckpt_t0[b];
-    for (int k = 0; k < K; ++k)
-      launch_forward_masked(h->A, h->AT, h->v, tau, sigma, 1.0 / (double)(t0 + k + 1),
-                            h->mask_x + (int64_t)k * n, h->mask_y + (int64_t)k * m, s);
-    if (h->ckpt_restart[b]) {  // the recorded check restarted: z <- zbar
-      LP_CU(cudaMemcpyAsync(h->v.x, h->v.xbar, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-      LP_CU(cudaMemcpyAsync(h->v.y, h->v.ybar, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    }
+  if (!launched) {
+    const lp_status e = backward_by_passes(h, s);
+    if (e != LP_OK) return e;
   }
   if (dl_dc) {
     launch_scatter(h->tmp, h->adj.ac, h->perm_x, n, s);
@@ -1571,6 +1626,7 @@ lp_status lp_backward(lp_handle h, const double *dl_dx, const double *dl_dy, dou
   }
   LP_CU(cudaGetLastError());
   LP_CU(cudaStreamSynchronize(s));
+  if (expired) return fail(LP_ERR_TIMEOUT, "a device-side barrier wait expired");
   return LP_OK;
 }
 

@@ -1201,6 +1201,7 @@ struct lp_batch {
   ResidentArgs res{};     // cluster kernel (lp_resident.cu), when res.cluster > 0
   size_t res_smem = 0;
   bool res_inside = false;  // the matrix stays in shared memory
+  size_t adj_smem = 0;      // adjoint kernel in the same clusters (0: the per-pass kernels)
 
   ~lp_batch() {
     if (ckpt) cudaFree(ckpt);
@@ -1603,7 +1604,7 @@ void plan_batch_resident(lp_batch *h, const HostSell &HA, const HostSell &HAT,
   int C = 1;
   while (C < kMaxCluster && (int64_t)h->count * C <= h->nsm) C *= 2;  // at most two blocks per SM
   if (largest / C > std::max(kLaunchCycles, kImbalance * total / h->nsm)) return;
-  size_t with = 0, without = 0;
+  size_t with = 0, without = 0, adjoint = 0;
   for (const BInst &B : hi)
     for (int b = 0; b < C; ++b) {
       int cols = 0, rows = 0, nc = 0, nr = 0;
@@ -1620,12 +1621,15 @@ void plan_batch_resident(lp_batch *h, const HostSell &HA, const HostSell &HAT,
                                                 B.ncol, B.nrow);
       without = std::max(without, fixed);
       with = std::max(with, fixed + (size_t)(elems * elem));
+      adjoint = std::max(adjoint, adjoint_fixed_bytes(nc, nr, cols, rows, opt.check_every, B.ncol,
+                                                      B.nrow) + (size_t)(elems * elem));
     }
   const int64_t per_sm = ((int64_t)h->count * C + h->nsm - 1) / h->nsm;
   h->res_inside = per_sm <= 2 && (int64_t)with * per_sm <= (int64_t)limit;
   h->res_smem = h->res_inside ? with : without;
   if (h->res_smem > limit || !cluster_fits(C, h->res_smem, h->mixed, h->res_inside, true)) return;
   h->res.cluster = C;
+  if (!h->mixed && adjoint <= limit && adjoint_fits(1, 1, C, adjoint)) h->adj_smem = adjoint;
 }
 
 double ms_since(std::chrono::steady_clock::time_point t0) {
@@ -2483,28 +2487,48 @@ lp_status lp_batch_backward(lp_batch_handle h, const double *dl_dx, const double
     for (int k = 0; k < K; ++k) h->launch_masked_step(k, h->wrec, s);
     return LP_OK;
   };
-  const int ga = blocks_for_slices(h->A.nslices), gat = blocks_for_slices(h->AT.nslices);
   const int64_t mstride = std::max(m, 1);
-  for (int64_t b = h->rec_blocks - 1; b >= 0; --b) {
-    lp_status e = restore(b);  // recompute the block's steps with their masks
-    if (e != LP_OK) return e;
-    b_adj_block_start_kernel<<<h->chunk_grid(), kBlock, 0, s>>>(
-        a, h->I, h->rec_rs + b * count, h->mask_y + (int64_t)(K - 1) * mstride, h->wrec, K);
-    for (int k = K - 1; k >= 0; --k) {
-      AdjColsEpi ce{a.ax, a.axb, a.ac, a.v, h->mask_x + (int64_t)k * n, 0.0, 0.0, 0.0};
-      b_adj_cols_kernel<<<gat, kBlock, 0, s>>>(h->AT, a.u, ce, h->I, h->sinst_at, h->wrec, K, k);
-      AdjRowsEpi re{a.ay, a.ayb, a.ab, a.u, k > 0 ? h->mask_y + (int64_t)(k - 1) * mstride : nullptr,
-                    0.0, 0.0, 0.0, k > 0 ? 1 : 0};
-      b_adj_rows_kernel<<<ga, kBlock, 0, s>>>(h->A, a.v, re, h->I, h->sinst_a, h->wrec, K, k);
-    }
-    LP_CU(cudaGetLastError());
+  bool launched = false;
+  if (h->res.cluster > 0 && h->adj_smem > 0) {  // one launch for all blocks, a cluster per problem
+    AdjointArgs q{};
+    q.r = h->res;
+    q.adj = a;
+    q.ckpt = h->ckpt;
+    q.slot = slot;
+    q.blocks = h->rec_blocks;
+    q.mstride = mstride;
+    q.t0 = h->rec_t0;
+    q.restarted = h->rec_rs;
+    q.mask_x = h->mask_x;
+    q.mask_y = h->mask_y;
+    q.K = K;
+    q.count = count;
+    launched = launch_adjoint(q, 0, h->adj_smem, s) == cudaSuccess;
+    if (!launched) cudaGetLastError();
   }
-  // restore the final state of the recorded solve: replay the last block
-  {
-    lp_status e = restore(h->rec_blocks - 1);
-    if (e != LP_OK) return e;
-    b_rec_restart_kernel<<<h->chunk_grid(), kBlock, 0, s>>>(h->v, h->I,
-                                                            h->rec_rs + (h->rec_blocks - 1) * count);
+  if (!launched) {
+    const int ga = blocks_for_slices(h->A.nslices), gat = blocks_for_slices(h->AT.nslices);
+    for (int64_t b = h->rec_blocks - 1; b >= 0; --b) {
+      lp_status e = restore(b);  // recompute the block's steps with their masks
+      if (e != LP_OK) return e;
+      b_adj_block_start_kernel<<<h->chunk_grid(), kBlock, 0, s>>>(
+          a, h->I, h->rec_rs + b * count, h->mask_y + (int64_t)(K - 1) * mstride, h->wrec, K);
+      for (int k = K - 1; k >= 0; --k) {
+        AdjColsEpi ce{a.ax, a.axb, a.ac, a.v, h->mask_x + (int64_t)k * n, 0.0, 0.0, 0.0};
+        b_adj_cols_kernel<<<gat, kBlock, 0, s>>>(h->AT, a.u, ce, h->I, h->sinst_at, h->wrec, K, k);
+        AdjRowsEpi re{a.ay, a.ayb, a.ab, a.u, k > 0 ? h->mask_y + (int64_t)(k - 1) * mstride : nullptr,
+                      0.0, 0.0, 0.0, k > 0 ? 1 : 0};
+        b_adj_rows_kernel<<<ga, kBlock, 0, s>>>(h->A, a.v, re, h->I, h->sinst_a, h->wrec, K, k);
+      }
+      LP_CU(cudaGetLastError());
+    }
+    // restore the final state of the recorded solve: replay the last block
+    {
+      lp_status e = restore(h->rec_blocks - 1);
+      if (e != LP_OK) return e;
+      b_rec_restart_kernel<<<h->chunk_grid(), kBlock, 0, s>>>(h->v, h->I,
+                                                              h->rec_rs + (h->rec_blocks - 1) * count);
+    }
   }
   if (dl_dc) {
     launch_scatter(h->tmp, a.ac, h->perm_x, n, s);

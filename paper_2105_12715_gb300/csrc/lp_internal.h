@@ -240,6 +240,19 @@ struct ResidentArgs {
   BGlobal *glob;
 };
 
+// Arguments of the adjoint kernels (lp_resident.cu).
+struct AdjointArgs {
+  ResidentArgs r;
+  AdjVecs adj;               // axb, ayb: the seeds; ac, ab: the results; v, u: exchanged (grid)
+  const double *ckpt;        // [blocks][slot]: x, y, xbar, ybar at block start
+  int64_t slot, blocks, mstride;
+  const int64_t *t0;         // [blocks][count] inner iterations at block start
+  const int8_t *restarted;   // [blocks][count]
+  uint8_t *mask_x, *mask_y;  // [K][n], [K][mstride]
+  int32_t *expired;          // set when a barrier's wait ran out
+  int32_t K, count;
+};
+
 // Launch with programmatic stream serialization: the kernel may be scheduled
 // while its predecessor in the stream finishes (it must call pdl_enter()
 // before reading the predecessor's results).  Works inside stream capture.
@@ -343,6 +356,8 @@ void launch_scatter(double *out, const double *in, const int32_t *perm, int64_t 
 void launch_project(const DevVecs &v, int n, int m, cudaStream_t s);
 void launch_fill(double *p, double val, int64_t n, cudaStream_t s);
 void launch_weights(DevState *st, double *w, cudaStream_t s);
+void launch_record(const DevState *st, int64_t *t0, int64_t *restarts, int8_t *restarted,
+                   int32_t *stopped, cudaStream_t s);
 void launch_norms(const DevVecs &v, DevState *st, double *partials, int pstride,
                   int grid, int n, int m, cudaStream_t s);
 size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed, int ncol,
@@ -352,6 +367,9 @@ bool resident_fits(int P, int nsm, size_t smem, bool mixed);
 bool cluster_fits(int C, size_t smem, bool mixed, bool res, bool batch);
 cudaError_t launch_cluster(const ResidentArgs &a, int problems, size_t smem, bool mixed, bool res,
                            cudaStream_t s);
+size_t adjoint_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, int ncol, int nrow);
+bool adjoint_fits(int P, int nsm, int cluster, size_t smem);
+cudaError_t launch_adjoint(const AdjointArgs &q, int P, size_t smem, cudaStream_t s);
 cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixed,
                             cudaStream_t s);
 int check_grid_for(const SellMat &A, int num_sms);

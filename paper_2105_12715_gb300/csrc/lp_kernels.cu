@@ -742,6 +742,20 @@ __global__ void weights_kernel(const DevState *st, double *w) {
   for (int k = threadIdx.x; k < st->K; k += blockDim.x) w[k] = 1.0 / (double)(t0 + k + 1);
 }
 
+// Recording for the adjoint, around a block's launches: the inner iteration
+// count and the outer count before it, whether its check restarted, and whether
+// the solve has stopped.
+__global__ void record_kernel(const DevState *st, int64_t *t0, int64_t *restarts, int8_t *restarted,
+                              int32_t *stopped) {
+  if (t0) {
+    *t0 = st->t0;
+    *restarts = st->restarts;
+  } else {
+    *restarted = st->restarts > *restarts ? 1 : 0;
+  }
+  if (st->status != kRunning) *stopped = 1;
+}
+
 // ------------------------------------------------------ power iteration
 
 __global__ void __launch_bounds__(kBlock) sumsq_kernel(const double *__restrict__ v, int64_t n,
@@ -1292,6 +1306,11 @@ void launch_adjoint_block_start(const AdjVecs &a, const uint8_t *my_last, int re
 
 void launch_advance(DevState *st, double *w, int r, cudaStream_t s) {
   advance_kernel<<<1, kBlock, 0, s>>>(st, w, r);
+}
+
+void launch_record(const DevState *st, int64_t *t0, int64_t *restarts, int8_t *restarted,
+                   int32_t *stopped, cudaStream_t s) {
+  record_kernel<<<1, 1, 0, s>>>(st, t0, restarts, restarted, stopped);
 }
 
 void launch_weights(DevState *st, double *w, cudaStream_t s) {

@@ -1235,6 +1235,260 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
   }
 }
 
+// ------------------------------------------------------------------ adjoint
+//
+// The whole of lp_backward (lp_batch_backward: of one problem) by the blocks of
+// one group: for every recorded block of K iterations, last first, the forward
+// steps from its checkpoint with their clamp and projection masks, then one
+// adjoint step per iteration in reverse (the recurrence of AdjColsEpi and
+// AdjRowsEpi).  Launched pass by pass this took four launches per iteration, 6 us
+// each; here a pass costs what it does in run_block (2k x 5k, 512 iterations, setup,
+// forward and backward: 12.1 ms instead of 19.3).  The running averages are recomputed only for the last
+// block, whose end is the state that the call leaves behind.
+template <int NT, class Link>
+__device__ __forceinline__ void run_adjoint(unsigned char *smem, const AdjointArgs &q,
+                                            const Share &sh, int problem, double tau, double sigma,
+                                            unsigned gen, Link &link) {
+  const ResidentArgs &a = q.r;
+  const int tid = (int)threadIdx.x, lane = tid & (kWarp - 1), warp = tid >> 5;
+  const int nc = sh.nc, nr = sh.nr, K = q.K;
+  unsigned char *p = smem;
+  Header *h = (Header *)carve(p, sizeof(Header));
+  double *ex = nullptr, *ey = nullptr;
+  if (Link::kCluster) {  // at the same place in every block: owners store into all of them
+    ex = (double *)carve(p, 8 * (size_t)sh.ncol);
+    ey = (double *)carve(p, 8 * (size_t)sh.nrow);
+  }
+  LSlice *cs = (LSlice *)carve(p, sizeof(LSlice) * nc), *rs = (LSlice *)carve(p, sizeof(LSlice) * nr);
+  double *w = (double *)carve(p, sizeof(double) * K);
+  if (warp == 0) build_slices<true>(a.AT, sh.c0, nc, sh.stride, sh.cfirst, cs, &h->ncl, &h->nce);
+  else if (warp == 1) build_slices<true>(a.A, sh.r0, nr, sh.stride, sh.rfirst, rs, &h->nrl, &h->nre);
+  if (tid == 0) h->dead = 0;
+  __syncthreads();
+  const int ncl = h->ncl, nrl = h->nrl;
+  auto array = [&](int count) { return (double *)carve(p, 8 * (size_t)count); };
+  int32_t *crow = (int32_t *)carve(p, 4 * (size_t)ncl), *rrow = (int32_t *)carve(p, 4 * (size_t)nrl);
+  int32_t *rt = (int32_t *)carve(p, 4 * (size_t)nrl);
+  double *c = array(ncl), *x = array(ncl), *xb = array(ncl), *ax = array(ncl), *axb = array(ncl),
+         *ac = array(ncl);
+  long long *lk = (long long *)array(ncl), *uk = (long long *)array(ncl);
+  double *b = array(nrl), *y = array(nrl), *yb = array(nrl), *ay = array(nrl), *ayb = array(nrl),
+         *ab = array(nrl);
+  int32_t *cidx = (int32_t *)carve(p, 4 * (size_t)h->nce);
+  double *cval = array(h->nce);
+  int32_t *ridx = (int32_t *)carve(p, 4 * (size_t)h->nre);
+  double *rval = array(h->nre);
+  load_slices<double, NT, true>(a.AT, a.AT.val, cs, nc, sh.row0, crow, cidx, cval);
+  load_slices<double, NT, true>(a.A, a.A.val, rs, nr, sh.col0, rrow, ridx, rval);
+  __syncthreads();
+  if constexpr (Link::kCluster) {
+    link.ex = ex;
+    link.ey = ey;
+    link.ax = (uint32_t)__cvta_generic_to_shared(ex);
+    link.ay = (uint32_t)__cvta_generic_to_shared(ey);
+  } else {
+    link.gen = gen;
+    link.dead = &h->dead;
+  }
+  for (int s = tid; s < ncl; s += NT) {
+    const int j = crow[s];
+    c[s] = a.v.c[j];
+    lk[s] = a.v.lbk[j];
+    uk[s] = a.v.ubk[j];
+    ax[s] = 0.0;
+    axb[s] = q.adj.axb[j];
+    ac[s] = 0.0;
+  }
+  for (int s = tid; s < nrl; s += NT) {
+    const int i = rrow[s];
+    b[s] = a.v.b[i];
+    rt[s] = (int)a.v.row_type[i];
+    ay[s] = 0.0;
+    ayb[s] = q.adj.ayb[i];
+    ab[s] = 0.0;
+  }
+  __syncthreads();
+  // sum of one local column / row slice, with its owner lane's slot (-1: none)
+  auto col_sum = [&](int i, bool init, int *slot) {
+    const LSlice sl = cs[i];
+    const int lg = sl.lg(), r = lane >> lg, s = sl.slot0 + r;
+    *slot = (lane & ((1 << lg) - 1)) == 0 && r < sl.rows() ? s : -1;
+    return slice_sum<false>(init && *slot >= 0 ? -c[s] : 0.0, cidx + sl.soff + lane,
+                            cval + sl.soff + lane, sl.steps(), lg, link.y(), 0);
+  };
+  auto row_sum = [&](int i, bool init, int *slot) {
+    const LSlice sl = rs[i];
+    const int lg = sl.lg(), r = lane >> lg, s = sl.slot0 + r;
+    *slot = (lane & ((1 << lg) - 1)) == 0 && r < sl.rows() ? s : -1;
+    return slice_sum<false>(init && *slot >= 0 ? -b[s] : 0.0, ridx + sl.soff + lane,
+                            rval + sl.soff + lane, sl.steps(), lg, link.x(), 0);
+  };
+
+  bool ok = true;
+  for (int64_t blk = q.blocks - 1; ok && blk >= 0; --blk) {
+    const double *ck = q.ckpt + blk * q.slot;
+    const bool final = blk == q.blocks - 1;
+    const int64_t t0 = q.t0[blk * q.count + problem];
+    const int restarted = q.restarted[blk * q.count + problem];
+    for (int k = tid; k < K; k += NT) w[k] = 1.0 / (double)(t0 + k + 1);
+    for (int s = tid; s < ncl; s += NT) {
+      const int j = crow[s];
+      x[s] = ck[j];
+      if (final) xb[s] = ck[(int64_t)a.n + a.m + j];
+    }
+    for (int s = tid; s < nrl; s += NT) {
+      const int i = rrow[s];
+      y[s] = ck[(int64_t)a.n + i];
+      if (final) yb[s] = ck[2 * (int64_t)a.n + a.m + i];
+    }
+    // a cluster's first stores into the other blocks' copies wait until all have started
+    if (Link::kCluster) ok = link.sync();
+    else __syncthreads();
+    for (int s = tid; s < nrl; s += NT) link.put_y(rrow[s], y[s]);
+    ok = ok && link.sync();
+    // ---- forward steps with masks
+    for (int k = 0; ok && k < K; ++k) {
+      for (int r = 0, i, s; (i = pick<NT>(r, warp)) < nc; ++r) {
+        const double neg_g = col_sum(i, true, &s);
+        if (s >= 0) {
+          const double xo = x[s];
+          long long key = ord_key(__double_as_longlong(fma(tau, neg_g, xo)));
+          const long long lo = lk[s], hi = uk[s];
+          q.mask_x[(int64_t)k * a.n + crow[s]] = key > lo && key < hi ? 1 : 0;
+          key = key < lo ? lo : key;
+          key = key > hi ? hi : key;
+          const double xn = __longlong_as_double(ord_key(key));
+          link.put_x(crow[s], fma(2.0, xn, -xo));
+          x[s] = xn;
+          if (final) xb[s] = fma(w[k], xn - xb[s], xb[s]);
+        }
+      }
+      if (!(ok = link.sync())) break;
+      for (int r = 0, i, s; (i = pick<NT>(r, warp)) < nr; ++r) {
+        const double res = row_sum(i, true, &s);
+        if (s >= 0) {
+          long long bits = __double_as_longlong(fma(-sigma, res, y[s]));
+          const int t = rt[s];
+          q.mask_y[(int64_t)k * q.mstride + rrow[s]] =
+              t == 0 || (t == 1 && bits > 0) || (t == 2 && bits < 0) ? 1 : 0;
+          if ((t == 1 && bits < 0) || (t == 2 && bits > 0)) bits = 0;
+          const double yn = __longlong_as_double(bits);
+          if (k + 1 < K) link.put_y(rrow[s], yn);  // the last y is gathered by nobody
+          y[s] = yn;
+          if (final) yb[s] = fma(w[k], yn - yb[s], yb[s]);
+        }
+      }
+      if (k + 1 < K) ok = link.sync();
+    }
+    if (!ok) break;
+    __syncthreads();
+    if (final) {  // the state of the recorded solve (its last check may have restarted)
+      for (int s = tid; s < ncl; s += NT) {
+        a.v.x[crow[s]] = restarted ? xb[s] : x[s];
+        a.v.xbar[crow[s]] = xb[s];
+      }
+      for (int s = tid; s < nrl; s += NT) {
+        a.v.y[rrow[s]] = restarted ? yb[s] : y[s];
+        a.v.ybar[rrow[s]] = yb[s];
+      }
+    }
+    // ---- start of the reverse block: its restart, then u of its last step
+    if (restarted)
+      for (int s = tid; s < ncl; s += NT) {
+        axb[s] += ax[s];
+        ax[s] = 0.0;
+      }
+    for (int s = tid; s < nrl; s += NT) {
+      if (restarted) {
+        ayb[s] += ay[s];
+        ay[s] = 0.0;
+      }
+      const double up =
+          q.mask_y[(int64_t)(K - 1) * q.mstride + rrow[s]] ? fma(w[K - 1], ayb[s], ay[s]) : 0.0;
+      ab[s] = fma(sigma, up, ab[s]);
+      ayb[s] = (1.0 - w[K - 1]) * ayb[s];
+      ay[s] = up;  // holds u between the passes
+      link.put_y(rrow[s], up);
+    }
+    ok = link.sync();
+    // ---- adjoint steps
+    for (int k = K - 1; ok && k >= 0; --k) {
+      const double wk = w[k], wp = k > 0 ? w[k - 1] : 0.0;
+      for (int r = 0, i, s; (i = pick<NT>(r, warp)) < nc; ++r) {
+        const double atu = col_sum(i, false, &s);
+        if (s >= 0) {
+          const double adj_xhat = -sigma * atu;
+          const double adj_xp = fma(2.0, adj_xhat, fma(wk, axb[s], ax[s]));
+          const double vv = q.mask_x[(int64_t)k * a.n + crow[s]] ? adj_xp : 0.0;
+          link.put_x(crow[s], vv);
+          ax[s] = vv - adj_xhat;
+          ac[s] = fma(-tau, vv, ac[s]);
+          axb[s] = (1.0 - wk) * axb[s];
+        }
+      }
+      if (!(ok = link.sync())) break;
+      for (int r = 0, i, s; (i = pick<NT>(r, warp)) < nr; ++r) {
+        const double av = row_sum(i, false, &s);
+        if (s >= 0) {
+          const double ayk = fma(tau, av, ay[s]);
+          if (k > 0) {
+            const double up =
+                q.mask_y[(int64_t)(k - 1) * q.mstride + rrow[s]] ? fma(wp, ayb[s], ayk) : 0.0;
+            link.put_y(rrow[s], up);
+            ab[s] = fma(sigma, up, ab[s]);
+            ayb[s] = (1.0 - wp) * ayb[s];
+            ay[s] = up;
+          } else {
+            ay[s] = ayk;
+          }
+        }
+      }
+      if (k > 0) ok = link.sync();
+    }
+    __syncthreads();
+  }
+  if (!ok) {
+    if (tid == 0) *q.expired = 1;
+    return;
+  }
+  for (int s = tid; s < ncl; s += NT) q.adj.ac[crow[s]] = ac[s];
+  for (int s = tid; s < nrl; s += NT) q.adj.ab[rrow[s]] = ab[s];
+  if (Link::kCluster) link.sync();  // no block leaves while another may store into its copies
+}
+
+__global__ void __launch_bounds__(kGridThreads, 1)
+    adjoint_kernel(const __grid_constant__ AdjointArgs q) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const ResidentArgs &a = q.r;
+  const int P = (int)gridDim.x, b = (int)blockIdx.x;
+  const Share sh{b, (a.AT.nslices - b + P - 1) / P, b, (a.A.nslices - b + P - 1) / P, P, 0, 0,
+                 0, a.n, 0, a.m, b, P};
+  GridLink<double> link{a.bar, 0u, nullptr, q.adj.v, q.adj.u};
+  run_adjoint<kGridThreads>(smem, q, sh, 0, a.st->tau, a.st->sigma, 0u, link);
+}
+
+__global__ void __launch_bounds__(kClusterThreads, 2)
+    adjoint_cluster_kernel(const __grid_constant__ AdjointArgs q) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const ResidentArgs &a = q.r;
+  const int C = a.cluster, rank = (int)blockIdx.x % C, problem = (int)blockIdx.x / C;
+  ClusterLink<double> link{};
+  link.C = C;
+  if (a.inst) {
+    const BInst &B = a.inst[problem];
+    const Share sh{B.cs0 + rank, (B.cs1 - B.cs0 - rank + C - 1) / C,
+                   B.rs0 + rank, (B.rs1 - B.rs0 - rank + C - 1) / C,
+                   C, B.cs0, B.rs0, B.col0, B.ncol, B.row0, B.nrow, rank, C};
+    link.col0 = sh.col0;
+    link.row0 = sh.row0;
+    run_adjoint<kClusterThreads>(smem, q, sh, problem, B.tau, B.sigma, 0u, link);
+  } else {
+    const Share sh{rank, (a.AT.nslices - rank + C - 1) / C, rank, (a.A.nslices - rank + C - 1) / C,
+                   C, 0, 0, 0, a.n, 0, a.m, rank, C};
+    run_adjoint<kClusterThreads>(smem, q, sh, 0, a.st->tau, a.st->sigma, 0u, link);
+  }
+}
+
 // One problem over the whole grid (cooperative launch).
 template <typename T>
 __global__ void __launch_bounds__(kGridThreads, 1)
@@ -1320,6 +1574,12 @@ size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed,
          16 * 28;
 }
 
+// The same for the adjoint kernels (the carving of run_adjoint).
+size_t adjoint_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, int ncol, int nrow) {
+  return sizeof(Header) + sizeof(LSlice) * ((size_t)nc + nr) + (4 + 8 * 8) * (size_t)ncl +
+         (8 + 6 * 8) * (size_t)nrl + 8 * ((size_t)ncol + nrow) + 8 * (size_t)K + 16 * 28;
+}
+
 // Largest dynamic shared memory of the kernels on the current device; 0 when it cannot launch
 // them (no cooperative launch).
 size_t resident_smem_limit(int device, bool mixed) {
@@ -1335,6 +1595,8 @@ size_t resident_smem_limit(int device, bool mixed) {
     return 0;
   for (int i = 0; i < 4; ++i)
     if (!set_smem(cluster_of(mixed, i & 1, i & 2), optin)) return 0;
+  if (!mixed && !(set_smem(adjoint_kernel, optin) && set_smem(adjoint_cluster_kernel, optin)))
+    return 0;
   return (size_t)optin;
 }
 
@@ -1383,6 +1645,47 @@ cudaLaunchConfig_t cluster_config(int problems, int C, size_t smem, cudaLaunchAt
   return cfg;
 }
 }  // namespace
+
+// lp_backward's recurrence over all recorded blocks: one problem on P blocks, or
+// one cluster per problem.
+cudaError_t launch_adjoint(const AdjointArgs &q, int P, size_t smem, cudaStream_t s) {
+  cudaLaunchAttribute at[1];
+  if (q.r.cluster > 0) {
+    cudaLaunchConfig_t cfg = cluster_config(q.count, q.r.cluster, smem, at);
+    cfg.stream = s;
+    return cudaLaunchKernelEx(&cfg, adjoint_cluster_kernel, q);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)P);
+  cfg.blockDim = dim3(kGridThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, adjoint_kernel, q);
+}
+
+// Whether the adjoint kernel's blocks (clusters) fit.
+bool adjoint_fits(int P, int nsm, int cluster, size_t smem) {
+  int n = 0;
+  cudaError_t e;
+  if (cluster > 0) {
+    cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg = cluster_config(1, cluster, smem, at);
+    e = cudaOccupancyMaxActiveClusters(&n, adjoint_cluster_kernel, &cfg);
+    P = 1;
+    nsm = 1;
+  } else {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, adjoint_kernel, kGridThreads, smem);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (int64_t)n * nsm >= P;
+}
 
 // Whether the device can hold a cluster of C blocks with smem bytes each.
 bool cluster_fits(int C, size_t smem, bool mixed, bool res, bool batch) {

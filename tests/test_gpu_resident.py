@@ -155,3 +155,47 @@ def test_batch_check_periods_and_schemes(lpm):
         for u, v in zip(got[0][1], got[1][1]):
             for k in ("iters", "restarts", "checks", "status", "returned"):
                 assert u[k] == v[k], (scheme, k)
+
+
+@pytest.mark.parametrize("name", ["31x33", "200x400", "empty_lines", "997x4999"])
+def test_adjoint_is_the_per_pass_adjoint(lpm, name):
+    """One launch for the whole reverse sweep against the launches pass by pass:
+    the same recurrence with the same sums; only c and b's gradients and the state
+    left behind come back."""
+    data = CASES[name]()
+    rng = np.random.default_rng(5)
+    wx, wy = rng.standard_normal(data.n), rng.standard_normal(data.m)
+    out = []
+    for autotune in (1, 0):
+        with lpm.LP(data, eta=0.05, autotune=autotune, check_every=20) as g:
+            lpm.lp_solve_recorded(g.h, 100)
+            before = g.state()
+            dc, db = np.empty(data.n), np.empty(data.m)
+            for _ in range(2):  # a second call repeats the first
+                lpm.lp_backward(g.h, wx, wy, dc, db)
+            after = g.state()
+            for k in before:
+                np.testing.assert_array_equal(after[k], before[k], err_msg=k)
+            out.append((dc, db, g.info().graph_kernels))
+    assert out[0][2] == 1 and out[1][2] > 1
+    # per-pass launches contract the recurrence's products into FMAs differently
+    for a, b in zip(out[0][:2], out[1][:2]):
+        np.testing.assert_allclose(a, b, rtol=0, atol=1e-12 * max(1.0, np.abs(b).max(initial=0.0)))
+
+
+def test_batch_adjoint_is_the_per_pass_adjoint(lpm):
+    for probs in (BATCHES["3_uneven"](), BATCHES["640"]()):
+        n, m = sum(p.n for p in probs), sum(p.m for p in probs)
+        rng = np.random.default_rng(6)
+        wx, wy = rng.standard_normal(n), rng.standard_normal(m)
+        out = []
+        for autotune in (1, 0):
+            with lpm.LPBatch(probs, eta=0.05, autotune=autotune, check_every=16) as g:
+                g.solve_recorded(80)
+                before = g.state()
+                out.append(g.backward(wx, wy))
+                after = g.state()
+                for k in before:
+                    np.testing.assert_array_equal(after[k], before[k], err_msg=k)
+        for a, b in zip(*out):
+            np.testing.assert_allclose(a, b, rtol=0, atol=1e-12 * max(1.0, np.abs(b).max()))
