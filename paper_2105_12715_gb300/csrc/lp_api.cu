@@ -87,6 +87,7 @@ struct lp_problem {
   double setup_ms[4] = {0, 0, 0, 0};  // lp_create phases (lp_info.setup_ms)
   int32_t sigma_steps = 0;            // Lanczos / power-iteration steps taken for sigma_max
   int32_t graph_kernels = 0;          // kernel nodes of the K-iteration graph
+  unsigned int *bar = nullptr;          // counters of the grid barrier, when a kernel uses one
   ResidentArgs res{};                 // resident kernel (lp_resident.cu), when res_blocks > 0
   int res_blocks = 0;
   size_t res_smem = 0;
@@ -227,8 +228,8 @@ cudaError_t capture_block(lp_problem *h) {
                    : launch_resident(h->res, h->res_blocks, h->res_smem, h->mixed, s);
   } else {
     for (int k = 0; k < h->opt.check_every; ++k) launch_iteration(h, k, s);
-    launch_check(h->A, h->AT, h->v, h->st, h->w, h->cs, h->n, h->m, h->nsearch, h->trace, true, s,
-                 h->mixed ? &h->mv : nullptr);
+    launched = launch_check(h->A, h->AT, h->v, h->st, h->w, h->cs, h->n, h->m, h->nsearch, h->trace,
+                            true, s, h->mixed ? &h->mv : nullptr);
   }
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(s, &g);
@@ -246,9 +247,10 @@ cudaError_t capture_block(lp_problem *h) {
 lp_status build_graph(lp_problem *h) {
   if (h->exec) return LP_OK;
   cudaError_t e = capture_block(h);
-  if (e != cudaSuccess && h->res_blocks > 0) {  // no cooperative launch here: the per-pass kernels
-    cudaGetLastError();
+  if (e != cudaSuccess && (h->res_blocks > 0 || h->cs.search_blocks > 0)) {
+    cudaGetLastError();  // no cooperative launch here: the per-pass kernels
     h->res_blocks = 0;
+    h->cs.search_blocks = 0;
     e = capture_block(h);
   }
   if (e != cudaSuccess) return cuda_fail(e, "capture of an iteration block");
@@ -273,8 +275,8 @@ lp_status set_run_params(lp_problem *h, double tol, cudaStream_t s) {
   const int32_t running = kRunning;
   LP_CU(cudaMemcpyAsync(&h->st->tol, &tol, sizeof(double), cudaMemcpyHostToDevice, s));
   LP_CU(cudaMemcpyAsync(&h->st->status, &running, sizeof(int32_t), cudaMemcpyHostToDevice, s));
-  if (h->res_blocks > 0) {  // grid barrier: counters and generation from zero
-    LP_CU(cudaMemsetAsync(h->res.bar, 0, sizeof(unsigned) * kResBarLines * 32, s));
+  if (h->bar) {  // grid barrier: counters and generation from zero
+    LP_CU(cudaMemsetAsync(h->bar, 0, sizeof(unsigned) * kResBarLines * 32, s));
     LP_CU(cudaMemsetAsync(&h->st->bar_gen, 0, sizeof(unsigned), s));
   }
   return LP_OK;
@@ -350,7 +352,8 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
   lp_status e;
   if ((e = h->alloc(&h->res.part, (int64_t)P * kResPart)) != LP_OK) return e;
   if ((e = h->alloc(&h->res.npart, (int64_t)2 * P * 8)) != LP_OK) return e;
-  if ((e = h->alloc(&h->res.bar, kResBarLines * 32)) != LP_OK) return e;
+  if ((e = h->alloc(&h->bar, kResBarLines * 32)) != LP_OK) return e;
+  h->res.bar = h->bar;
   if (h->mixed &&
       (e = h->alloc(&h->res.rpart, (int64_t)2 * (h->cs.cols_grid + h->cs.rows_grid))) != LP_OK)
     return e;
@@ -371,6 +374,21 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
   h->res.m = h->m;
   h->res_smem = smem;
   h->res_blocks = P;
+  return LP_OK;
+}
+
+// The multiplier search of the per-pass check in one cooperative launch, with
+// autotune on (without it the check keeps its fixed sequence of launches).
+lp_status plan_search(lp_problem *h) {
+  if (!h->opt.autotune || h->res_blocks > 0 || h->nsearch == 0) return LP_OK;
+  const int64_t N = (int64_t)h->n + h->m;
+  const int P = (int)std::min<int64_t>(h->nsm, (N + kSearchBlockElems - 1) / kSearchBlockElems);
+  if (!search_fits(P, h->nsm)) return LP_OK;
+  lp_status e;
+  if ((e = h->alloc(&h->cs.npart, (int64_t)2 * P * 8)) != LP_OK) return e;
+  if ((e = h->alloc(&h->bar, kResBarLines * 32)) != LP_OK) return e;
+  h->cs.bar = h->bar;
+  h->cs.search_blocks = P;
   return LP_OK;
 }
 
@@ -1173,6 +1191,7 @@ lp_status lp_create(int32_t m, int32_t n, int64_t nnz, const int32_t *row_ptr,
   LP_CU(cudaMemcpyAsync(&h->st->tau, &tau, sizeof(double), cudaMemcpyHostToDevice, s));
   LP_CU(cudaMemcpyAsync(&h->st->sigma, &sigma, sizeof(double), cudaMemcpyHostToDevice, s));
   if ((e = plan_resident(h.get(), s)) != LP_OK) return e;
+  if ((e = plan_search(h.get())) != LP_OK) return e;
   if (opt.autotune && h->res_blocks == 0 && (e = tune_variants(h.get(), s)) != LP_OK) return e;
   // z^{0,0} = proj(0)
   launch_fill(h->v.x, 0.0, n, s);
@@ -1437,6 +1456,7 @@ lp_status lp_normalized_gap(lp_handle h, const double *x, const double *y, doubl
   LP_CU(cudaStreamSynchronize(s));
   cs.pair_x = cs.pair_y = nullptr;  // the handle's pair buffers belong to its solve
   cs.cand[0] = cs.cand[1] = nullptr;  // and so do its candidate lists: full scans
+  cs.search_blocks = 0;               // and the search's barrier
   launch_check(A, AT, v, st, nullptr, cs, n, m, 1, nullptr, false, s);
   LP_CU(cudaGetLastError());
   LSearch L{};
@@ -1606,7 +1626,7 @@ lp_status lp_backward(lp_handle h, const double *dl_dx, const double *dl_dy, dou
     q.K = K;
     q.count = 1;
     LP_CU(cudaMemsetAsync(h->rec_flag, 0, sizeof(int32_t), s));
-    LP_CU(cudaMemsetAsync(h->res.bar, 0, sizeof(unsigned) * kResBarLines * 32, s));
+    LP_CU(cudaMemsetAsync(h->bar, 0, sizeof(unsigned) * kResBarLines * 32, s));
     launched = launch_adjoint(q, h->res_blocks, h->adj_smem, s) == cudaSuccess;
     if (!launched) cudaGetLastError();
     LP_CU(cudaMemcpyAsync(&expired, h->rec_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -1796,6 +1816,7 @@ extern "C" lp_status lp_normalized_gap_static(lp_handle h, const double *x, cons
   LP_CU(cudaMemcpyAsync(st, &hs, sizeof(DevState), cudaMemcpyHostToDevice, s));
   cs.pair_x = cs.pair_y = nullptr;  // the handle's pair buffers belong to its solve
   cs.cand[0] = cs.cand[1] = nullptr;  // and so do its candidate lists: full scans
+  cs.search_blocks = 0;               // and the search's barrier
   launch_check(A, AT, v, st, nullptr, cs, n, m, 1, nullptr, false, s);
   LP_CU(cudaGetLastError());
   LSearch L{};

@@ -22,10 +22,8 @@
 //   b_finalize: one block per due problem: its sums, relative KKT,
 //       termination, radius, search setup;
 //   b_search: one block (or an 8-block cluster for large problems) per due
-//       problem: the multiplier search of Section 6.3 (radix passes over
-//       the breakpoints' bit patterns from their common prefix down,
-//       per-warp histograms, per-warp candidate lists after the first pass,
-//       bracket selection in-block);
+//       problem: the multiplier search of Section 6.3 (Newton steps over the
+//       breakpoints);
 //   b_decide: restart rule, counters, running count (one thread per problem);
 //   b_restart_copy: z^{n+1,0} <- zbar, z <- zbar for restarting problems;
 //   b_list_scan / b_list_fill: the next block's slice work lists and
@@ -61,16 +59,11 @@ constexpr int kMaxClasses = 8;
 constexpr int kStatusIterLimit = 4;
 constexpr int kListThreads = 1024;
 constexpr int kSearchWarps = 8;
-constexpr int kSearchThreads = kSearchWarps * kWarp;  // one thread per bucket
-static_assert(kSearchThreads == kBuckets, "bracket selection uses one thread per bucket");
-constexpr size_t kSearchHistBytes = sizeof(double) * kSearchWarps * kBuckets * 3;
-constexpr size_t kSearchCntBytes = sizeof(unsigned) * kSearchWarps * kBuckets;
-constexpr size_t kSearchSmem = kSearchHistBytes + kSearchCntBytes + sizeof(double) * kSearchWarps * kWarp * 3;
+constexpr int kSearchThreads = kSearchWarps * kWarp;
 
 struct SearchArrays {
   uint64_t *keys[2];
   double *d2[2], *g2[2], *gd[2];
-  int32_t *cand[2];  // per-warp candidate lists, [n + m + 256 count] each
 };
 
 // ---------------------------------------------------------------- iteration
@@ -272,83 +265,30 @@ __global__ void __launch_bounds__(kBlock) b_finalize_kernel(BInst *I, const BGlo
   }
 }
 
-// One block per (due problem, candidate): the multiplier search of
-// Section 6.3 over the problem's breakpoints, with the bracket logic of the
-// single-problem solver (radix passes of 8 bits over the bit patterns of the
-// breakpoints, exact f at bucket edges, closed form on the final bracket),
-// organised for one block:
-//   * a first scan finds the smallest and largest breakpoint key; bits
-//     above their first difference are common to every key, so the passes
-//     start right below them (bracket [P, P + 2^(shift0+8)) with P the
-//     common prefix); if f exceeds r^2 already at P, lambda* lies below
-//     every breakpoint (closed form with all of them above it);
-//   * pass 0 scans every element; afterwards each warp gathers the elements
-//     of the chosen bucket into its own list (global scratch), and later
-//     passes scan only these lists;
-//   * full scans load four rounds of keys (and values) before using them.
-// Warp w owns elements w*32 + 256 t + lane; within a warp, equal buckets are
-// summed by their lowest lane in lane order; warps are combined in order:
-// the result is deterministic.
+// One block, or a cluster of CS, per (due problem, candidate): the multiplier
+// search of Section 6.3 by Newton's method (newton_next) over the problem's
+// breakpoints.  Thread t of the cluster owns elements t, t + CS 256, ..., four
+// in flight.  lambda only rises, so an element once clamped stays clamped: its
+// d^2 and d g go into the thread's running sums at the step that clamps it, and
+// a step reads all keys and g^2 and adds the g^2 of the others.  What bounds a
+// step is the FP64 pipe (19 cycles of the SM per warp and addition: one per 32
+// elements and six per warp to reduce) and, in a cluster, one barrier.  The
+// sums of a warp, a block and the cluster are taken in a fixed order, so the
+// result is deterministic and the same in every block.
 constexpr int kScanUnroll = 4;
-constexpr int kMaxCluster = 8;          // blocks per problem in the clustered search
-constexpr int64_t kClusterMinElems = 8192;  // problems with at least n + m elements use it
-
-__device__ __forceinline__ void hist_add(bool act, int bk, double vd, double vg, double ve,
-                                         double (*hist)[kBuckets][3], unsigned (*cnt)[kBuckets],
-                                         double (*stage)[kWarp][3], int warp, int lane) {
-  if (__ballot_sync(kFull, act) == 0u) return;
-  const unsigned grp = __match_any_sync(kFull, act ? bk : -1);
-  const bool leader = act && (grp & ((1u << lane) - 1u)) == 0u;
-  if (act) {
-    stage[warp][lane][0] = vd;
-    stage[warp][lane][1] = vg;
-    stage[warp][lane][2] = ve;
-  }
-  __syncwarp();
-  if (leader) {
-    double sd = 0.0, sg = 0.0, se = 0.0;
-    unsigned gm = grp;
-    while (gm) {
-      const int l = __ffs(gm) - 1;
-      gm &= gm - 1u;
-      sd += stage[warp][l][0];
-      sg += stage[warp][l][1];
-      se += stage[warp][l][2];
-    }
-    hist[warp][bk][0] += sd;
-    hist[warp][bk][1] += sg;
-    hist[warp][bk][2] += se;
-    cnt[warp][bk] += (unsigned)__popc(grp);
-  }
-  __syncwarp();
-}
-
-__device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v, int o) {
-  return (unsigned long long)__shfl_xor_sync(kFull, (long long)v, o);
-}
+constexpr int kMaxCluster = 8;  // blocks per problem in the clustered search
+constexpr int64_t kClusterMinElems = 2048;  // problems with at least n + m elements use it
 
 template <int CS>
 __global__ void __launch_bounds__(kSearchThreads) b_search_kernel(BInst *I,
                                                                   const int32_t *__restrict__ plist,
                                                                   int64_t nx_total,
                                                                   SearchArrays sa) {
-  const int pk = plist[blockIdx.x / CS];
-  BInst &B = I[pk];
+  BInst &B = I[plist[blockIdx.x / CS]];
   const int sidx = blockIdx.y;
   __shared__ LSearch L;
-  __shared__ double bc[kBuckets], bsd[kBuckets], bsg[kBuckets], bse[kBuckets];
-  __shared__ double lb[CS > 1 ? 2 : 1][4][kBuckets];  // this block's bucket sums (cluster exchange)
-  __shared__ double cum_d[kBuckets + 1], cum_e[kBuckets + 1], tail_g[kBuckets + 1];
-  __shared__ double wt[3][8];
-  __shared__ int kstar;
-  __shared__ unsigned long long wmin[kSearchWarps], wmax[kSearchWarps];
-  __shared__ int64_t wcnt[kSearchWarps];
-  extern __shared__ __align__(16) unsigned char dsm[];
-  double(*hist)[kBuckets][3] = reinterpret_cast<double(*)[kBuckets][3]>(dsm);
-  unsigned(*cnt)[kBuckets] = reinterpret_cast<unsigned(*)[kBuckets]>(dsm + kSearchHistBytes);
-  double(*stage)[kWarp][3] =
-      reinterpret_cast<double(*)[kWarp][3]>(dsm + kSearchHistBytes + kSearchCntBytes);
-  const int tid = threadIdx.x;
+  __shared__ double red[kSearchWarps][4], part[2][4], tot[4];
+  const int tid = threadIdx.x, lane = tid & (kWarp - 1), warp = tid >> 5;
   if (tid == 0) L = B.ls[sidx];
   __syncthreads();
   // every block of a cluster reads the same state: the whole cluster leaves together
@@ -361,253 +301,68 @@ __global__ void __launch_bounds__(kSearchThreads) b_search_kernel(BInst *I,
   const double *__restrict__ gd = sidx ? sa.gd[1] : sa.gd[0];
   const int64_t nx = B.ncol, N = nx + B.nrow;
   const int64_t xbase = B.col0, ybase = nx_total + B.row0 - nx;
-  const int lane = tid & (kWarp - 1), warp = tid >> 5;
-  const int gw = rank * kSearchWarps + warp;              // warp index in the cluster
   constexpr int64_t kRound = (int64_t)CS * kSearchThreads;  // elements per round of a cluster
-  const int64_t cap = ((N + kRound - 1) / kRound) * kWarp;
-  int32_t *list = (sidx ? sa.cand[1] : sa.cand[0]) + (int64_t)B.col0 + B.row0 +
-                  (int64_t)kMaxCluster * kSearchThreads * pk + gw * cap;
-  auto elem = [&](int64_t v) { return v < nx ? xbase + v : ybase + v; };
+  double ad = 0.0, ae = 0.0;  // this thread's sums of d^2 and d g over its clamped coordinates,
+  uint64_t last = 0ull;       // whose keys are below last,
+  int seen = 0;               // and their number
+  int count = -1;             // thread 0's
 
-  // smallest and largest breakpoint key (over the cluster)
-  {
-    unsigned long long lo = ~0ull, hi = 0ull;
-    for (int64_t base = (int64_t)gw * kWarp; base < N; base += kScanUnroll * kRound) {
+  for (int step = 0; step < kNewtonMax; ++step) {
+    const uint64_t to = (uint64_t)dbits(L.lambda) + 1;  // clamped: keys below to
+    double above = 0.0;
+    for (int64_t base = (int64_t)rank * kSearchThreads + tid; base < N;
+         base += kScanUnroll * kRound) {
       uint64_t k[kScanUnroll];
+      double g[kScanUnroll];
 #pragma unroll
       for (int r = 0; r < kScanUnroll; ++r) {
-        const int64_t v = base + r * kRound + lane;
-        k[r] = v < N ? keys[elem(v)] : kNoKey;
+        const int64_t v = base + r * kRound;
+        const int64_t e = (v < nx ? xbase : ybase) + v;
+        k[r] = v < N ? keys[e] : kNoKey;
+        g[r] = v < N ? g2[e] : 0.0;
       }
 #pragma unroll
       for (int r = 0; r < kScanUnroll; ++r) {
-        if (k[r] != kNoKey) {
-          lo = k[r] < lo ? k[r] : lo;
-          hi = k[r] > hi ? k[r] : hi;
-        }
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long a = shfl_xor_u64(lo, o), b = shfl_xor_u64(hi, o);
-      lo = a < lo ? a : lo;
-      hi = b > hi ? b : hi;
-    }
-    if (lane == 0) {
-      wmin[warp] = lo;
-      wmax[warp] = hi;
-    }
-  }
-  if (CS > 1) cluster.sync();
-  else __syncthreads();
-  unsigned long long kmin = ~0ull, kmax = 0ull;
-  for (int r = 0; r < CS; ++r) {
-    const unsigned long long *rmin = CS > 1 ? cluster.map_shared_rank(wmin, r) : wmin;
-    const unsigned long long *rmax = CS > 1 ? cluster.map_shared_rank(wmax, r) : wmax;
-    for (int w = 0; w < kSearchWarps; ++w) {
-      kmin = rmin[w] < kmin ? rmin[w] : kmin;
-      kmax = rmax[w] > kmax ? rmax[w] : kmax;
-    }
-  }
-  if (kmin > kmax) {  // no finite breakpoint: every coordinate moves without bound
-    if (tid == 0 && rank == 0) {
-      L.lambda = sqrt(fmax(L.r2 - L.f_lo, 0.0) / L.f_hi);
-      L.rho_r = L.e_lo + L.lambda * L.f_hi;
-      L.done = 1;
-      B.ls[sidx] = L;
-    }
-    if (CS > 1) cluster.sync();  // no block leaves while another may read its memory
-    return;
-  }
-  const int cp = (kmin == kmax) ? 64 : __clzll((long long)(kmin ^ kmax));
-  // bucket bits [shift0, shift0 + 8) hold the first differing bit (63 - cp);
-  // every bit from shift0 + 8 up is common to all keys
-  const int shift0 = (56 - cp) > 0 ? ((56 - cp + 7) / 8) * 8 : 0;
-  if (tid == 0) L.prefix = (shift0 + 8 >= 64) ? 0ull : (kmin & ~((1ull << (shift0 + 8)) - 1ull));
-  if (tid < kSearchWarps) wcnt[tid] = 0;
-  __syncthreads();
-
-  for (int shift = shift0, pass = 0; shift >= 0; shift -= 8, ++pass) {
-    const uint64_t pre = L.prefix;
-    for (int i = tid; i < kSearchWarps * kBuckets; i += kSearchThreads) {
-      double *h = &hist[0][0][0] + 3 * i;
-      h[0] = 0.0;
-      h[1] = 0.0;
-      h[2] = 0.0;
-      (&cnt[0][0])[i] = 0u;
-    }
-    __syncthreads();
-    const bool full_prefix = (shift + 8 >= 64);
-    auto match = [&](uint64_t k) {
-      return k != kNoKey && (full_prefix || (k >> (shift + 8)) == (pre >> (shift + 8)));
-    };
-    if (pass == 0) {
-      for (int64_t base = (int64_t)gw * kWarp; base < N; base += kScanUnroll * kRound) {
-        uint64_t k[kScanUnroll];
-        double a[kScanUnroll], b[kScanUnroll], c[kScanUnroll];
-#pragma unroll
-        for (int r = 0; r < kScanUnroll; ++r) {
-          const int64_t v = base + r * kRound + lane;
-          k[r] = kNoKey;
-          if (v < N) {
-            const int64_t e = elem(v);
-            k[r] = keys[e];
-            a[r] = d2[e];
-            b[r] = g2[e];
-            c[r] = gd[e];
+        if (k[r] < to) {
+          if (k[r] >= last) {
+            const int64_t v = base + r * kRound;
+            const int64_t e = (v < nx ? xbase : ybase) + v;
+            ad += d2[e];
+            ae += gd[e];
+            ++seen;
           }
-        }
-#pragma unroll
-        for (int r = 0; r < kScanUnroll; ++r) {
-          const bool act = match(k[r]);
-          hist_add(act, act ? (int)((k[r] >> shift) & 255u) : -1, act ? a[r] : 0.0,
-                   act ? b[r] : 0.0, act ? c[r] : 0.0, hist, cnt, stage, warp, lane);
-        }
-      }
-    } else {
-      const int64_t nl = wcnt[warp];
-      for (int64_t base = 0; base < nl; base += kWarp) {
-        const int64_t i = base + lane;
-        uint64_t k = kNoKey;
-        int32_t e = 0;
-        if (i < nl) {
-          e = list[i];
-          k = keys[e];
-        }
-        const bool act = match(k);
-        hist_add(act, act ? (int)((k >> shift) & 255u) : -1, act ? d2[e] : 0.0,
-                 act ? g2[e] : 0.0, act ? gd[e] : 0.0, hist, cnt, stage, warp, lane);
-      }
-    }
-    __syncthreads();
-    const int b = tid;
-    {
-      double c = 0.0, sd = 0.0, sg = 0.0, se = 0.0;
-      for (int w = 0; w < kSearchWarps; ++w) {
-        c += (double)cnt[w][b];
-        sd += hist[w][b][0];
-        sg += hist[w][b][1];
-        se += hist[w][b][2];
-      }
-      if (CS > 1) {
-        double(*mine)[kBuckets] = lb[pass & 1];
-        mine[0][b] = c;
-        mine[1][b] = sd;
-        mine[2][b] = sg;
-        mine[3][b] = se;
-        // lb is double-buffered by pass parity: a block rewrites this buffer two
-        // passes later, after the next cluster barrier, which every reader of
-        // this pass has reached
-        cluster.sync();
-        c = sd = sg = se = 0.0;
-        for (int r = 0; r < CS; ++r) {  // blocks in rank order: the same sums in every block
-          const double *rem = cluster.map_shared_rank(&lb[pass & 1][0][0], r);
-          c += rem[b];
-          sd += rem[kBuckets + b];
-          sg += rem[2 * kBuckets + b];
-          se += rem[3 * kBuckets + b];
-        }
-      }
-      bc[b] = c;
-      bsd[b] = sd;
-      bsg[b] = sg;
-      bse[b] = se;
-      if (b == 0) kstar = -1;
-    }
-    __syncthreads();
-    const double pd = scan256(bsd[b], wt[0]);
-    const double pe = scan256(bse[b], wt[1]);
-    const double pg = scan256(bsg[kBuckets - 1 - b], wt[2]);  // reversed: suffix sums
-    __syncthreads();
-    {
-      double od = 0.0, oe = 0.0, og = 0.0;
-      for (int w = 0; w < (b >> 5); ++w) {
-        od += wt[0][w];
-        oe += wt[1][w];
-        og += wt[2][w];
-      }
-      cum_d[b + 1] = od + pd;
-      cum_e[b + 1] = oe + pe;
-      tail_g[kBuckets - 1 - b] = og + pg;
-      if (b == 0) {
-        cum_d[0] = 0.0;
-        cum_e[0] = 0.0;
-        tail_g[kBuckets] = 0.0;
-      }
-    }
-    __syncthreads();
-    {
-      const uint64_t edge_bits = pre | ((uint64_t)b << shift);
-      const double edge = __longlong_as_double((long long)edge_bits);
-      bool ok = false;
-      if ((edge_bits >> 63) == 0ull && isfinite(edge)) {  // nonnegative finite edges only
-        const double f = L.f_lo + cum_d[b] + edge * edge * (L.f_hi + tail_g[b]);
-        ok = f <= L.r2;
-      }
-      if (ok) atomicMax(&kstar, b);
-    }
-    __syncthreads();
-    if (tid == 0) {
-      if (kstar < 0) {
-        // f > r^2 at the bracket's lower end (only possible in the first pass,
-        // at the common prefix): lambda* lies below every breakpoint
-        L.f_hi += tail_g[0];
-        L.lambda = sqrt(fmax(L.r2 - L.f_lo, 0.0) / L.f_hi);
-        L.rho_r = L.e_lo + L.lambda * L.f_hi;
-        L.done = 1;
-      } else {
-        const int k = kstar;
-        L.f_lo += cum_d[k];
-        L.e_lo += cum_e[k];
-        L.f_hi += tail_g[k + 1];
-        L.prefix = pre | ((uint64_t)k << shift);
-        if (bc[k] == 0.0 || shift == 0) {
-          if (bc[k] != 0.0) {  // last pass: breakpoints equal to the edge are clamped
-            L.f_lo += bsd[k];
-            L.e_lo += bse[k];
-          }
-          if (L.f_hi > 0.0) {
-            L.lambda = sqrt(fmax(L.r2 - L.f_lo, 0.0) / L.f_hi);
-            L.rho_r = L.e_lo + L.lambda * L.f_hi;
-          } else {
-            L.lambda = INFINITY;
-            L.rho_r = L.e_lo;
-          }
-          L.done = 1;
+        } else if (k[r] != kNoKey) {
+          above += g[r];
         }
       }
     }
+    last = to;
+    double u[4] = {ad, ae, above, 0.0};
+    const double su = warp_sum_multi<4>(u);
+    const int cnt = __reduce_add_sync(kFull, seen);
+    if ((lane & 7) == 0) red[warp][lane >> 3] = lane == 24 ? (double)cnt : su;
+    __syncthreads();
+    if (tid < 4) {
+      double s = 0.0;
+      for (int w = 0; w < kSearchWarps; ++w) s += red[w][tid];
+      (CS > 1 ? part[step & 1] : tot)[tid] = s;
+    }
+    if (CS > 1) {
+      // part is double-buffered: a block rewrites this half two steps later, after
+      // the next cluster barrier, which every reader of this step has reached
+      cluster.sync();
+      if (tid < 4) {
+        double s = 0.0;
+        for (int r = 0; r < CS; ++r) s += cluster.map_shared_rank(&part[step & 1][0], r)[tid];
+        tot[tid] = s;
+      }
+    }
+    __syncthreads();
+    if (tid == 0)
+      L.done = newton_next(tot[0], tot[1], tot[2] + L.f_hi, (int)tot[3], L.r2, step, L.lambda,
+                           L.rho_r, count);
     __syncthreads();
     if (L.done) break;  // the same decision in every block of the cluster
-    if (pass == 0) {
-      // gather the chosen bucket's elements (keys matching the new prefix
-      // down to bit shift) into this warp's list, in scan order
-      const uint64_t np = L.prefix;
-      int64_t n_out = 0;
-      for (int64_t base = (int64_t)gw * kWarp; base < N; base += kScanUnroll * kRound) {
-        uint64_t k[kScanUnroll];
-        int64_t e[kScanUnroll];
-#pragma unroll
-        for (int r = 0; r < kScanUnroll; ++r) {
-          const int64_t v = base + r * kRound + lane;
-          k[r] = kNoKey;
-          e[r] = 0;
-          if (v < N) {
-            e[r] = elem(v);
-            k[r] = keys[e[r]];
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < kScanUnroll; ++r) {
-          const bool keep = k[r] != kNoKey && (k[r] >> shift) == (np >> shift);
-          const unsigned bal = __ballot_sync(kFull, keep);
-          if (keep) list[n_out + __popc(bal & ((1u << lane) - 1u))] = (int32_t)e[r];
-          n_out += __popc(bal);
-        }
-      }
-      if (lane == 0) wcnt[warp] = n_out;
-      __syncthreads();
-    }
   }
   if (tid == 0 && rank == 0) B.ls[sidx] = L;
   if (CS > 1) cluster.sync();  // no block leaves while another may read its memory
@@ -1357,14 +1112,13 @@ struct lp_batch {
         A, v.xbar, v.x, re, I, sinst_a, chunk_a, nchunk_a, G, spart, pstride, nchunk_at);
     b_finalize_kernel<<<count, kBlock, 0, s>>>(I, G, spart, pstride, nchunk_at);
     if (nsearch > 0 && n_small > 0)
-      b_search_kernel<1><<<dim3(n_small, nsearch), kSearchThreads, kSearchSmem, s>>>(
+      b_search_kernel<1><<<dim3(n_small, nsearch), kSearchThreads, 0, s>>>(
           I, plist_small, n, sa);
     if (nsearch > 0 && n_big > 0) {
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute attr[1];
       cfg.gridDim = dim3((unsigned)(n_big * kMaxCluster), (unsigned)nsearch);
       cfg.blockDim = dim3(kSearchThreads);
-      cfg.dynamicSmemBytes = kSearchSmem;
       cfg.stream = s;
       attr[0].id = cudaLaunchAttributeClusterDimension;
       attr[0].val.clusterDim.x = kMaxCluster;
@@ -1921,20 +1675,13 @@ lp_status lp_batch_create(int32_t count, const int32_t *host_row_start,
       h->sa.d2[1] = h->sa.d2[0];
       h->sa.g2[1] = h->sa.g2[0];
       h->sa.gd[1] = h->sa.gd[0];
-      h->sa.cand[1] = h->sa.cand[0];
       break;
     }
-    if ((e = h->alloc(&h->sa.cand[k], N + (int64_t)kMaxCluster * kSearchThreads * count)) != LP_OK)
-      return e;
     if ((e = h->alloc(&h->sa.keys[k], N)) != LP_OK) return e;
     if ((e = h->alloc(&h->sa.d2[k], N)) != LP_OK) return e;
     if ((e = h->alloc(&h->sa.g2[k], N)) != LP_OK) return e;
     if ((e = h->alloc(&h->sa.gd[k], N)) != LP_OK) return e;
   }
-  LP_CU(cudaFuncSetAttribute(b_search_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kSearchSmem));
-  LP_CU(cudaFuncSetAttribute(b_search_kernel<kMaxCluster>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSearchSmem));
   {
     // problems with many elements search with a cluster of kMaxCluster blocks,
     // if the device can hold such a cluster (else every problem uses one block)
@@ -1942,7 +1689,6 @@ lp_status lp_batch_create(int32_t count, const int32_t *host_row_start,
     cudaLaunchAttribute attr[1];
     cfg.gridDim = dim3(kMaxCluster);
     cfg.blockDim = dim3(kSearchThreads);
-    cfg.dynamicSmemBytes = kSearchSmem;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = kMaxCluster;
     attr[0].val.clusterDim.y = 1;

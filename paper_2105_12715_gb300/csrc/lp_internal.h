@@ -14,6 +14,7 @@ constexpr int kWarpsPerBlock = kBlock / kWarp;
 constexpr int kBuckets = 256;         // buckets per pass of the multiplier search
 constexpr int kSearchPasses = 8;      // 8 x 8 bits cover a 64-bit key
 constexpr int kHistWarps = 4;         // warps per block of the histogram kernel
+constexpr int kNewtonMax = 1024;      // Newton steps of a search (each clamps at least one more)
 constexpr uint64_t kNoKey = ~0ull;    // element that takes no part in the search
 constexpr int32_t kRunning = -1;      // DevState::status while iterating
 
@@ -121,7 +122,7 @@ struct DevState {
   unsigned int sel_counter[2];
   int32_t mixed;        // 1: mixed-precision iterations (MixVecs)
   double mix_s;         // scale of the current correction
-  unsigned int bar_gen;  // resident kernel: grid barriers passed since the counters were zero
+  unsigned int bar_gen;  // resident and search kernels: grid barriers passed since the counters were zero
 };
 
 // Device arrays of one problem, permuted order.
@@ -182,6 +183,11 @@ struct CheckScratch {
   // the bracket after the first pass) and a count; null: every pass scans all elements
   int32_t *cand[2], *ccnt[2];
   int64_t cand_cap;
+  // multiplier search in one cooperative launch of search_blocks blocks (0: the radix
+  // kernels): the barrier's counters and [2][search_blocks][8] sums
+  int32_t search_blocks;
+  unsigned int *bar;
+  double *npart;
 };
 
 // Per-problem state of a batch (device, one per problem).
@@ -326,15 +332,21 @@ void lay_vectors(const int32_t *perm_x, int32_t n, const double *c, const double
                  long long *uk, const int32_t *perm_y, int32_t m, const double *b,
                  const int8_t *rt, double *pb, int8_t *prt, int nsm, cudaStream_t s);
 
+// ---- multiplier search in one launch (lp_resident.cu) ----
+constexpr int kSearchBlockElems = 4096;  // coordinates per block at least
+bool search_fits(int P, int nsm);
+cudaError_t launch_search(const CheckScratch &cs, int64_t N, int nsearch, DevState *st,
+                          cudaStream_t s);
+
 // ---- launchers (lp_kernels.cu) ----
 void launch_primal_step(const SellMat &AT, const DevVecs &v, DevState *st,
                         const double *w, int k, int unroll, int grid_cap, cudaStream_t s);
 void launch_dual_step(const SellMat &A, const DevVecs &v, DevState *st,
                       const double *w, int k, int unroll, int grid_cap, cudaStream_t s);
-void launch_check(const SellMat &A, const SellMat &AT, const DevVecs &v,
-                  DevState *st, double *w, const CheckScratch &cs, int n,
-                  int m, int nsearch, double *trace, bool decide,
-                  cudaStream_t s, const MixVecs *mv = nullptr);
+cudaError_t launch_check(const SellMat &A, const SellMat &AT, const DevVecs &v,
+                         DevState *st, double *w, const CheckScratch &cs, int n,
+                         int m, int nsearch, double *trace, bool decide,
+                         cudaStream_t s, const MixVecs *mv = nullptr);
 void launch_advance(DevState *st, double *w, int r, cudaStream_t s);
 void launch_spmv(const SellMat &A, const double *v, double *out, cudaStream_t s,
                  DevState *st_guard);

@@ -1125,9 +1125,10 @@ void launch_dual_step(const SellMat &A, const DevVecs &v, DevState *st, const do
   }
 }
 
-void launch_check(const SellMat &A, const SellMat &AT, const DevVecs &v, DevState *st, double *w,
-                  const CheckScratch &cs, int n, int m, int nsearch, double *trace,
-                  bool decide, cudaStream_t s, const MixVecs *mv) {
+cudaError_t launch_check(const SellMat &A, const SellMat &AT, const DevVecs &v, DevState *st,
+                         double *w, const CheckScratch &cs, int n, int m, int nsearch,
+                         double *trace, bool decide, cudaStream_t s, const MixVecs *mv) {
+  cudaError_t launched = cudaSuccess;
   if (mv) launch_combine(v, *mv, st, n, m, 0, s);
   CheckColsEpi ce{};
   if (mv) {
@@ -1191,8 +1192,10 @@ void launch_check(const SellMat &A, const SellMat &AT, const DevVecs &v, DevStat
   else
     check_kernel<CheckRowsEpi, false><<<gr, kBlock, 0, s>>>(A, r0, r1, re, st, P, ps, gc);
   check_finalize_kernel<<<NQ, kBlock, 0, s>>>(st, cs.partials, cs.pstride, nparts);
-  if (nsearch > 0) {
-    const int64_t N = (int64_t)n + m;
+  const int64_t N = (int64_t)n + m;
+  if (nsearch > 0 && cs.search_blocks > 0) {
+    launched = launch_search(cs, N, nsearch, st, s);
+  } else if (nsearch > 0) {
     for (int p = 0; p < kSearchPasses; ++p) {
       ls_hist_kernel<<<dim3(cs.hist_grid, nsearch), kHistWarps * kWarp, 0, s>>>(
           cs.keys[0], cs.d2[0], cs.g2[0], cs.gd[0], cs.keys[1], cs.d2[1], cs.g2[1], cs.gd[1], N,
@@ -1206,6 +1209,7 @@ void launch_check(const SellMat &A, const SellMat &AT, const DevVecs &v, DevStat
     restart_copy_kernel<<<grid_for((int64_t)n + m, num_sms()), kBlock, 0, s>>>(v, st, n, m);
     if (mv) launch_recenter(v, *mv, st, n, m, 0, s);
   }
+  return launched;
 }
 
 template <int U, bool PIPE>

@@ -57,7 +57,6 @@ namespace {
 constexpr int kGridThreads = 512;      // threads per block of the grid kernel
 constexpr int kClusterThreads = 256;   // and of the cluster kernel
 constexpr int kU = 8;                  // gathers in flight per lane
-constexpr int kNewtonMax = 1024;       // Newton steps (each clamps at least one more coordinate)
 constexpr int kStatusIterLimit = 4;
 constexpr int kStatusTimeout = 6;
 constexpr int kBarLines = kResBarLines;  // arrival counters of the grid barrier
@@ -332,27 +331,6 @@ __device__ __forceinline__ void check_sums(const LSlice *sl, int count, const in
       o1[s.slot0 + r] = a1;
     }
   }
-}
-
-// Sums of N per-thread values over the warp (N a power of two <= 32): the
-// transposed butterfly issues N - 1 + log2(32 / N) additions instead of 5 N.
-// Lane l returns the sum of value l / (32 / N).
-template <int N>
-__device__ __forceinline__ double warp_sum_multi(double (&v)[N]) {
-  const int lane = threadIdx.x & (kWarp - 1);
-  int o = 16;
-#pragma unroll
-  for (int half = N / 2; half > 0; half >>= 1, o >>= 1) {
-    const bool hi = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < half; ++i) {
-      const double keep = hi ? v[i + half] : v[i], send = hi ? v[i] : v[i + half];
-      v[i] = keep + __shfl_xor_sync(kFull, send, o);
-    }
-  }
-  double s = v[0];
-  for (; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-  return s;
 }
 
 // Sum over the P blocks of quantity q's partials, by one warp, fixed order.
@@ -1133,17 +1111,8 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
       const double A = S.nw[4 * c], E = S.nw[4 * c + 1];
       const double B = S.nw[4 * c + 2] + tot[c ? Q_G2INF_C : Q_G2INF_A];
       const int same = (int)S.nw[4 * c + 3];
-      if (!(B > 0.0)) {
-        S.h->rho_r[c] = E;
-        S.h->done[c] = 1;
-      } else {
-        const double ln = sqrt(fmax(S.h->r2[c] - A, 0.0) / B);
-        S.h->rho_r[c] = E + ln * B;
-        // the clamped set repeats (or rounding stops the increase): exact
-        if (same == S.h->count[c] || (step > 0 && !(ln > S.h->lam[c]))) S.h->done[c] = 1;
-        S.h->count[c] = same;
-        S.h->lam[c] = ln;
-      }
+      S.h->done[c] = newton_next(A, E, B, same, S.h->r2[c], step, S.h->lam[c], S.h->rho_r[c],
+                                 S.h->count[c]);
     }
     __syncthreads();
   }
@@ -1558,6 +1527,119 @@ ClusterKernel cluster_of(bool mixed, bool res, bool batch) {
   return k[(mixed ? 4 : 0) + (res ? 2 : 0) + (batch ? 1 : 0)];
 }
 
+// The multiplier search of the per-pass check in one cooperative launch: Newton
+// steps (newton_next) over N breakpoints, one grid barrier each.  lambda only
+// rises, so a coordinate once clamped stays clamped: its d^2 and d g go into the
+// thread's running sums at the step that clamps it, and a step reads the keys
+// and g^2 (16 bytes per coordinate, from L2) and adds the g^2 of the others,
+// one FP64 addition per coordinate.
+constexpr int kNewtonThreads = 1024;
+struct SearchArgs {
+  CheckScratch cs;
+  DevState *st;
+  int64_t N;
+  int32_t nsearch;
+};
+
+__global__ void __launch_bounds__(kNewtonThreads, 1) search_kernel(SearchArgs a) {
+  constexpr int W = kNewtonThreads / kWarp, U = 4;
+  __shared__ LSearch L[2];
+  __shared__ double red[W][8], nw[8];
+  __shared__ int32_t dead;
+  const int tid = threadIdx.x, lane = tid & (kWarp - 1), warp = tid >> 5;
+  const int P = (int)gridDim.x;
+  if (a.st->status != kRunning) return;  // nothing here changes it but a wait that runs out
+  GridLink<double> link{a.cs.bar, a.st->bar_gen, &dead, nullptr, nullptr};
+  if (tid < 2) {
+    L[tid] = a.st->ls[tid];
+    if (tid >= a.nsearch) L[tid].done = 1;
+  }
+  if (tid == 0) dead = 0;
+  __syncthreads();
+  const unsigned gen0 = link.gen;
+  double clamped[2][2] = {{0.0, 0.0}, {0.0, 0.0}};  // this thread's sums of d^2, d g
+  uint64_t last[2] = {0ull, 0ull};                  // keys below are in them
+  int seen[2] = {0, 0};                             // and their number
+  int count[2] = {-1, -1};                          // thread 0's
+  for (int step = 0; step < kNewtonMax; ++step) {
+    const bool done0 = L[0].done != 0, done1 = L[1].done != 0;
+    if (done0 && done1) break;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      if (c ? done1 : done0) continue;
+      const uint64_t *__restrict__ keys = a.cs.keys[c];
+      const double *__restrict__ d2 = a.cs.d2[c], *__restrict__ gd = a.cs.gd[c];
+      const double *__restrict__ g2 = a.cs.g2[c];
+      const uint64_t to = (uint64_t)dbits(L[c].lambda) + 1;  // clamped: keys below to
+      double above = 0.0;
+      const int64_t stride = (int64_t)P * kNewtonThreads;
+      for (int64_t e0 = (int64_t)blockIdx.x * kNewtonThreads + tid; e0 < a.N; e0 += U * stride) {
+        uint64_t k[U];
+        double g[U];
+#pragma unroll
+        for (int r = 0; r < U; ++r) {
+          const int64_t e = e0 + r * stride;
+          k[r] = e < a.N ? keys[e] : kNoKey;
+          g[r] = e < a.N ? g2[e] : 0.0;
+        }
+#pragma unroll
+        for (int r = 0; r < U; ++r) {
+          if (k[r] < to) {
+            if (k[r] >= last[c]) {
+              const int64_t e = e0 + r * stride;
+              clamped[c][0] += d2[e];
+              clamped[c][1] += gd[e];
+              ++seen[c];
+            }
+          } else if (k[r] != kNoKey) {
+            above += g[r];
+          }
+        }
+      }
+      last[c] = to;
+      double u[4] = {clamped[c][0], clamped[c][1], above, 0.0};
+      const double su = warp_sum_multi<4>(u);
+      const int cnt = __reduce_add_sync(kFull, seen[c]);
+      if ((lane & 7) == 0) red[warp][4 * c + (lane >> 3)] = lane == 24 ? (double)cnt : su;
+    }
+    __syncthreads();
+    // two buffers in turn: a block may still read the last step's sums
+    double *np = a.cs.npart + (size_t)(step & 1) * P * 8;
+    if (tid < 8 && !(tid < 4 ? done0 : done1)) {
+      double s = 0.0;
+      for (int i = 0; i < W; ++i) s += red[i][tid];
+      __stcg(np + (size_t)blockIdx.x * 8 + tid, s);
+    }
+    if (!link.sync()) {
+      if (tid == 0) a.st->status = kStatusTimeout;
+      return;
+    }
+    if (warp < 8 && !(warp < 4 ? done0 : done1)) {
+      const double s = sum_parts(np, 8, warp, P);
+      if (lane == 0) nw[warp] = s;
+    }
+    __syncthreads();
+    if (tid == 0) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        LSearch &l = L[c];
+        if (!l.done)
+          l.done = newton_next(nw[4 * c], nw[4 * c + 1], nw[4 * c + 2] + l.f_hi,
+                               (int)nw[4 * c + 3], l.r2, step, l.lambda, l.rho_r, count[c]);
+      }
+    }
+    __syncthreads();
+  }
+  // every block has read the state: each passed a barrier after that
+  if (blockIdx.x == 0 && link.gen != gen0 && tid < 2) {
+    if (tid < a.nsearch) {
+      L[tid].done = 1;
+      a.st->ls[tid] = L[tid];
+    }
+    if (tid == 0) a.st->bar_gen = link.gen;
+  }
+}
+
 }  // namespace
 
 // Bytes of shared memory of a block that owns nc + nr slices with ncl columns and nrl rows and
@@ -1612,6 +1694,30 @@ bool resident_fits(int P, int nsm, size_t smem, bool mixed) {
     return false;
   }
   return (int64_t)per_sm * nsm >= P;
+}
+
+bool search_fits(int P, int nsm) {
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, search_kernel, kNewtonThreads, 0) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (int64_t)per_sm * nsm >= P;
+}
+
+cudaError_t launch_search(const CheckScratch &cs, int64_t N, int nsearch, DevState *st,
+                          cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)cs.search_blocks);
+  cfg.blockDim = dim3(kNewtonThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, search_kernel, SearchArgs{cs, st, N, nsearch});
 }
 
 cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixed,

@@ -721,6 +721,50 @@ __device__ __forceinline__ void kkt_from(const double *t, int qp, int qd, int qp
   out[0] = rp; out[1] = rd; out[2] = p; out[3] = d; out[4] = rel;
 }
 
+// Sums of N per-thread values over the warp (N a power of two <= 32): the
+// transposed butterfly issues N - 1 + log2(32 / N) additions instead of 5 N.
+// Lane l returns the sum of value l / (32 / N).
+template <int N>
+__device__ __forceinline__ double warp_sum_multi(double (&v)[N]) {
+  const int lane = threadIdx.x & (kWarp - 1);
+  int o = 16;
+#pragma unroll
+  for (int half = N / 2; half > 0; half >>= 1, o >>= 1) {
+    const bool hi = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const double keep = hi ? v[i + half] : v[i], send = hi ? v[i] : v[i + half];
+      v[i] = keep + __shfl_xor_sync(kFull, send, o);
+    }
+  }
+  double s = v[0];
+  for (; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+  return s;
+}
+
+// One step of Newton's method for the multiplier lambda* of Section 6.3, in
+// mu = lambda^2: f(mu) = sum_{clamped} d^2 + mu sum_{others} g^2 is piecewise
+// linear, nondecreasing and concave, so from lambda = 0 the iterates rise to
+// f = r^2 without passing it, and the step from the clamped set that repeats
+// is exact.  A, E, B: sums of d^2 and d g over the coordinates whose
+// breakpoint is at most lam, of g^2 over the others; same: how many are
+// clamped.  Returns 1 when lam and rho_r hold the result.
+__device__ __forceinline__ int newton_next(double A, double E, double B, int same, double r2,
+                                           int step, double &lam, double &rho_r, int &count) {
+  if (!(B > 0.0)) {  // every coordinate clamped
+    lam = INFINITY;
+    rho_r = E;
+    return 1;
+  }
+  const double ln = sqrt(fmax(r2 - A, 0.0) / B);
+  rho_r = E + ln * B;
+  // the clamped set repeats, or rounding stops the increase
+  const int done = same == count || (step > 0 && !(ln > lam)) ? 1 : 0;
+  count = same;
+  lam = ln;
+  return done;
+}
+
 // Fixed-order inclusive scan of 256 values held one per thread of the
 // first 256 threads (8 warps): shuffle scan inside each warp, then the warp
 // totals.  Returns the inclusive prefix for thread b.

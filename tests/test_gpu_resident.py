@@ -199,3 +199,33 @@ def test_batch_adjoint_is_the_per_pass_adjoint(lpm):
                     np.testing.assert_array_equal(after[k], before[k], err_msg=k)
         for a, b in zip(*out):
             np.testing.assert_allclose(a, b, rtol=0, atol=1e-12 * max(1.0, np.abs(b).max()))
+
+
+@pytest.mark.parametrize("name", ["1x1", "no_rows", "empty_lines", "997x4999", "20000x90001"])
+@pytest.mark.parametrize("scheme,precision", [("ADAPTIVE", 0), ("FLEXIBLE", 0), ("ADAPTIVE", 1)])
+def test_search_by_newton_steps_in_the_per_pass_check(lpm, name, scheme, precision):
+    """K = 1025 exceeds the resident kernels: one search launch against the radix
+    passes.  Both sum n + m positive terms and take one square root."""
+    data = CASES[name]()
+    opts = dict(check_every=1025, max_iter=2050, precision=precision,
+                restart_scheme=getattr(lpm, "LP_RESTART_" + scheme))
+    _, a, t1, i1 = run(lpm, data, 1, **opts)
+    _, b, t0, i0 = run(lpm, data, 0, **opts)
+    assert i1.graph_kernels == i0.graph_kernels - 15
+    for k in a:
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    np.testing.assert_allclose(t1, t0, rtol=1e-9, atol=1e-11)
+
+
+@pytest.mark.parametrize("scheme", ["ADAPTIVE", "FLEXIBLE"])
+def test_batch_search_at_the_edges_of_its_cluster(lpm, scheme):
+    """n + m = 2047 (one block), 2048 and more (a cluster), against single solves."""
+    sizes = [(1, 1), (447, 1600), (448, 1600), (449, 1600), (3000, 9001), (255, 1)]
+    probs = [lpgen.tiny_standard_form(k, m=m, n=n, per_col=min(m, 4))
+             for k, (m, n) in enumerate(sizes)]
+    opts = dict(check_every=16, max_iter=16, restart_scheme=getattr(lpm, "LP_RESTART_" + scheme))
+    _, _, infos = batch_run(lpm, probs, 0, **opts)
+    for p, u in zip(probs, infos):
+        _, _, _, i = run(lpm, p, 0, **opts)
+        # the iterates of 16 steps agree to rounding, so do the gaps
+        np.testing.assert_allclose(u["last_rho"], i.last_rho, rtol=1e-9, atol=1e-11)
