@@ -519,12 +519,8 @@ lp_status host_layout(lp_problem *h, const int32_t *row_ptr, const int32_t *col_
   HostSell HA, HAT;
   const LanePolicy policy{opt.long_row_threshold, opt.lane_steps, opt.single_lane_max};
   const int64_t target = (int64_t)opt.lane_auto * h->nsm;
-  const LanePolicy pa = choose_lanes(policy, target, h->mixed, [&](const LanePolicy &p) {
-    return layout_work(rp, perm_y, p);
-  });
-  const LanePolicy pat = choose_lanes(policy, target, h->mixed, [&](const LanePolicy &p) {
-    return layout_work(cp, perm_x, p);
-  });
+  const LanePolicy pa = choose_lanes(policy, target, h->mixed, length_runs(rp, perm_y));
+  const LanePolicy pat = choose_lanes(policy, target, h->mixed, length_runs(cp, perm_x));
   const int32_t split_len = opt.split_row_len;
   build_sell(m, n, rp, hci, hv, perm_y, inv_x, pa, HA, {}, split_len);
   build_sell(n, m, cp, ri.data(), cv.data(), perm_x, inv_y, pat, HAT, {}, split_len);
@@ -769,30 +765,11 @@ lp_status device_layout(lp_problem *h, const int32_t *row_ptr, const int32_t *co
     if (warp_rows) *warp_rows = wr;
     return true;
   };
-  // the same work as layout_work's: of a run's rows, longest first, every
-  // (32 >> lg)-th opens a slice
-  auto hist_work = [](const std::vector<int64_t> &hist, const LanePolicy &p) {
-    LayoutWork w;
-    int run_lg = -1;
-    int64_t pos = 0;  // rows of the current run before this length
-    for (int64_t len = (int64_t)hist.size() - 1; len >= 0; --len) {
-      const int64_t rows = hist[(size_t)len];
-      if (rows == 0) continue;
-      const int lg = lanes_log2(len, p);
-      if (lg != run_lg) {
-        run_lg = lg;
-        pos = 0;
-      }
-      const int64_t cap = kWarp >> lg;
-      const int64_t opened = (pos + rows + cap - 1) / cap - (pos + cap - 1) / cap;
-      if (opened > 0) w.add(len, lg, p, opened);
-      pos += rows;
-    }
-    return w;
-  };
   auto choose = [&](const std::vector<int64_t> &hist, const LanePolicy &p) {
-    return choose_lanes(p, (int64_t)opt.lane_auto * nsm, h->mixed,
-                        [&](const LanePolicy &q) { return hist_work(hist, q); });
+    std::vector<LengthRun> runs;
+    for (int64_t len = (int64_t)hist.size() - 1; len >= 0; --len)
+      if (hist[(size_t)len] > 0) runs.push_back({len, hist[(size_t)len], runs.empty()});
+    return choose_lanes(p, (int64_t)opt.lane_auto * nsm, h->mixed, runs);
   };
   const LanePolicy policy{opt.long_row_threshold, opt.lane_steps, opt.single_lane_max};
   const int32_t split_len = opt.split_row_len;

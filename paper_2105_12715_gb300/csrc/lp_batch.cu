@@ -1535,12 +1535,8 @@ lp_status lp_batch_create(int32_t count, const int32_t *host_row_start,
   const LanePolicy policy{opt.long_row_threshold, opt.lane_steps, opt.single_lane_max};
   const int64_t target = (int64_t)opt.lane_auto * h->nsm;
   const bool fp32 = opt.precision == LP_PRECISION_MIXED;
-  const LanePolicy pa = choose_lanes(policy, target, fp32, [&](const LanePolicy &p) {
-    return layout_work(rp, perm_y, p, brk_rows);
-  });
-  const LanePolicy pat = choose_lanes(policy, target, fp32, [&](const LanePolicy &p) {
-    return layout_work(cp, perm_x, p, brk_cols);
-  });
+  const LanePolicy pa = choose_lanes(policy, target, fp32, length_runs(rp, perm_y, brk_rows));
+  const LanePolicy pat = choose_lanes(policy, target, fp32, length_runs(cp, perm_x, brk_cols));
   build_sell(m, n, rp, hci, hv, perm_y, inv_x, pa, HA, brk_rows);
   build_sell(n, m, cp, ri.data(), cv.data(), perm_x, inv_y, pat, HAT, brk_cols);
 

@@ -233,23 +233,47 @@ struct LayoutWork {
   }
 };
 
-// The layout's work for rows perm[0..) (longest first within each segment
-// between breaks).
-inline LayoutWork layout_work(const std::vector<int64_t> &ptr, const std::vector<int32_t> &perm,
-                              const LanePolicy &p, const std::vector<int32_t> &breaks = {}) {
+// Rows of one length that follow one another in the layout's order; opens: the
+// first of a segment (a slice must start there).
+struct LengthRun {
+  int64_t len, rows;
+  bool opens;
+};
+
+// Runs of the rows perm[0..) (longest first within each segment between breaks).
+inline std::vector<LengthRun> length_runs(const std::vector<int64_t> &ptr,
+                                          const std::vector<int32_t> &perm,
+                                          const std::vector<int32_t> &breaks = {}) {
+  std::vector<LengthRun> runs;
   const int32_t nrows = (int32_t)perm.size();
-  LayoutWork w;
-  int32_t r = 0;
   size_t bi = 0;
-  while (r < nrows) {
-    const int32_t lim = slice_limit(breaks, &bi, r, nrows);
+  int32_t lim = 0;
+  for (int32_t r = 0; r < nrows; ++r) {
     const int64_t len = ptr[perm[r] + 1] - ptr[perm[r]];
-    const int lg = lanes_log2(len, p);
-    const int cap = kWarp >> lg;
-    int32_t q = r;
-    while (q < lim && q - r < cap && lanes_log2(ptr[perm[q] + 1] - ptr[perm[q]], p) == lg) ++q;
-    w.add(len, lg, p, 1);
-    r = q;
+    const bool opens = r == lim;
+    if (opens) lim = slice_limit(breaks, &bi, r, nrows);
+    if (opens || runs.back().len != len) runs.push_back({len, 0, opens});
+    ++runs.back().rows;
+  }
+  return runs;
+}
+
+// The layout's work: of rows with equally many lanes, every (32 >> lg)-th opens
+// a slice.
+inline LayoutWork layout_work(const std::vector<LengthRun> &runs, const LanePolicy &p) {
+  LayoutWork w;
+  int cur = -1;
+  int64_t pos = 0;  // rows with this many lanes so far
+  for (const LengthRun &r : runs) {
+    const int lg = lanes_log2(r.len, p);
+    if (lg != cur || r.opens) {
+      cur = lg;
+      pos = 0;
+    }
+    const int64_t cap = kWarp >> lg;
+    const int64_t opened = (pos + r.rows + cap - 1) / cap - (pos + cap - 1) / cap;
+    if (opened > 0) w.add(r.len, lg, p, opened);
+    pos += r.rows;
   }
   return w;
 }
@@ -265,10 +289,11 @@ inline LayoutWork layout_work(const std::vector<int64_t> &ptr, const std::vector
 // among single_max halved up to three times and lane_steps halved up to once, not
 // below 8, is taken (100k x 500k, rows of 50: 23.5 us per row pass with one lane
 // per row, 38.2 with the 8 lanes that `target` asks for; 40k rows: 13.8 with 4
-// lanes, 16.5 with 8, 17.3 with 1).  work(p) gives the layout's work under p.
-template <class F>
-inline LanePolicy choose_lanes(LanePolicy p, int64_t target, bool mixed, F work) {
+// lanes, 16.5 with 8, 17.3 with 1).
+inline LanePolicy choose_lanes(LanePolicy p, int64_t target, bool mixed,
+                               const std::vector<LengthRun> &runs) {
   if (target <= 0) return p;
+  auto work = [&](const LanePolicy &q) { return layout_work(runs, q); };
   if (mixed) {
     while (work(p).slices < target && (p.single_max > 1 || p.lane_steps > 1)) {
       p.single_max = p.single_max / 2;
