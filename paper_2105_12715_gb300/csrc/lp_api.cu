@@ -295,6 +295,10 @@ lp_status set_run_params(lp_problem *h, double tol, cudaStream_t s) {
 // cluster, 0.33 on the grid; 2k x 10k: 0.41 and 0.43; 600 x 1400 in mixed
 // precision: 0.72 and 0.35).  Else the grid, with at least four slices per block
 // and pass, so that the barriers and reductions of a small LP span few blocks.
+// The grid's gathers go through L1, so its blocks take at most 195 KB: above,
+// the SM's carve-out goes to its last step and leaves 28 KB of L1 instead of 60
+// (20k rows, FP64, us per iteration, per-pass kernels in brackets: 90k columns,
+// 192 KB, 14.7 [17.6]; 100k, 209 KB, 19.2 [17.3]).
 lp_status plan_resident(lp_problem *h, cudaStream_t s) {
   constexpr int kSlicesPerBlock = 4, kClusterBlocks = 8;
   const int kClusterElems = h->mixed ? 768 : 2048;
@@ -304,7 +308,8 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
     return LP_OK;
   const int64_t elem = h->mixed ? 8 : 12;  // bytes of an index and a value
   const size_t limit = resident_smem_limit(h->device, h->mixed);
-  if (limit == 0 || 2 * h->nnz * elem > (int64_t)limit * h->nsm) return LP_OK;
+  constexpr size_t kKeepL1 = 32 << 10;
+  if (limit <= kKeepL1 || 2 * h->nnz * elem > (int64_t)limit * h->nsm) return LP_OK;
   std::vector<SliceInfo> ic((size_t)h->AT.nslices + 1), ir((size_t)h->A.nslices + 1);
   LP_CU(cudaMemcpyAsync(ic.data(), h->AT.info, sizeof(SliceInfo) * ic.size(),
                         cudaMemcpyDeviceToHost, s));
@@ -347,7 +352,7 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
   if (!cluster) {
     P = std::max(1, std::min(h->nsm, (most + kSlicesPerBlock - 1) / kSlicesPerBlock));
     smem = block_bytes(P, false, false);
-    if (smem > limit || !resident_fits(P, h->nsm, smem, h->mixed)) return LP_OK;
+    if (smem > limit - kKeepL1 || !resident_fits(P, h->nsm, smem, h->mixed)) return LP_OK;
   }
   lp_status e;
   if ((e = h->alloc(&h->res.part, (int64_t)P * kResPart)) != LP_OK) return e;
