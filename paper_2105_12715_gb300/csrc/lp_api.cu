@@ -398,33 +398,45 @@ lp_status plan_search(lp_problem *h) {
 }
 
 // Kernel-variant tuner (lp_options.autotune): on this problem, times every
-// unroll variant of the column pass, then of the row pass (a warm-up and two
-// timed launches per variant, CUDA events on the stream, and a second round for
-// those within 5% of the fastest) and keeps the fastest.  Every variant sums each row in the same order, so the choice
-// changes speed, not results.  The launches advance the iterate: the caller
-// resets the state afterwards.
+// unroll variant of the column pass, then of the row pass (CUDA events on the
+// stream around kReps launches after a warm-up, and a second round in the other
+// order for those within kNear of the fastest) and keeps the fastest.  The host
+// waits once per round, so that the launches follow one another as in a block
+// of iterations: with a wait per variant and two launches the windows of 8 us
+// passes were mostly launch latency, and 80k x 220k in mixed precision ran at
+// 18.8 us per iteration in three creates of five, 17.2 with the right variant.
+// A short pass is launched more often (about 60 us per window, at least three).
+// Every variant sums each row in the same order, so the choice changes speed,
+// not results.  The launches advance the iterate: the caller resets the state
+// afterwards.
 lp_status tune_variants(lp_problem *h, cudaStream_t s) {
-  // (48 to 96 launches took 3.7 ms of a 20 ms lp_create at 100k x 500k)
-  constexpr int kCands = 4, kRounds = 2, kReps = 2;
-  constexpr float kOut = 1.05f;  // slower than this by more: not timed again
+  constexpr int kCands = 4, kRounds = 2;
+  constexpr float kNear = 1.1f;
   const int cands[kCands] = {-2, -4, 2, 4};
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  LP_CU(cudaEventCreate(&e0));
-  LP_CU(cudaEventCreate(&e1));
+  // a pass reads the matrix at a few TB/s and takes some us more
+  const double pass_us = 4.0 + (h->mixed ? 8.0 : 12.0) * (double)h->nnz / 5e6;
+  const int reps = std::max(3, std::min(8, (int)(60.0 / pass_us)));
+  cudaEvent_t ev[2 * kCands] = {};
   lp_status st = LP_OK;
-  // Rounds visit the candidates in rotated order (no candidate always runs
-  // first after the previous pass); each candidate keeps its best time.
+  for (cudaEvent_t &e : ev)
+    if (st == LP_OK) {
+      const cudaError_t err = cudaEventCreate(&e);
+      if (err != cudaSuccess) st = cuda_fail(err, "variant tuning");
+    }
   for (int pass = 0; pass < 2 && st == LP_OK; ++pass) {
     int32_t &u = pass ? h->opt.spmv_unroll_rows : h->opt.spmv_unroll;
     float best[kCands];
     for (float &b : best) b = 1e30f;
     for (int round = 0; round < kRounds && st == LP_OK; ++round) {
+      const float out = round > 0 ? kNear * *std::min_element(best, best + kCands) : 2e30f;
+      bool timed[kCands];
       for (int i = 0; i < kCands; ++i) {
-        const int ci = (i + round) % kCands;
-        if (best[ci] > kOut * *std::min_element(best, best + kCands) && round > 0) continue;
+        const int ci = round > 0 ? kCands - 1 - i : i;
+        timed[ci] = best[ci] <= out;
+        if (!timed[ci]) continue;
         u = cands[ci];
-        for (int r = 0; r <= kReps; ++r) {
-          if (r == 1) cudaEventRecord(e0, s);
+        for (int r = 0; r <= reps; ++r) {
+          if (r == 1) cudaEventRecord(ev[2 * ci], s);
           if (h->mixed) {
             if (pass == 0) launch_primal_mix(h->AT, h->mv, h->st, h->w, 0, u, s);
             else launch_dual_mix(h->A, h->mv, h->v, h->st, h->w, 0, u, s);
@@ -434,24 +446,24 @@ lp_status tune_variants(lp_problem *h, cudaStream_t s) {
             launch_dual_step(h->A, h->v, h->st, h->w, 0, u, h->grid_cap, s);
           }
         }
-        cudaEventRecord(e1, s);
+        cudaEventRecord(ev[2 * ci + 1], s);
+      }
+      cudaError_t err = cudaStreamSynchronize(s);
+      for (int ci = 0; ci < kCands && err == cudaSuccess; ++ci) {
+        if (!timed[ci]) continue;
         float ms = 0.0f;
-        cudaError_t err = cudaEventSynchronize(e1);
-        if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
-        if (err != cudaSuccess) {
-          st = cuda_fail(err, "variant tuning");
-          break;
-        }
+        err = cudaEventElapsedTime(&ms, ev[2 * ci], ev[2 * ci + 1]);
         best[ci] = std::min(best[ci], ms);
       }
+      if (err != cudaSuccess) st = cuda_fail(err, "variant tuning");
     }
     int pick = 0;
     for (int ci = 1; ci < kCands; ++ci)
       if (best[ci] < best[pick]) pick = ci;
     u = cands[pick];
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
+  for (cudaEvent_t e : ev)
+    if (e) cudaEventDestroy(e);
   return st;
 }
 
