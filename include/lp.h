@@ -111,7 +111,8 @@ typedef struct {
                              the SMs' shared memory (without split rows, check_every <= 1024) runs
                              K iterations and the check in one launch; for others every
                              unroll variant of the column and row passes is timed on this problem
-                             and the fastest kept (overrides spmv_unroll and spmv_unroll_rows).
+                             and the fastest kept (overrides spmv_unroll and spmv_unroll_rows),
+                             and the check's multiplier search is one launch instead of 16.
                              Iterates do not depend on the choice: every variant sums each row in
                              the same order.  0: the per-pass kernels with the unrolls given (1) */
   int32_t sigma_method;   /* estimator of sigma_max(A) when eta = 0: LP_SIGMA_LANCZOS (default;
@@ -148,7 +149,8 @@ typedef struct {
   int32_t spmv_unroll, spmv_unroll_rows; /* kernel variants in use (tuned or given) */
   int32_t sigma_steps;  /* steps of the sigma_max estimator (0 when eta was given) */
   int32_t graph_kernels; /* kernel launches per replay of the graph of K iterations + check
-                            (1: the resident kernel runs them all)
+                            (1: the resident kernel runs them all; 2K + 8, with
+                            autotune = 0 2K + 23: the per-pass kernels)
                             (0 until the first lp_solve / lp_iterate builds it) */
   int32_t n_split_slices; /* chunk slices of split rows in A and A^T together (split_row_len) */
 } lp_info;
