@@ -1833,6 +1833,9 @@ lp_status lp_batch_create(int32_t count, const int32_t *host_row_start,
     ResidentArgs &r = h->res;
     if ((e = h->alloc(&r.part, (int64_t)count * r.cluster * kResPart)) != LP_OK) return e;
     if ((e = h->alloc(&r.npart, (int64_t)2 * count * r.cluster * 8)) != LP_OK) return e;
+    r.cs.cols_grid = h->nchunk_at;
+    r.cs.rows_grid = h->nchunk_a;
+    if (h->mixed && (e = h->alloc(&r.rpart, 2 * h->pstride)) != LP_OK) return e;
     r.A = h->A;
     r.AT = h->AT;
     r.v = h->v;

@@ -238,7 +238,8 @@ struct ResidentArgs {
   CheckScratch cs;
   double *part;   // per problem [P][kResPart]
   double *npart;  // per problem [2][P][8]
-  double *rpart;  // mixed precision, single problem: [2][cols_grid + rows_grid] radius sums
+  double *rpart;  // mixed precision: [2][cs.cols_grid + cs.rows_grid] radius sums (batch: one
+                  // entry per check chunk)
   unsigned int *bar;     // [kResBarLines][32] arrival counters of the grid barrier
   int32_t n, m;
   int32_t cluster;       // blocks per problem of the cluster kernel

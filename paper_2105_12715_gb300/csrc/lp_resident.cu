@@ -432,7 +432,10 @@ constexpr size_t row_bytes() {
 // Mixed precision: the radius of a restart scales the next correction (mix_s),
 // whose data are rounded to FP32, so its last bits must not depend on the
 // kernel.  These sums of (z - z0)^2 over the columns and the rows repeat the
-// order of the per-pass kernels' check.
+// order of the per-pass kernels' check.  A block reads rows that others own, so
+// the parts are formed before the check's barrier: behind it the owners may
+// already be writing the restart point (a search that needs no step has no
+// further barrier).
 //
 // Of the owned rows of one slice, lane by lane.
 __device__ __forceinline__ double slice_dist2(const SellMat &A, int slice, const double *z,
@@ -499,30 +502,22 @@ __device__ __forceinline__ double radius_total(const double *part, int n, int lo
   return r;
 }
 
-// A batch's problem (b_check_kernel, b_finalize_kernel): chunks of 8 slices.
+// A batch's problem (b_check_kernel, b_finalize_kernel): one entry of out per
+// chunk of 8 slices, the chunks shared out over the warps of the cluster.
 template <int NT>
-__device__ __forceinline__ double radius_batch(const SellMat &A, int s0, int s1, const double *z,
-                                               const double *z0, double *red) {
+__device__ __forceinline__ void radius_chunks(const Share &sh, const SellMat &A, int s0, int s1,
+                                              const double *z, const double *z0, double *out) {
   constexpr int W = NT / kWarp;
   const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x >> 5;
   const int nch = (s1 - s0 + kCheckChunk - 1) / kCheckChunk;
-  double acc = 0.0;
-  for (int c0 = 0; c0 < nch; c0 += kWarp) {
-    for (int c = c0 + warp; c < min(nch, c0 + kWarp); c += W) {
-      double q = 0.0;
-      const int e = min(s1, s0 + (c + 1) * kCheckChunk);
-      for (int s = s0 + c * kCheckChunk; s < e; ++s) q = slice_dist2(A, s, z, z0, q);
+  for (int c = sh.rank * W + warp; c < nch; c += sh.P * W) {
+    double q = 0.0;
+    const int e = min(s1, s0 + (c + 1) * kCheckChunk);
+    for (int s = s0 + c * kCheckChunk; s < e; ++s) q = slice_dist2(A, s, z, z0, q);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(kFull, q, o);
-      if (lane == 0) red[c - c0] = q;
-    }
-    __syncthreads();
-    if (c0 + lane < nch) acc += red[lane];
-    __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(kFull, q, o);
+    if (lane == 0) __stcg(out + c, q);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
-  return acc;
 }
 
 __device__ __forceinline__ const float *values(const SellMat &A, float) { return A.valf; }
@@ -913,9 +908,19 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
   double *part = a.part + (size_t)P * kResPart * (blockIdx.x / P);
   const int ncand = gap_c ? 2 : gap_a ? 1 : 0;
   const int nrad = a.cs.cols_grid + a.cs.rows_grid;
-  if (MIX && !IO::kBatch)
-    for (int c = 0; c < ncand; ++c)
-      radius_parts<NT>(a, sh, S.red, c, a.rpart + (size_t)c * nrad);
+  if constexpr (MIX) {
+    for (int c = 0; c < ncand; ++c) {
+      double *rp = a.rpart + (size_t)c * nrad;
+      if constexpr (IO::kBatch) {
+        const BInst &B = *io.B;
+        radius_chunks<NT>(sh, a.AT, B.cs0, B.cs1, c ? a.v.x : a.v.xbar, a.v.x0, rp + B.cc0);
+        radius_chunks<NT>(sh, a.A, B.rs0, B.rs1, c ? a.v.y : a.v.ybar, a.v.y0,
+                          rp + a.cs.cols_grid + B.rc0);
+      } else {
+        radius_parts<NT>(a, sh, S.red, c, rp);
+      }
+    }
+  }
   if (warp < busy) {
     CheckColsEpi ce{};
     CheckRowsEpi re{};
@@ -992,12 +997,12 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
   if constexpr (MIX) {
     for (int c = 0; c < ncand; ++c) {
       double rx, ry;
+      const double *rp = a.rpart + (size_t)c * nrad;
       if constexpr (IO::kBatch) {
         const BInst &B = *io.B;
-        rx = radius_batch<NT>(a.AT, B.cs0, B.cs1, c ? a.v.x : a.v.xbar, a.v.x0, S.red);
-        ry = radius_batch<NT>(a.A, B.rs0, B.rs1, c ? a.v.y : a.v.ybar, a.v.y0, S.red);
+        rx = sum_parts(rp + B.cc0, 1, 0, B.cc1 - B.cc0);
+        ry = sum_parts(rp + a.cs.cols_grid + B.rc0, 1, 0, B.rc1 - B.rc0);
       } else {
-        const double *rp = a.rpart + (size_t)c * nrad;
         rx = radius_total(rp, nrad, 0, a.cs.cols_grid, S.red);
         ry = radius_total(rp, nrad, a.cs.cols_grid, nrad, S.red);
       }
