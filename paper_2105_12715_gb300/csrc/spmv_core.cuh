@@ -219,6 +219,7 @@ __device__ __forceinline__ void process_split_item(const SellMat &A, const T *__
     }
   }
   if (!__shfl_sync(kFull, last, 0)) return;
+  __syncwarp();  // orders lane 0's fence before the other lanes' loads (a shuffle does not)
   // The whole warp adds the partials: FP64 lane by lane and a butterfly (one
   // lane adding the 391 partials of a 200,000-element row in a chain took 20 of
   // the pass's 35 us), FP32 in chunk order, 32 loads at a time.
