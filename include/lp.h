@@ -186,7 +186,9 @@ lp_status lp_create(int32_t m, int32_t n, int64_t nnz, const int32_t *row_ptr,
  * the relative KKT error of the running average or of the current iterate
  * is <= tol at a check (every K iterations; the average wins ties), or
  * until opt.max_iter further iterations.  Returns LP_OK, LP_ITER_LIMIT,
- * LP_ERR_NUMERICAL, LP_ERR_INVALID_ARG (tol <= 0) or LP_ERR_CUDA.  Blocks
+ * LP_ERR_NUMERICAL, LP_ERR_INVALID_ARG (tol <= 0), LP_ERR_CUDA or
+ * LP_ERR_TIMEOUT (a bounded wait of a grid barrier ran out, as when the GPU is
+ * taken away for 2 s: the state is undefined until lp_set_state).  Blocks
  * the host until the solve ends (one 4-byte read per check).
  */
 lp_status lp_solve(lp_handle h, double tol, void *cuda_stream);
@@ -196,7 +198,8 @@ lp_status lp_solve(lp_handle h, double tol, void *cuda_stream);
  * (KKT, normalized gap, restart decision), without any host
  * synchronization.  Blocks after convergence (relative KKT <= tol) do no
  * work.  The iteration count is not capped by max_iter.  Returns LP_OK or
- * an error of the enqueue.
+ * an error of the enqueue; lp_info.status tells how the blocks ended
+ * (LP_ERR_TIMEOUT as in lp_solve among them).
  */
 lp_status lp_iterate(lp_handle h, int32_t n_checks, double tol, void *cuda_stream);
 
@@ -277,7 +280,8 @@ lp_status lp_profile_kernel(lp_handle h, int32_t which, int32_t reps, void *cuda
  * relative KKT error of the average and the current iterate at the last
  * check.  Then the handle takes the omega with the smallest value (first on
  * ties; *host_best receives it), its restart scheme is restored, and its
- * state is reset to the projection of zero.  Synchronizes the stream.
+ * state is reset to the projection of zero.  LP_ERR_TIMEOUT (see lp_solve)
+ * leaves the handle with its former omega.  Synchronizes the stream.
  */
 lp_status lp_select_omega(lp_handle h, const double *host_omegas, int32_t count,
                           int64_t iters, double *host_kkt, double *host_best,
@@ -290,7 +294,9 @@ lp_status lp_select_omega(lp_handle h, const double *host_omegas, int32_t count,
  * restarts; no termination test), keeping a checkpoint of (x, y, xbar, ybar)
  * and the inner iteration count at the start of every block of K
  * iterations and the restart decision of every check.  The unrolled map's
- * output is the running average (xbar, ybar) after the last check.
+ * output is the running average (xbar, ybar) after the last check.  Returns
+ * LP_ERR_NUMERICAL if the solve stops before its last check and
+ * LP_ERR_TIMEOUT (see lp_solve) in any block; no recording is kept then.
  */
 lp_status lp_solve_recorded(lp_handle h, int64_t iters, void *cuda_stream);
 
@@ -303,7 +309,8 @@ lp_status lp_solve_recorded(lp_handle h, int64_t iters, void *cuda_stream);
  * not change); blocks are recomputed from their checkpoints in reverse
  * order, each adjoint step running the transposed products of the forward
  * step.  Leaves the state of the recorded solve.  LP_ERR_NOT_SOLVED without
- * a recording.  Synchronizes the stream.
+ * a recording; after LP_ERR_TIMEOUT (see lp_solve) the call may be repeated.
+ * Synchronizes the stream.
  */
 lp_status lp_backward(lp_handle h, const double *dl_dx, const double *dl_dy,
                       double *dl_dc, double *dl_db, void *cuda_stream);

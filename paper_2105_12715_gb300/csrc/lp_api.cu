@@ -59,7 +59,7 @@ struct lp_problem {
   int64_t rec_blocks = 0;
   int64_t *rec_t0 = nullptr;           // device copies of the two, and [blocks] outer counts
   int8_t *rec_rs = nullptr;
-  int32_t *rec_flag = nullptr;         // a recorded solve stopped / an adjoint's wait ran out
+  int32_t *rec_flag = nullptr;         // status a recorded solve stopped with / an adjoint's wait ran out
   AdjVecs adj{};
   uint8_t *mask_x = nullptr, *mask_y = nullptr;  // [K][n], [K][m]
   DevState *st = nullptr;
@@ -88,6 +88,7 @@ struct lp_problem {
   int32_t sigma_steps = 0;            // Lanczos / power-iteration steps taken for sigma_max
   int32_t graph_kernels = 0;          // kernel nodes of the K-iteration graph
   unsigned int *bar = nullptr;          // counters of the grid barrier, when a kernel uses one
+  int hold_barrier = 0;                 // 1: its waits run out (lp_hold_barrier)
   ResidentArgs res{};                 // resident kernel (lp_resident.cu), when res_blocks > 0
   int res_blocks = 0;
   size_t res_smem = 0;
@@ -277,7 +278,8 @@ lp_status set_run_params(lp_problem *h, double tol, cudaStream_t s) {
   LP_CU(cudaMemcpyAsync(&h->st->status, &running, sizeof(int32_t), cudaMemcpyHostToDevice, s));
   if (h->bar) {  // grid barrier: counters and generation from zero
     LP_CU(cudaMemsetAsync(h->bar, 0, sizeof(unsigned) * kResBarLines * 32, s));
-    LP_CU(cudaMemsetAsync(&h->st->bar_gen, 0, sizeof(unsigned), s));
+    // held: a generation that no number of arrivals reaches
+    LP_CU(cudaMemsetAsync(&h->st->bar_gen, h->hold_barrier, sizeof(unsigned), s));
   }
   return LP_OK;
 }
@@ -1497,6 +1499,12 @@ lp_status lp_select_omega(lp_handle h, const double *omegas, int32_t count, int6
     DevState hs{};
     LP_CU(cudaMemcpyAsync(&hs, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
     LP_CU(cudaStreamSynchronize(s));
+    if (hs.status == LP_ERR_TIMEOUT) {  // no check to rank by: the handle as it was
+      if ((e = set_weight(h->opt.omega, scheme)) != LP_OK) return e;
+      h->solved = false;
+      if ((e = lp_set_state(h, nullptr, nullptr, cuda_stream)) != LP_OK) return e;
+      return fail(LP_ERR_TIMEOUT, "a device-side barrier wait expired");
+    }
     double v = std::fmin(hs.kkt_a[4], hs.kkt_c[4]);
     if (!std::isfinite(v)) v = INFINITY;
     kkt_out[k] = v;
@@ -1546,8 +1554,9 @@ lp_status lp_solve_recorded(lp_handle h, int64_t iters, void *cuda_stream) {
   h->rec_blocks = 0;
   LP_CU(cudaMalloc(&h->rec_t0, sizeof(int64_t) * (blocks + 1)));
   LP_CU(cudaMalloc(&h->rec_rs, sizeof(int8_t) * blocks));
-  if (!h->rec_flag && (e = h->alloc(&h->rec_flag, 2)) != LP_OK) return e;
-  LP_CU(cudaMemsetAsync(h->rec_flag, 0, sizeof(int32_t), s));
+  if (!h->rec_flag && (e = h->alloc(&h->rec_flag, 1)) != LP_OK) return e;
+  int32_t stop = kRunning;
+  LP_CU(cudaMemcpyAsync(h->rec_flag, &stop, sizeof(int32_t), cudaMemcpyHostToDevice, s));
   if ((e = set_run_params(h, 1e-300, s)) != LP_OK) return e;
   for (int64_t b = 0; b < blocks; ++b) {
     double *c = h->ckpt + b * slot;
@@ -1555,21 +1564,19 @@ lp_status lp_solve_recorded(lp_handle h, int64_t iters, void *cuda_stream) {
     LP_CU(cudaMemcpyAsync(c + n, h->v.y, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
     LP_CU(cudaMemcpyAsync(c + n + m, h->v.xbar, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     LP_CU(cudaMemcpyAsync(c + 2 * n + m, h->v.ybar, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    launch_record(h->st, h->rec_t0 + b, h->rec_t0 + blocks, nullptr, h->rec_flag, s);
+    launch_record(h->st, h->rec_t0 + b, h->rec_t0 + blocks, nullptr, h->rec_flag, false, s);
     LP_CU(cudaGraphLaunch(h->exec, s));
-    // a stop in the last block's check does not spoil the recording
-    launch_record(h->st, nullptr, h->rec_t0 + blocks, h->rec_rs + b,
-                  b + 1 < blocks ? h->rec_flag : h->rec_flag + 1, s);
+    launch_record(h->st, nullptr, h->rec_t0 + blocks, h->rec_rs + b, h->rec_flag, b + 1 == blocks, s);
   }
   LP_CU(cudaGetLastError());
   h->ckpt_t0.assign(blocks, 0);
   h->ckpt_restart.assign(blocks, 0);
-  int32_t stopped = 0;
   LP_CU(cudaMemcpyAsync(h->ckpt_t0.data(), h->rec_t0, sizeof(int64_t) * blocks, cudaMemcpyDeviceToHost, s));
   LP_CU(cudaMemcpyAsync(h->ckpt_restart.data(), h->rec_rs, sizeof(int8_t) * blocks, cudaMemcpyDeviceToHost, s));
-  LP_CU(cudaMemcpyAsync(&stopped, h->rec_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  LP_CU(cudaMemcpyAsync(&stop, h->rec_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   LP_CU(cudaStreamSynchronize(s));
-  if (stopped) return fail(LP_ERR_NUMERICAL, "solve stopped during recording");
+  if (stop == LP_ERR_TIMEOUT) return fail(LP_ERR_TIMEOUT, "a device-side barrier wait expired");
+  if (stop != kRunning) return fail(LP_ERR_NUMERICAL, "solve stopped during recording");
   h->rec_blocks = blocks;
   h->solved = true;
   return LP_OK;
@@ -1619,6 +1626,7 @@ lp_status lp_backward(lp_handle h, const double *dl_dx, const double *dl_dy, dou
     q.expired = h->rec_flag;
     q.K = K;
     q.count = 1;
+    q.gen = h->hold_barrier;
     LP_CU(cudaMemsetAsync(h->rec_flag, 0, sizeof(int32_t), s));
     LP_CU(cudaMemsetAsync(h->bar, 0, sizeof(unsigned) * kResBarLines * 32, s));
     launched = launch_adjoint(q, h->res_blocks, h->adj_smem, s) == cudaSuccess;
@@ -1641,6 +1649,17 @@ lp_status lp_backward(lp_handle h, const double *dl_dx, const double *dl_dy, dou
   LP_CU(cudaGetLastError());
   LP_CU(cudaStreamSynchronize(s));
   if (expired) return fail(LP_ERR_TIMEOUT, "a device-side barrier wait expired");
+  return LP_OK;
+}
+
+// For tests, not part of the ABI in lp.h: with on = 1 the grid barriers of the
+// handle's following calls wait for arrivals that never come, so that their
+// bounded wait (2 s) runs out and the kernel returns.  Fails on a handle whose
+// kernels use no grid barrier.
+lp_status lp_hold_barrier(lp_handle h, int32_t on) {
+  err_msg().clear();
+  if (!h || !h->bar) return fail(LP_ERR_INVALID_ARG, "no grid barrier");
+  h->hold_barrier = on ? 1 : 0;
   return LP_OK;
 }
 

@@ -17,6 +17,7 @@ constexpr int kHistWarps = 4;         // warps per block of the histogram kernel
 constexpr int kNewtonMax = 1024;      // Newton steps of a search (each clamps at least one more)
 constexpr uint64_t kNoKey = ~0ull;    // element that takes no part in the search
 constexpr int32_t kRunning = -1;      // DevState::status while iterating
+constexpr int32_t kStatusTimeout = 6;  // LP_ERR_TIMEOUT: a bounded wait ran out
 
 // Per-slice metadata of the sliced layout (see SellMat).
 struct SliceInfo {
@@ -258,6 +259,7 @@ struct AdjointArgs {
   uint8_t *mask_x, *mask_y;  // [K][n], [K][mstride]
   int32_t *expired;          // set when a barrier's wait ran out
   int32_t K, count;
+  unsigned gen;              // generation that the grid barrier starts from
 };
 
 // Launch with programmatic stream serialization: the kernel may be scheduled
@@ -370,7 +372,7 @@ void launch_project(const DevVecs &v, int n, int m, cudaStream_t s);
 void launch_fill(double *p, double val, int64_t n, cudaStream_t s);
 void launch_weights(DevState *st, double *w, cudaStream_t s);
 void launch_record(const DevState *st, int64_t *t0, int64_t *restarts, int8_t *restarted,
-                   int32_t *stopped, cudaStream_t s);
+                   int32_t *stop, bool last, cudaStream_t s);
 void launch_norms(const DevVecs &v, DevState *st, double *partials, int pstride,
                   int grid, int n, int m, cudaStream_t s);
 size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed, int ncol,

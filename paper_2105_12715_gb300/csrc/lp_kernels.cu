@@ -743,17 +743,18 @@ __global__ void weights_kernel(const DevState *st, double *w) {
 }
 
 // Recording for the adjoint, around a block's launches: the inner iteration
-// count and the outer count before it, whether its check restarted, and whether
-// the solve has stopped.
+// count and the outer count before it, whether its check restarted, and the status
+// with which the solve first stopped (a stop in the last block's check does not
+// spoil a recording, an expired wait there does).
 __global__ void record_kernel(const DevState *st, int64_t *t0, int64_t *restarts, int8_t *restarted,
-                              int32_t *stopped) {
+                              int32_t *stop, bool last) {
   if (t0) {
     *t0 = st->t0;
     *restarts = st->restarts;
   } else {
     *restarted = st->restarts > *restarts ? 1 : 0;
   }
-  if (st->status != kRunning) *stopped = 1;
+  if (*stop == kRunning && (!last || st->status == kStatusTimeout)) *stop = st->status;
 }
 
 // ------------------------------------------------------ power iteration
@@ -1313,8 +1314,8 @@ void launch_advance(DevState *st, double *w, int r, cudaStream_t s) {
 }
 
 void launch_record(const DevState *st, int64_t *t0, int64_t *restarts, int8_t *restarted,
-                   int32_t *stopped, cudaStream_t s) {
-  record_kernel<<<1, 1, 0, s>>>(st, t0, restarts, restarted, stopped);
+                   int32_t *stop, bool last, cudaStream_t s) {
+  record_kernel<<<1, 1, 0, s>>>(st, t0, restarts, restarted, stop, last);
 }
 
 void launch_weights(DevState *st, double *w, cudaStream_t s) {

@@ -58,7 +58,6 @@ constexpr int kGridThreads = 512;      // threads per block of the grid kernel
 constexpr int kClusterThreads = 256;   // and of the cluster kernel
 constexpr int kU = 8;                  // gathers in flight per lane
 constexpr int kStatusIterLimit = 4;
-constexpr int kStatusTimeout = 6;
 constexpr int kBarLines = kResBarLines;  // arrival counters of the grid barrier
 constexpr unsigned long long kWaitNs = 2000000000ull;  // longest wait at a barrier
 
@@ -549,8 +548,8 @@ struct SingleIO {
       st->kkt_c[i] = h.kkt[1][i];
     }
     st->returned = h.returned;
-    if (h.status != kRunning) {
-      st->status = h.status;
+    if (h.status != kRunning) {  // not over another block's expired wait
+      atomicCAS(&st->status, kRunning, h.status);
       return;
     }
     if (trace && st->trace_count < st->trace_cap) {
@@ -1438,7 +1437,7 @@ __global__ void __launch_bounds__(kGridThreads, 1)
   const Share sh{b, (a.AT.nslices - b + P - 1) / P, b, (a.A.nslices - b + P - 1) / P, P, 0, 0,
                  0, a.n, 0, a.m, b, P};
   GridLink<double> link{a.bar, 0u, nullptr, q.adj.v, q.adj.u};
-  run_adjoint<kGridThreads>(smem, q, sh, 0, a.st->tau, a.st->sigma, 0u, link);
+  run_adjoint<kGridThreads>(smem, q, sh, 0, a.st->tau, a.st->sigma, q.gen, link);
 }
 
 __global__ void __launch_bounds__(kClusterThreads, 2)
