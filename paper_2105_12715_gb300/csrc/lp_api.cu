@@ -1663,6 +1663,16 @@ lp_status lp_hold_barrier(lp_handle h, int32_t on) {
   return LP_OK;
 }
 
+// For tests, not part of the ABI in lp.h, before the handle's first solve: the
+// device refuses the resident kernel (its shared memory exceeds what a block may
+// have).  Fails on a handle that takes the per-pass kernels anyway.
+lp_status lp_refuse_resident(lp_handle h) {
+  err_msg().clear();
+  if (!h || h->exec || h->res_blocks == 0) return fail(LP_ERR_INVALID_ARG, "no resident kernel");
+  h->res_smem = size_t(1) << 20;
+  return LP_OK;
+}
+
 lp_status lp_profile_kernel(lp_handle h, int32_t which, int32_t reps, void *cuda_stream) {
   err_msg().clear();
   if (!h) return fail(LP_ERR_INVALID_ARG, "NULL handle");

@@ -1141,10 +1141,12 @@ struct lp_batch {
 
 namespace {
 
-lp_status batch_build_graph(lp_batch *h) {
-  if (h->exec) return LP_OK;
+// Captures one block of K_base iterations and the checks due: the cluster kernel,
+// or the per-pass kernels and the check's.
+cudaError_t batch_capture(lp_batch *h) {
   cudaStream_t s = h->cap_stream;
-  LP_CU(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+  cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
   cudaError_t launched = cudaSuccess;
   if (h->res.cluster > 0) {  // each cluster iterates, checks and counts its own problem
     launched = cudaMemsetAsync(&h->G->running, 0, sizeof(int32_t), s);
@@ -1158,14 +1160,27 @@ lp_status batch_build_graph(lp_batch *h) {
     h->launch_check(s);
   }
   cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamEndCapture(s, &g);
-  if (e == cudaSuccess && launched != cudaSuccess) {
-    cudaGraphDestroy(g);
-    e = launched;
+  e = cudaStreamEndCapture(s, &g);
+  if (e == cudaSuccess) e = launched;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&h->exec, g, 0);
+  if (e != cudaSuccess) {
+    if (g) cudaGraphDestroy(g);
+    h->exec = nullptr;
+    return e;
+  }
+  h->graph = g;
+  return cudaSuccess;
+}
+
+lp_status batch_build_graph(lp_batch *h) {
+  if (h->exec) return LP_OK;
+  cudaError_t e = batch_capture(h);
+  if (e != cudaSuccess && h->res.cluster > 0) {
+    cudaGetLastError();  // no such cluster here: the per-pass kernels
+    h->res.cluster = 0;
+    e = batch_capture(h);
   }
   if (e != cudaSuccess) return cuda_fail(e, "capture of an iteration block");
-  h->graph = g;
-  LP_CU(cudaGraphInstantiate(&h->exec, g, 0));
   return LP_OK;
 }
 
@@ -1860,6 +1875,14 @@ lp_status lp_batch_create(int32_t count, const int32_t *host_row_start,
   if ((e = batch_reset(h.get(), s)) != LP_OK) return e;
   h->setup_ms = ms_since(t_start);
   *out = h.release();
+  return LP_OK;
+}
+
+// For tests, not part of the ABI in lp_batch.h (see lp_refuse_resident).
+lp_status lp_batch_refuse_resident(lp_batch_handle h) {
+  err_msg().clear();
+  if (!h || h->exec || h->res.cluster == 0) return fail(LP_ERR_INVALID_ARG, "no resident kernel");
+  h->res_smem = size_t(1) << 20;
   return LP_OK;
 }
 
