@@ -45,7 +45,8 @@ extern "C" {
 typedef struct lp_batch *lp_batch_handle;
 
 /* Choices of the batch's own tuner (lp_batch_create with autotune != 0).
- * Kernel variants are timed on the batch itself; the check period of each
+ * Kernel variants are timed on the batch itself (a batch in clusters has none
+ * to choose from, see above); the check period of each
  * size class (problems binned by nonzeros, powers of 4) is the smallest
  * K_base * 2^s (s <= max_k_shift) whose measured check cost is at most
  * check_budget times the cost of the class's K iterations. */

@@ -1249,14 +1249,14 @@ lp_status batch_start(lp_batch *h, double tol, cudaStream_t s) {
   return LP_OK;
 }
 
-// Milliseconds per call of f (enqueued `reps` times on s after one warm-up
-// call), by CUDA events on s.
+// Milliseconds per call of f (enqueued `reps` times on s, after one warm-up
+// call if `warm`), by CUDA events on s.
 template <class F>
-lp_status time_ms(cudaStream_t s, int reps, F f, double *out) {
+lp_status time_ms(cudaStream_t s, int reps, F f, double *out, bool warm = true) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   LP_CU(cudaEventCreate(&e0));
   LP_CU(cudaEventCreate(&e1));
-  f();
+  if (warm) f();
   cudaEventRecord(e0, s);
   for (int r = 0; r < reps; ++r) f();
   cudaEventRecord(e1, s);
@@ -1271,16 +1271,20 @@ lp_status time_ms(cudaStream_t s, int reps, F f, double *out) {
   return LP_OK;
 }
 
-// The batch's tuner (run at create on the batch itself, from z = proj(0)):
-//  (1) kernel variants: for each pass, every unroll code of {2, 4, -2, -4}
-//      with one warp per slice or a grid of 8 blocks per SM (grid-stride
-//      over the work list), timed over 5 launches; the fastest is kept;
+// The batch's tuner (run at create on the batch itself, from z = proj(0)), on the
+// kernels that will run it:
+//  (1) kernel variants of the per-pass kernels: for each pass, every unroll code
+//      of {2, 4, -2, -4} with one warp per slice or a grid of 8 blocks per SM
+//      (grid-stride over the work list), timed over 5 launches; the fastest is kept;
 //  (2) check period per size class: with only that class running, the
-//      cost of one iteration (both passes) and of one check (the whole
-//      chain, every problem due) are timed; the class gets the smallest
-//      K = K_base 2^s (s <= max_k_shift) with check <= budget x K x iteration.
+//      cost of one iteration and of one check (the whole chain, every problem due)
+//      are timed; the class gets the smallest K = K_base 2^s (s <= max_k_shift)
+//      with check <= budget x K x iteration.  The cluster kernel's are taken from
+//      one block of K_base iterations without and one with a check due, after a
+//      first one of the whole batch (512 problems of 200 x 400: 11 us and 80 us in
+//      2.2 ms; the per-pass kernels' 17 and 136 say nothing about it).
 // Leaves the state dirty: the caller resets it.
-lp_status batch_tune(lp_batch *h, cudaStream_t s) {
+lp_status tune_passes(lp_batch *h, cudaStream_t s) {
   lp_status e;
   const int cands[4] = {2, 4, -2, -4};
   const int g_full[2] = {blocks_for_slices(h->AT.nslices), blocks_for_slices(h->A.nslices)};
@@ -1307,27 +1311,54 @@ lp_status batch_tune(lp_batch *h, cudaStream_t s) {
     (pass ? h->unroll_rows : h->unroll_cols) = bu;
     (pass ? h->grid_rows : h->grid_cols) = bg;
   }
-  // check period per size class
+  return LP_OK;
+}
+
+lp_status batch_tune(lp_batch *h, cudaStream_t s) {
+  lp_status e;
   std::vector<BInst> hi(h->count), run(h->count);
   LP_CU(cudaMemcpy(hi.data(), h->I, sizeof(BInst) * h->count, cudaMemcpyDeviceToHost));
+  auto block = [&] {
+    return launch_cluster(h->res, h->count, h->res_smem, h->mixed, h->res_inside, s);
+  };
+  if (h->res.cluster > 0 && block() != cudaSuccess) {
+    cudaGetLastError();  // no such cluster here: the per-pass kernels
+    h->res.cluster = 0;
+  }
+  if (h->res.cluster == 0 && (e = tune_passes(h, s)) != LP_OK) return e;
+  // check period per size class
   const int Kb = h->opt.check_every;
   for (int c = 0; c < kMaxClasses; ++c) {
     bool any = false;
     for (int32_t q = 0; q < h->count; ++q) any |= (h->size_class[q] == c);
     if (!any) continue;
-    for (int32_t q = 0; q < h->count; ++q) {
-      run[q] = hi[q];
-      run[q].status = (h->size_class[q] == c) ? kRunning : LP_ERR_NOT_SOLVED;
-      run[q].K = Kb;
-      run[q].since = 0;
-      run[q].iter_cap = INT64_MAX;
-    }
-    LP_CU(cudaMemcpyAsync(h->I, run.data(), sizeof(BInst) * h->count, cudaMemcpyHostToDevice, s));
-    h->launch_worklist(s);
+    auto start = [&](int32_t K) -> lp_status {  // the class from the start, checked every K
+      for (int32_t q = 0; q < h->count; ++q) {
+        run[q] = hi[q];
+        run[q].status = (h->size_class[q] == c) ? kRunning : LP_ERR_NOT_SOLVED;
+        run[q].K = K;
+        run[q].since = 0;
+        run[q].iter_cap = INT64_MAX;
+      }
+      LP_CU(cudaMemcpyAsync(h->I, run.data(), sizeof(BInst) * h->count, cudaMemcpyHostToDevice, s));
+      h->launch_worklist(s);
+      return LP_OK;
+    };
     double t_it = 0.0, t_ck = 0.0;
-    if ((e = time_ms(s, 4, [&] { h->launch_primal(0, s); h->launch_dual(0, s); }, &t_it)) != LP_OK)
-      return e;
-    if ((e = time_ms(s, 3, [&] { h->launch_check(s); }, &t_ck)) != LP_OK) return e;
+    if (h->res.cluster > 0) {
+      double without = 0.0, with = 0.0;
+      if ((e = start(INT32_MAX)) != LP_OK) return e;
+      if ((e = time_ms(s, 1, block, &without, false)) != LP_OK) return e;
+      if ((e = start(Kb)) != LP_OK) return e;
+      if ((e = time_ms(s, 1, block, &with, false)) != LP_OK) return e;
+      t_it = without / Kb;
+      t_ck = std::max(0.0, with - without);
+    } else {
+      if ((e = start(Kb)) != LP_OK) return e;
+      if ((e = time_ms(s, 4, [&] { h->launch_primal(0, s); h->launch_dual(0, s); }, &t_it)) != LP_OK)
+        return e;
+      if ((e = time_ms(s, 3, [&] { h->launch_check(s); }, &t_ck)) != LP_OK) return e;
+    }
     int sh = 0;
     while (sh < h->tune.max_k_shift && t_ck > h->tune.check_budget * (double)(Kb << sh) * t_it) ++sh;
     h->class_k[c] = Kb << sh;
