@@ -25,7 +25,11 @@
  *     buffers.  The handle owns all device memory it allocates.
  *   - Errors are reported as lp_status codes, never as exceptions; the
  *     message of the last error on the calling thread is lp_last_error().
- *   - A handle may be used by one host thread at a time.
+ *   - A handle may be used by one host thread at a time; handles on different
+ *     streams may work at the same time.  With autotune = 1 a block of
+ *     iterations of an LP that runs resident (see lp_options.autotune) starts
+ *     when all of its thread blocks find room: LPs that take the whole GPU run
+ *     one after the other, smaller ones side by side.
  */
 #ifndef LP_GB300_LP_H
 #define LP_GB300_LP_H

@@ -92,6 +92,7 @@ struct lp_problem {
   ResidentArgs res{};                 // resident kernel (lp_resident.cu), when res_blocks > 0
   int res_blocks = 0;
   size_t res_smem = 0;
+  bool res_lean = false;              // the grid kernel that leaves room for a second block per SM
   size_t adj_smem = 0;                // adjoint kernel on the same blocks (0: the per-pass kernels)
 
   ~lp_problem() {
@@ -226,7 +227,7 @@ cudaError_t capture_block(lp_problem *h) {
   if (h->res_blocks > 0) {
     launched = h->res.cluster > 0
                    ? launch_cluster(h->res, 1, h->res_smem, h->mixed, true, s)
-                   : launch_resident(h->res, h->res_blocks, h->res_smem, h->mixed, s);
+                   : launch_resident(h->res, h->res_blocks, h->res_smem, h->mixed, h->res_lean, s);
   } else {
     for (int k = 0; k < h->opt.check_every; ++k) launch_iteration(h, k, s);
     launched = launch_check(h->A, h->AT, h->v, h->st, h->w, h->cs, h->n, h->m, h->nsearch, h->trace,
@@ -296,13 +297,24 @@ lp_status set_run_params(lp_problem *h, double tol, cudaStream_t s) {
 // cycles instead of 2,800 but whose work has only 8 SMs (200 x 400: 0.25 ms in a
 // cluster, 0.33 on the grid; 2k x 10k: 0.41 and 0.43; 600 x 1400 in mixed
 // precision: 0.72 and 0.35).  Else the grid, with at least four slices per block
-// and pass, so that the barriers and reductions of a small LP span few blocks.
+// and pass, so that the barriers and reductions of a small LP span few blocks; in
+// mixed precision, whose slices are short, one per warp (16) unless the matrix needs
+// the room of more blocks.
+// A grid of one block per SM keeps LPs on other streams waiting, so blocks of up
+// to 64 KB leave room for a second one per SM where that costs the LP alone at most
+// 2%: in mixed precision, and in FP64 up to 8 slices per block and pass (5k x 25k, 11
+// of them, would lose 3%).  Two blocks of more than 64 KB would also leave too little
+// L1 to the gathers (10k x 50k mixed, 89 KB: 0.60 -> 0.63 ms alone).  64 iterations
+// and a check, ms per LP on 1, 4 and 8 streams, in brackets with one block per SM and
+// 4 slices per block, then the per-pass kernels: 2k x 10k 0.40, 0.23, 0.23 [0.40,
+// 0.39, 0.39; 0.90, 0.31, 0.30], 1k x 3k mixed 0.31, 0.09, 0.09 [0.32, 0.32, 0.32; 0.53,
+// 0.16, 0.09], 5k x 25k mixed 0.55, 0.31, 0.31 [0.54, 0.53, 0.53; 0.71, 0.36, 0.36].
 // The grid's gathers go through L1, so its blocks take at most 195 KB: above,
 // the SM's carve-out goes to its last step and leaves 28 KB of L1 instead of 60
 // (20k rows, FP64, us per iteration, per-pass kernels in brackets: 90k columns,
 // 192 KB, 14.7 [17.6]; 100k, 209 KB, 19.2 [17.3]).
 lp_status plan_resident(lp_problem *h, cudaStream_t s) {
-  constexpr int kSlicesPerBlock = 4, kClusterBlocks = 8;
+  constexpr int kClusterBlocks = 8;
   const int kClusterElems = h->mixed ? 768 : 2048;
   constexpr int kMaxCheckEvery = 1024;  // the weights lie in shared memory
   const lp_options &opt = h->opt;
@@ -310,7 +322,8 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
     return LP_OK;
   const int64_t elem = h->mixed ? 8 : 12;  // bytes of an index and a value
   const size_t limit = resident_smem_limit(h->device, h->mixed);
-  constexpr size_t kKeepL1 = 32 << 10;
+  constexpr size_t kKeepL1 = 32 << 10, kLeanBytes = 64 << 10;
+  constexpr int kLeanSlices = 8;
   if (limit <= kKeepL1 || 2 * h->nnz * elem > (int64_t)limit * h->nsm) return LP_OK;
   std::vector<SliceInfo> ic((size_t)h->AT.nslices + 1), ir((size_t)h->A.nslices + 1);
   LP_CU(cudaMemcpyAsync(ic.data(), h->AT.info, sizeof(SliceInfo) * ic.size(),
@@ -351,11 +364,14 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
     }
     P = cluster;
   }
-  if (!cluster) {
-    P = std::max(1, std::min(h->nsm, (most + kSlicesPerBlock - 1) / kSlicesPerBlock));
+  bool lean = false, fits = cluster > 0;
+  for (int per_block = h->mixed ? 16 : 4; !fits && per_block >= 4; per_block /= 4) {
+    P = std::max(1, std::min(h->nsm, (most + per_block - 1) / per_block));
     smem = block_bytes(P, false, false);
-    if (smem > limit - kKeepL1 || !resident_fits(P, h->nsm, smem, h->mixed)) return LP_OK;
+    lean = smem <= kLeanBytes && (h->mixed || most <= kLeanSlices * h->nsm);
+    fits = smem <= limit - kKeepL1 && resident_fits(P, h->nsm, smem, h->mixed, lean);
   }
+  if (!fits) return LP_OK;
   lp_status e;
   if ((e = h->alloc(&h->res.part, (int64_t)P * kResPart)) != LP_OK) return e;
   if ((e = h->alloc(&h->res.npart, (int64_t)2 * P * 8)) != LP_OK) return e;
@@ -380,6 +396,7 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
   h->res.n = h->n;
   h->res.m = h->m;
   h->res_smem = smem;
+  h->res_lean = lean;
   h->res_blocks = P;
   return LP_OK;
 }

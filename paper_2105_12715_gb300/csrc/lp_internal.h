@@ -378,14 +378,14 @@ void launch_norms(const DevVecs &v, DevState *st, double *partials, int pstride,
 size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed, int ncol,
                             int nrow);
 size_t resident_smem_limit(int device, bool mixed);
-bool resident_fits(int P, int nsm, size_t smem, bool mixed);
+bool resident_fits(int P, int nsm, size_t smem, bool mixed, bool lean);
 bool cluster_fits(int C, size_t smem, bool mixed, bool res, bool batch);
 cudaError_t launch_cluster(const ResidentArgs &a, int problems, size_t smem, bool mixed, bool res,
                            cudaStream_t s);
 size_t adjoint_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, int ncol, int nrow);
 bool adjoint_fits(int P, int nsm, int cluster, size_t smem);
 cudaError_t launch_adjoint(const AdjointArgs &q, int P, size_t smem, cudaStream_t s);
-cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixed,
+cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixed, bool lean,
                             cudaStream_t s);
 int check_grid_for(const SellMat &A, int num_sms);
 int split_grid(const SellMat &A);

@@ -57,6 +57,7 @@ namespace {
 constexpr int kGridThreads = 512;      // threads per block of the grid kernel
 constexpr int kClusterThreads = 256;   // and of the cluster kernel
 constexpr int kU = 8;                  // gathers in flight per lane
+constexpr int kLeanU = 4;              // where the registers of two blocks per SM hold no more
 constexpr int kStatusIterLimit = 4;
 constexpr int kBarLines = kResBarLines;  // arrival counters of the grid barrier
 constexpr unsigned long long kWaitNs = 2000000000ull;  // longest wait at a barrier
@@ -253,7 +254,7 @@ struct ClusterLink {
 // indices and values.  All lanes of a row return its sum.  The gathers are
 // plain loads: the barrier's acquire makes L1 safe to use.  SHIFT: vec starts at
 // element `base` of the index space (padding, index 0, reads element base).
-template <bool SHIFT, typename T>
+template <bool SHIFT, int UR = kU, typename T>
 __device__ __forceinline__ T slice_sum(T a, const int32_t *ip, const T *vp, int steps, int lg,
                                        const T *vec, int base) {
   if constexpr (SHIFT) {  // streamed from global memory: indices and values load together
@@ -272,13 +273,13 @@ __device__ __forceinline__ T slice_sum(T a, const int32_t *ip, const T *vp, int 
         if (t + u < steps) a = fma_t(c[u], vec[max(j[u] - base, 0)], a);
     }
   } else {
-    for (int t = 0; t < steps; t += kU) {
-      T g[kU];
+    for (int t = 0; t < steps; t += UR) {
+      T g[UR];
 #pragma unroll
-      for (int u = 0; u < kU; ++u)
+      for (int u = 0; u < UR; ++u)
         if (t + u < steps) g[u] = vec[ip[kWarp * (t + u)]];
 #pragma unroll
-      for (int u = 0; u < kU; ++u)
+      for (int u = 0; u < UR; ++u)
         if (t + u < steps) a = fma_t(vp[kWarp * (t + u)], g[u], a);
     }
   }
@@ -426,6 +427,66 @@ constexpr size_t col_bytes() {
 template <typename T>
 constexpr size_t row_bytes() {
   return sizeof(T) == 8 ? 4 + 8 + 8 + 8 + 4 : 4 + 4 + 4 + 8 + 8 + 16;
+}
+
+// The layout of run_block's shared memory: the arrays whose sizes are known from
+// the start, and, once the header tells the numbers of local rows and elements,
+// those behind them.
+template <typename T, int NT, bool CLUSTER>
+__device__ __forceinline__ unsigned char *lay_lists(Sm<T> &S, unsigned char *p, const Share &sh,
+                                                    int K) {
+  S.h = (Header *)carve(p, sizeof(Header));
+  if (CLUSTER) {  // at the same place in every block: owners store into all of them
+    S.ex = (T *)carve(p, sizeof(T) * sh.ncol);
+    S.ey = (T *)carve(p, sizeof(T) * sh.nrow);
+  }
+  S.cs = (LSlice *)carve(p, sizeof(LSlice) * sh.nc);
+  S.rs = (LSlice *)carve(p, sizeof(LSlice) * sh.nr);
+  S.red = (double *)carve(p, sizeof(double) * (NT / kWarp) * 32);
+  S.tot = (double *)carve(p, sizeof(double) * 32);
+  S.nw = (double *)carve(p, sizeof(double) * 8);
+  S.w = (double *)carve(p, sizeof(double) * K);
+  return p;
+}
+
+template <typename T, bool RES>
+__device__ __forceinline__ void lay_arrays(Sm<T> &S, unsigned char *p) {
+  const int ncl = S.h->ncl, nrl = S.h->nrl;
+  S.crow = (int32_t *)carve(p, 4 * (size_t)ncl);
+  S.rrow = (int32_t *)carve(p, 4 * (size_t)nrl);
+  S.c = (T *)carve(p, sizeof(T) * ncl);
+  S.x = (T *)carve(p, sizeof(T) * ncl);
+  S.xb = (double *)carve(p, 8 * (size_t)ncl);
+  S.b = (T *)carve(p, sizeof(T) * nrl);
+  S.y = (T *)carve(p, sizeof(T) * nrl);
+  S.yb = (double *)carve(p, 8 * (size_t)nrl);
+  if constexpr (sizeof(T) == 4) {
+    S.lf = (float *)carve(p, 4 * (size_t)ncl);
+    S.uf = (float *)carve(p, 4 * (size_t)ncl);
+    S.lo = (float *)carve(p, 4 * (size_t)nrl);
+    S.hi = (float *)carve(p, 4 * (size_t)nrl);
+    S.cs0 = (double *)carve(p, 8 * (size_t)ncl);
+    S.cs1 = (double *)carve(p, 8 * (size_t)ncl);
+    S.rs0 = (double *)carve(p, 8 * (size_t)nrl);
+    S.rs1 = (double *)carve(p, 8 * (size_t)nrl);
+  } else {
+    S.lk = (long long *)carve(p, 8 * (size_t)ncl);
+    S.uk = (long long *)carve(p, 8 * (size_t)ncl);
+    S.rt = (int32_t *)carve(p, 4 * (size_t)nrl);
+    // the check comes after the state has gone back to global memory
+    S.cs0 = S.xb;
+    S.cs1 = S.c;
+    S.rs0 = S.yb;
+    S.rs1 = S.b;
+  }
+  S.cidx = S.ridx = nullptr;
+  S.cval = S.rval = nullptr;
+  if constexpr (RES) {
+    S.cidx = (int32_t *)carve(p, 4 * (size_t)S.h->nce);
+    S.cval = (T *)carve(p, sizeof(T) * S.h->nce);
+    S.ridx = (int32_t *)carve(p, 4 * (size_t)S.h->nre);
+    S.rval = (T *)carve(p, sizeof(T) * S.h->nre);
+  }
 }
 
 // Mixed precision: the radius of a restart scales the next correction (mix_s),
@@ -628,31 +689,25 @@ struct BatchIO {
 //
 // K iterations and, when due, the check of one problem by the blocks of one
 // group.  T: float for mixed precision.  RES: the block's slices stay in shared
-// memory (else they are read from global memory in every pass).
-template <typename T, int NT, bool RES, class IO, class Link>
+// memory (else they are read from global memory in every pass).  LEAN: 64
+// registers per thread.  In mixed precision what the check needs is then laid out
+// again after the iterations instead of being kept through them, and 4 gathers are
+// in flight (5k x 25k, us per iteration: 7.5 without either, 7.2 with the first, 7.0
+// with both, 6.9 with 128 registers; in FP64 neither helps).
+template <typename T, int NT, bool RES, bool LEAN, class IO, class Link>
 __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArgs &a,
                                           const Share &sh, IO &io, Link &link) {
   constexpr bool MIX = sizeof(T) == 4;
   constexpr bool SHIFT = Link::kCluster && !RES;  // resident indices count from the problem's first
   constexpr int W = NT / kWarp;
+  constexpr int U = MIX && LEAN ? kLeanU : kU;
   const int P = sh.P, tid = (int)threadIdx.x;
   const int lane = tid & (kWarp - 1), warp = tid >> 5;
   const int nc = sh.nc, nr = sh.nr, K = io.iterations();
 
   // ---- layout of shared memory
   Sm<T> S;
-  unsigned char *p = smem;
-  S.h = (Header *)carve(p, sizeof(Header));
-  if (Link::kCluster) {  // at the same place in every block: owners store into all of them
-    S.ex = (T *)carve(p, sizeof(T) * sh.ncol);
-    S.ey = (T *)carve(p, sizeof(T) * sh.nrow);
-  }
-  S.cs = (LSlice *)carve(p, sizeof(LSlice) * nc);
-  S.rs = (LSlice *)carve(p, sizeof(LSlice) * nr);
-  S.red = (double *)carve(p, sizeof(double) * W * 32);
-  S.tot = (double *)carve(p, sizeof(double) * 32);
-  S.nw = (double *)carve(p, sizeof(double) * 8);
-  S.w = (double *)carve(p, sizeof(double) * K);
+  unsigned char *const behind = lay_lists<T, NT, Link::kCluster>(S, smem, sh, K);
   if (warp == 0)
     build_slices<RES>(a.AT, sh.c0, nc, sh.stride, sh.cfirst, S.cs, &S.h->ncl, &S.h->nce);
   else if (warp == 1)
@@ -670,47 +725,15 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
   __syncthreads();
   const int ncl = S.h->ncl, nrl = S.h->nrl;
   for (int k = tid; k < K; k += NT) S.w[k] = 1.0 / (double)(S.h->sc.t0 + k + 1);
-  S.crow = (int32_t *)carve(p, 4 * (size_t)ncl);
-  S.rrow = (int32_t *)carve(p, 4 * (size_t)nrl);
-  S.c = (T *)carve(p, sizeof(T) * ncl);
-  S.x = (T *)carve(p, sizeof(T) * ncl);
-  S.xb = (double *)carve(p, 8 * (size_t)ncl);
-  S.b = (T *)carve(p, sizeof(T) * nrl);
-  S.y = (T *)carve(p, sizeof(T) * nrl);
-  S.yb = (double *)carve(p, 8 * (size_t)nrl);
-  if constexpr (MIX) {
-    S.lf = (float *)carve(p, 4 * (size_t)ncl);
-    S.uf = (float *)carve(p, 4 * (size_t)ncl);
-    S.lo = (float *)carve(p, 4 * (size_t)nrl);
-    S.hi = (float *)carve(p, 4 * (size_t)nrl);
-    S.cs0 = (double *)carve(p, 8 * (size_t)ncl);
-    S.cs1 = (double *)carve(p, 8 * (size_t)ncl);
-    S.rs0 = (double *)carve(p, 8 * (size_t)nrl);
-    S.rs1 = (double *)carve(p, 8 * (size_t)nrl);
-  } else {
-    S.lk = (long long *)carve(p, 8 * (size_t)ncl);
-    S.uk = (long long *)carve(p, 8 * (size_t)ncl);
-    S.rt = (int32_t *)carve(p, 4 * (size_t)nrl);
-    // the check comes after the state has gone back to global memory
-    S.cs0 = S.xb;
-    S.cs1 = S.c;
-    S.rs0 = S.yb;
-    S.rs1 = S.b;
-  }
+  lay_arrays<T, RES>(S, behind);
   const int32_t *cidx, *ridx;  // indexed by LSlice::soff
   const T *cval, *rval;
   if constexpr (RES) {
-    S.cidx = (int32_t *)carve(p, 4 * (size_t)S.h->nce);
-    S.cval = (T *)carve(p, sizeof(T) * S.h->nce);
-    S.ridx = (int32_t *)carve(p, 4 * (size_t)S.h->nre);
-    S.rval = (T *)carve(p, sizeof(T) * S.h->nre);
     cidx = S.cidx;
     cval = S.cval;
     ridx = S.ridx;
     rval = S.rval;
   } else {
-    S.cidx = S.ridx = nullptr;
-    S.cval = S.rval = nullptr;
     const int64_t oc = a.AT.info[sh.cfirst].off, orr = a.A.info[sh.rfirst].off;
     cidx = a.AT.idx + oc;
     cval = values(a.AT, T(0)) + oc;
@@ -781,7 +804,7 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
       const LSlice sl = S.cs[i];
       const int lg = sl.lg(), r = lane >> lg, s = sl.slot0 + r;
       const bool owner = (lane & ((1 << lg) - 1)) == 0 && r < sl.rows();
-      const T neg_g = slice_sum<SHIFT>(owner ? -S.c[s] : T(0), cidx + sl.soff + lane,
+      const T neg_g = slice_sum<SHIFT, U>(owner ? -S.c[s] : T(0), cidx + sl.soff + lane,
                                        cval + sl.soff + lane, sl.steps(), lg, link.y(), sh.row0);
       if (owner) {
         const T x = S.x[s];
@@ -812,7 +835,7 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
       const LSlice sl = S.rs[i];
       const int lg = sl.lg(), r = lane >> lg, s = sl.slot0 + r;
       const bool owner = (lane & ((1 << lg) - 1)) == 0 && r < sl.rows();
-      const T res = slice_sum<SHIFT>(owner ? -S.b[s] : T(0), ridx + sl.soff + lane,
+      const T res = slice_sum<SHIFT, U>(owner ? -S.b[s] : T(0), ridx + sl.soff + lane,
                                      rval + sl.soff + lane, sl.steps(), lg, link.x(), sh.col0);
       if (owner) {
         const T y = S.y[s];
@@ -840,6 +863,12 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
       lost = true;
       break;
     }
+  }
+
+  if constexpr (LEAN && MIX) {
+    int zero = 0;
+    asm volatile("" : "+r"(zero));  // keeps the compiler from carrying the pointers over
+    lay_arrays<T, RES>(S, lay_lists<T, NT, Link::kCluster>(S, smem + zero, sh, K));
   }
 
   // ---- publish the iterate and the average (in mixed precision also in FP64)
@@ -1462,9 +1491,12 @@ __global__ void __launch_bounds__(kClusterThreads, 2)
   }
 }
 
-// One problem over the whole grid (cooperative launch).
-template <typename T>
-__global__ void __launch_bounds__(kGridThreads, 1)
+// One problem over the whole grid (cooperative launch).  A cooperative grid starts
+// once all of its blocks find room, so with one block per SM LPs that are solved on
+// several streams wait for one another; LEAN (64 registers) lets an SM hold blocks
+// of two of them (plan_resident has the rule and the figures).
+template <typename T, bool LEAN>
+__global__ void __launch_bounds__(kGridThreads, LEAN ? 2 : 1)
     resident_kernel(const __grid_constant__ ResidentArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   SingleIO io{a.st, a.w, a.trace};
@@ -1480,7 +1512,7 @@ __global__ void __launch_bounds__(kGridThreads, 1)
     link.gx = a.v.xhat;
     link.gy = a.v.y;
   }
-  run_block<T, kGridThreads, true>(smem, a, sh, io, link);
+  run_block<T, kGridThreads, true, LEAN>(smem, a, sh, io, link);
 }
 
 // One problem per cluster of a.cluster blocks: the single problem, or the
@@ -1497,7 +1529,7 @@ __global__ void __launch_bounds__(kClusterThreads, RES ? 2 : 4)
     if (!io.running()) return;
     const Share sh{rank, (a.AT.nslices - rank + C - 1) / C, rank, (a.A.nslices - rank + C - 1) / C,
                    C, 0, 0, 0, a.n, 0, a.m, rank, C};
-    run_block<T, kClusterThreads, RES>(smem, a, sh, io, link);
+    run_block<T, kClusterThreads, RES, false>(smem, a, sh, io, link);
   } else {
     BatchIO io{a.inst + blockIdx.x / C, a.glob};
     if (!io.running()) return;
@@ -1507,7 +1539,7 @@ __global__ void __launch_bounds__(kClusterThreads, RES ? 2 : 4)
                    C, B.cs0, B.rs0, B.col0, B.ncol, B.row0, B.nrow, rank, C};
     link.col0 = sh.col0;
     link.row0 = sh.row0;
-    run_block<T, kClusterThreads, RES>(smem, a, sh, io, link);
+    run_block<T, kClusterThreads, RES, false>(smem, a, sh, io, link);
   }
 }
 
@@ -1518,6 +1550,14 @@ bool set_smem(F *kernel, int bytes) {
     return true;
   cudaGetLastError();
   return false;
+}
+
+// The grid kernel of a precision, for one block per SM or two.
+using ResidentKernel = void (*)(ResidentArgs);
+ResidentKernel resident_of(bool mixed, bool lean) {
+  static const ResidentKernel k[4] = {resident_kernel<double, false>, resident_kernel<double, true>,
+                                      resident_kernel<float, false>, resident_kernel<float, true>};
+  return k[(mixed ? 2 : 0) + (lean ? 1 : 0)];
 }
 
 // The cluster kernel of a precision, residency and kind of problem.
@@ -1679,8 +1719,8 @@ size_t resident_smem_limit(int device, bool mixed) {
     cudaGetLastError();
     return 0;
   }
-  if (!(mixed ? set_smem(resident_kernel<float>, optin) : set_smem(resident_kernel<double>, optin)))
-    return 0;
+  for (int lean = 0; lean < 2; ++lean)
+    if (!set_smem(resident_of(mixed, lean != 0), optin)) return 0;
   for (int i = 0; i < 4; ++i)
     if (!set_smem(cluster_of(mixed, i & 1, i & 2), optin)) return 0;
   if (!mixed && !(set_smem(adjoint_kernel, optin) && set_smem(adjoint_cluster_kernel, optin)))
@@ -1689,12 +1729,10 @@ size_t resident_smem_limit(int device, bool mixed) {
 }
 
 // Whether P blocks with smem bytes each can be resident at once.
-bool resident_fits(int P, int nsm, size_t smem, bool mixed) {
+bool resident_fits(int P, int nsm, size_t smem, bool mixed, bool lean) {
   int per_sm = 0;
-  const cudaError_t e = mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                    &per_sm, resident_kernel<float>, kGridThreads, smem)
-                              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                    &per_sm, resident_kernel<double>, kGridThreads, smem);
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &per_sm, resident_of(mixed, lean), kGridThreads, smem);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -1726,7 +1764,7 @@ cudaError_t launch_search(const CheckScratch &cs, int64_t N, int nsearch, DevSta
   return cudaLaunchKernelEx(&cfg, search_kernel, SearchArgs{cs, st, N, nsearch});
 }
 
-cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixed,
+cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixed, bool lean,
                             cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)P);
@@ -1738,8 +1776,7 @@ cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixe
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return mixed ? cudaLaunchKernelEx(&cfg, resident_kernel<float>, a)
-               : cudaLaunchKernelEx(&cfg, resident_kernel<double>, a);
+  return cudaLaunchKernelEx(&cfg, resident_of(mixed, lean), a);
 }
 
 namespace {
