@@ -1280,9 +1280,9 @@ lp_status time_ms(cudaStream_t s, int reps, F f, double *out, bool warm = true) 
 //      cost of one iteration and of one check (the whole chain, every problem due)
 //      are timed; the class gets the smallest K = K_base 2^s (s <= max_k_shift)
 //      with check <= budget x K x iteration.  The cluster kernel's are taken from
-//      one block of K_base iterations without and one with a check due, after a
-//      first one of the whole batch (512 problems of 200 x 400: 11 us and 80 us in
-//      2.2 ms; the per-pass kernels' 17 and 136 say nothing about it).
+//      one block of K_base iterations without and one with a check due (512
+//      problems of 200 x 400: 11 us and 80 us; the per-pass kernels' 17 and 136 say
+//      nothing about it).
 // Leaves the state dirty: the caller resets it.
 lp_status tune_passes(lp_batch *h, cudaStream_t s) {
   lp_status e;
@@ -1318,43 +1318,47 @@ lp_status batch_tune(lp_batch *h, cudaStream_t s) {
   lp_status e;
   std::vector<BInst> hi(h->count), run(h->count);
   LP_CU(cudaMemcpy(hi.data(), h->I, sizeof(BInst) * h->count, cudaMemcpyDeviceToHost));
+  const int Kb = h->opt.check_every;
+  auto start = [&](int c, int32_t K) -> lp_status {  // class c from the start, checked every K
+    for (int32_t q = 0; q < h->count; ++q) {
+      run[q] = hi[q];
+      run[q].status = (h->size_class[q] == c) ? kRunning : LP_ERR_NOT_SOLVED;
+      run[q].K = K;
+      run[q].since = 0;
+      run[q].iter_cap = INT64_MAX;
+    }
+    LP_CU(cudaMemcpyAsync(h->I, run.data(), sizeof(BInst) * h->count, cudaMemcpyHostToDevice, s));
+    h->launch_worklist(s);
+    return LP_OK;
+  };
   auto block = [&] {
     return launch_cluster(h->res, h->count, h->res_smem, h->mixed, h->res_inside, s);
   };
-  if (h->res.cluster > 0 && block() != cudaSuccess) {
-    cudaGetLastError();  // no such cluster here: the per-pass kernels
-    h->res.cluster = 0;
+  if (h->res.cluster > 0) {  // loads the kernel; no problem runs
+    if ((e = start(-1, Kb)) != LP_OK) return e;
+    if (block() != cudaSuccess) {
+      cudaGetLastError();  // no such cluster here: the per-pass kernels
+      h->res.cluster = 0;
+      if ((e = batch_reset(h, s)) != LP_OK) return e;
+    }
   }
   if (h->res.cluster == 0 && (e = tune_passes(h, s)) != LP_OK) return e;
   // check period per size class
-  const int Kb = h->opt.check_every;
   for (int c = 0; c < kMaxClasses; ++c) {
     bool any = false;
     for (int32_t q = 0; q < h->count; ++q) any |= (h->size_class[q] == c);
     if (!any) continue;
-    auto start = [&](int32_t K) -> lp_status {  // the class from the start, checked every K
-      for (int32_t q = 0; q < h->count; ++q) {
-        run[q] = hi[q];
-        run[q].status = (h->size_class[q] == c) ? kRunning : LP_ERR_NOT_SOLVED;
-        run[q].K = K;
-        run[q].since = 0;
-        run[q].iter_cap = INT64_MAX;
-      }
-      LP_CU(cudaMemcpyAsync(h->I, run.data(), sizeof(BInst) * h->count, cudaMemcpyHostToDevice, s));
-      h->launch_worklist(s);
-      return LP_OK;
-    };
     double t_it = 0.0, t_ck = 0.0;
     if (h->res.cluster > 0) {
       double without = 0.0, with = 0.0;
-      if ((e = start(INT32_MAX)) != LP_OK) return e;
+      if ((e = start(c, INT32_MAX)) != LP_OK) return e;
       if ((e = time_ms(s, 1, block, &without, false)) != LP_OK) return e;
-      if ((e = start(Kb)) != LP_OK) return e;
+      if ((e = start(c, Kb)) != LP_OK) return e;
       if ((e = time_ms(s, 1, block, &with, false)) != LP_OK) return e;
       t_it = without / Kb;
       t_ck = std::max(0.0, with - without);
     } else {
-      if ((e = start(Kb)) != LP_OK) return e;
+      if ((e = start(c, Kb)) != LP_OK) return e;
       if ((e = time_ms(s, 4, [&] { h->launch_primal(0, s); h->launch_dual(0, s); }, &t_it)) != LP_OK)
         return e;
       if ((e = time_ms(s, 3, [&] { h->launch_check(s); }, &t_ck)) != LP_OK) return e;
