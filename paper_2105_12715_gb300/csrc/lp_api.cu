@@ -301,14 +301,15 @@ lp_status set_run_params(lp_problem *h, double tol, cudaStream_t s) {
 // mixed precision, whose slices are short, one per warp (16) unless the matrix needs
 // the room of more blocks.
 // A grid of one block per SM keeps LPs on other streams waiting, so blocks of up
-// to 64 KB leave room for a second one per SM where that costs the LP alone at most
-// 2%: in mixed precision, and in FP64 up to 8 slices per block and pass (5k x 25k, 11
-// of them, would lose 3%).  Two blocks of more than 64 KB would also leave too little
-// L1 to the gathers (10k x 50k mixed, 89 KB: 0.60 -> 0.63 ms alone).  64 iterations
-// and a check, ms per LP on 1, 4 and 8 streams, in brackets with one block per SM and
-// 4 slices per block, then the per-pass kernels: 2k x 10k 0.40, 0.23, 0.23 [0.40,
-// 0.39, 0.39; 0.90, 0.31, 0.30], 1k x 3k mixed 0.31, 0.09, 0.09 [0.32, 0.32, 0.32; 0.53,
-// 0.16, 0.09], 5k x 25k mixed 0.55, 0.31, 0.31 [0.54, 0.53, 0.53; 0.71, 0.36, 0.36].
+// to 64 KB leave room for a second one per SM: in FP64 with 256 threads, for up to 8
+// slices per block and pass (one per warp), in mixed precision with 64 registers per
+// thread, which costs the LP alone up to 2%.  Two blocks of more than 64 KB would
+// leave too little L1 to the gathers (10k x 50k mixed, 89 KB: 0.60 -> 0.63 ms alone).
+// 64 iterations and a check, ms per LP on 1, 4 and 8 streams, in brackets with one
+// block per SM and 4 slices per block, then the per-pass kernels: 2k x 10k 0.40, 0.22,
+// 0.22 [0.40, 0.39, 0.39; 0.90, 0.31, 0.30], 1k x 3k mixed 0.31, 0.09, 0.09 [0.32, 0.32,
+// 0.32; 0.53, 0.16, 0.09], 5k x 25k mixed 0.55, 0.32, 0.31 [0.54, 0.53, 0.53; 0.71, 0.36,
+// 0.36].
 // The grid's gathers go through L1, so its blocks take at most 195 KB: above,
 // the SM's carve-out goes to its last step and leaves 28 KB of L1 instead of 60
 // (20k rows, FP64, us per iteration, per-pass kernels in brackets: 90k columns,

@@ -450,8 +450,7 @@ __device__ __forceinline__ unsigned char *lay_lists(Sm<T> &S, unsigned char *p, 
 }
 
 template <typename T, bool RES>
-__device__ __forceinline__ void lay_arrays(Sm<T> &S, unsigned char *p) {
-  const int ncl = S.h->ncl, nrl = S.h->nrl;
+__device__ __forceinline__ void lay_arrays(Sm<T> &S, unsigned char *p, int ncl, int nrl) {
   S.crow = (int32_t *)carve(p, 4 * (size_t)ncl);
   S.rrow = (int32_t *)carve(p, 4 * (size_t)nrl);
   S.c = (T *)carve(p, sizeof(T) * ncl);
@@ -690,17 +689,17 @@ struct BatchIO {
 // K iterations and, when due, the check of one problem by the blocks of one
 // group.  T: float for mixed precision.  RES: the block's slices stay in shared
 // memory (else they are read from global memory in every pass).  LEAN: 64
-// registers per thread.  In mixed precision what the check needs is then laid out
-// again after the iterations instead of being kept through them, and 4 gathers are
-// in flight (5k x 25k, us per iteration: 7.5 without either, 7.2 with the first, 7.0
-// with both, 6.9 with 128 registers; in FP64 neither helps).
+// registers per thread, so what the check needs is laid out again after the
+// iterations instead of being kept through them, and 4 gathers are in flight
+// (5k x 25k in mixed precision, us per iteration: 7.5 without either, 7.2 with the
+// first, 7.0 with both, 6.9 with 128 registers).
 template <typename T, int NT, bool RES, bool LEAN, class IO, class Link>
 __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArgs &a,
                                           const Share &sh, IO &io, Link &link) {
   constexpr bool MIX = sizeof(T) == 4;
   constexpr bool SHIFT = Link::kCluster && !RES;  // resident indices count from the problem's first
   constexpr int W = NT / kWarp;
-  constexpr int U = MIX && LEAN ? kLeanU : kU;
+  constexpr int U = LEAN ? kLeanU : kU;
   const int P = sh.P, tid = (int)threadIdx.x;
   const int lane = tid & (kWarp - 1), warp = tid >> 5;
   const int nc = sh.nc, nr = sh.nr, K = io.iterations();
@@ -725,7 +724,7 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
   __syncthreads();
   const int ncl = S.h->ncl, nrl = S.h->nrl;
   for (int k = tid; k < K; k += NT) S.w[k] = 1.0 / (double)(S.h->sc.t0 + k + 1);
-  lay_arrays<T, RES>(S, behind);
+  lay_arrays<T, RES>(S, behind, ncl, nrl);
   const int32_t *cidx, *ridx;  // indexed by LSlice::soff
   const T *cval, *rval;
   if constexpr (RES) {
@@ -865,10 +864,10 @@ __device__ __forceinline__ void run_block(unsigned char *smem, const ResidentArg
     }
   }
 
-  if constexpr (LEAN && MIX) {
+  if constexpr (LEAN) {
     int zero = 0;
     asm volatile("" : "+r"(zero));  // keeps the compiler from carrying the pointers over
-    lay_arrays<T, RES>(S, lay_lists<T, NT, Link::kCluster>(S, smem + zero, sh, K));
+    lay_arrays<T, RES>(S, lay_lists<T, NT, Link::kCluster>(S, smem + zero, sh, K), S.h->ncl, S.h->nrl);
   }
 
   // ---- publish the iterate and the average (in mixed precision also in FP64)
@@ -1493,10 +1492,11 @@ __global__ void __launch_bounds__(kClusterThreads, 2)
 
 // One problem over the whole grid (cooperative launch).  A cooperative grid starts
 // once all of its blocks find room, so with one block per SM LPs that are solved on
-// several streams wait for one another; LEAN (64 registers) lets an SM hold blocks
-// of two of them (plan_resident has the rule and the figures).
-template <typename T, bool LEAN>
-__global__ void __launch_bounds__(kGridThreads, LEAN ? 2 : 1)
+// several streams wait for one another; PER_SM = 2 lets an SM hold blocks of two of
+// them (plan_resident has the rule and the figures): in FP64 with half the threads,
+// in mixed precision, whose blocks own more slices, with half the registers.
+template <typename T, int NT, int PER_SM>
+__global__ void __launch_bounds__(NT, PER_SM)
     resident_kernel(const __grid_constant__ ResidentArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   SingleIO io{a.st, a.w, a.trace};
@@ -1512,7 +1512,7 @@ __global__ void __launch_bounds__(kGridThreads, LEAN ? 2 : 1)
     link.gx = a.v.xhat;
     link.gy = a.v.y;
   }
-  run_block<T, kGridThreads, true, LEAN>(smem, a, sh, io, link);
+  run_block<T, NT, true, (NT * PER_SM > kGridThreads)>(smem, a, sh, io, link);
 }
 
 // One problem per cluster of a.cluster blocks: the single problem, or the
@@ -1555,9 +1555,13 @@ bool set_smem(F *kernel, int bytes) {
 // The grid kernel of a precision, for one block per SM or two.
 using ResidentKernel = void (*)(ResidentArgs);
 ResidentKernel resident_of(bool mixed, bool lean) {
-  static const ResidentKernel k[4] = {resident_kernel<double, false>, resident_kernel<double, true>,
-                                      resident_kernel<float, false>, resident_kernel<float, true>};
+  static const ResidentKernel k[4] = {
+      resident_kernel<double, kGridThreads, 1>, resident_kernel<double, kGridThreads / 2, 2>,
+      resident_kernel<float, kGridThreads, 1>, resident_kernel<float, kGridThreads, 2>};
   return k[(mixed ? 2 : 0) + (lean ? 1 : 0)];
+}
+int resident_threads(bool mixed, bool lean) {
+  return lean && !mixed ? kGridThreads / 2 : kGridThreads;
 }
 
 // The cluster kernel of a precision, residency and kind of problem.
@@ -1732,7 +1736,7 @@ size_t resident_smem_limit(int device, bool mixed) {
 bool resident_fits(int P, int nsm, size_t smem, bool mixed, bool lean) {
   int per_sm = 0;
   const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &per_sm, resident_of(mixed, lean), kGridThreads, smem);
+      &per_sm, resident_of(mixed, lean), resident_threads(mixed, lean), smem);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -1768,7 +1772,7 @@ cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixe
                             cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)P);
-  cfg.blockDim = dim3(kGridThreads);
+  cfg.blockDim = dim3((unsigned)resident_threads(mixed, lean));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
