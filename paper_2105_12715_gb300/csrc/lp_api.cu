@@ -287,14 +287,14 @@ lp_status set_run_params(lp_problem *h, double tol, cudaStream_t s) {
 
 // Decides whether a resident kernel (lp_resident.cu) runs this problem, which
 // one, and on how many blocks.  One does whenever autotune is on, no row is
-// split, and the matrix and the vectors fit into the shared memory of P blocks,
-// one per SM: for 5k x 25k (246k nonzeros, FP64) 64 iterations and a check take
+// split, and the matrix and the vectors fit into the shared memory of P blocks, at
+// most one per SM: for 5k x 25k (246k nonzeros, FP64) 64 iterations and a check take
 // 0.50 ms instead of 1.02, for 20k x 100k (1.0M nonzeros, mixed precision) 0.82
 // ms instead of 1.37.  A larger matrix would have to be streamed again in every
 // pass, which the per-pass kernels do with more warps in flight.
 // Few rows and columns (2,048; in mixed precision, whose layout has more and
-// shorter slices, 768): one cluster of up to 8 blocks, whose barrier takes 500
-// cycles instead of 2,800 but whose work has only 8 SMs (200 x 400: 0.25 ms in a
+// shorter slices, 768): one cluster of up to 8 blocks, whose barrier takes 700
+// cycles instead of 2,500 but whose work has only 8 SMs (200 x 400: 0.25 ms in a
 // cluster, 0.33 on the grid; 2k x 10k: 0.41 and 0.43; 600 x 1400 in mixed
 // precision: 0.72 and 0.35).  Else the grid, with at least four slices per block
 // and pass, so that the barriers and reductions of a small LP span few blocks; in
@@ -361,7 +361,7 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
     for (int C = kClusterBlocks; C >= 1 && !cluster; C /= 2) {
       if (C > 1 && C > most) continue;
       smem = block_bytes(C, true, false);
-      if (smem <= limit && cluster_fits(C, smem, h->mixed, true, false)) cluster = C;
+      if (smem <= limit && cluster_active(C, smem, h->mixed, true, false) > 0) cluster = C;
     }
     P = cluster;
   }
@@ -384,7 +384,9 @@ lp_status plan_resident(lp_problem *h, cudaStream_t s) {
   h->res.cluster = cluster;
   if (!h->mixed) {
     const size_t bytes = block_bytes(P, cluster > 0, true);
-    if (bytes <= limit && adjoint_fits(P, h->nsm, cluster, bytes)) h->adj_smem = bytes;
+    if (bytes <= limit &&
+        (cluster > 0 ? adjoint_active(cluster, bytes) > 0 : adjoint_fits(P, h->nsm, bytes)))
+      h->adj_smem = bytes;
   }
   h->res.A = h->A;
   h->res.AT = h->AT;

@@ -959,7 +959,8 @@ struct lp_batch {
   ResidentArgs res{};     // cluster kernel (lp_resident.cu), when res.cluster > 0
   size_t res_smem = 0;
   bool res_inside = false;  // the matrix stays in shared memory
-  size_t adj_smem = 0;      // adjoint kernel in the same clusters (0: the per-pass kernels)
+  size_t adj_smem = 0;      // adjoint kernel in clusters of adj_cluster (0: the per-pass kernels)
+  int adj_cluster = 0;
 
   ~lp_batch() {
     if (ckpt) cudaFree(ckpt);
@@ -1374,69 +1375,128 @@ lp_status batch_tune(lp_batch *h, cudaStream_t s) {
   return LP_OK;
 }
 
+// Time of an iteration by a model (us, GB300).  Per-pass kernels: from the batch's
+// slices and steps per SM and the longest slices of the two passes.  A cluster of C
+// blocks: from its problem's slices and steps per block and, where an SM holds more
+// than one block, from those of the others.  Fitted to 178 batches of 4 to 1,024
+// problems of 100 x 200 to 4000 x 8000, every C, inside and streamed (within 25%; the
+// per-pass kernels within 20%, in mixed precision 46%).
+struct PassModel {
+  double base, slice, step, chain;
+};
+struct ClusterModel {
+  double base, cluster, slice, step, slice_other, step_other;
+};
+constexpr PassModel kPerPass[2] = {{6.0, 0.0553, 0.0109, 0.1416}, {6.5, 0.0299, 0.0117, 0.0}};
+constexpr ClusterModel kInside[2] = {{1.05, 1.17, 0.0006, 0.0220, 0.0461, 0.0096},
+                                     {0.0, 1.93, 0.0526, 0.0059, 0.0066, 0.0062}};
+constexpr ClusterModel kStreamed[2] = {{1.12, 2.11, 0.0832, 0.0150, 0.0326, 0.0086},
+                                       {0.0, 2.69, 0.0688, 0.0111, 0.0095, 0.0039}};
+
 // Decides whether the cluster kernel (lp_resident.cu) runs the batch, every
 // problem in a cluster of C blocks, and whether the matrix stays in shared
 // memory.  Two launches per iteration cost a batch of small problems 8 us and
 // more, and a check ten launches; in the cluster kernel 512 problems of 200 x
-// 400 are bound by the FP64 pipe (21,500 cycles per iteration with four blocks
-// per SM, of which the FP64 instructions take 19,800): 0.80 ms per 64
-// iterations and check instead of 1.30 (1.74 with the lanes of the batch's
-// former layout).
-//   C: as many blocks (up to 8) as give every SM one, or two (128 problems of
-// 1000 x 2000: 1.21 ms per 64 iterations and check with C = 2, 1.43 with 1; 42
-// mixed-precision ones of 471 x 942: 0.75 with C = 4, 0.92 with 2).  The matrix
-// stays inside when all blocks then still fit at once (at most two per SM by
-// registers); otherwise it streams from L2 and four blocks fit.
-//   The batch goes this way when its largest problem does not hold the others
-// up: its FP64 time per iteration on C SMs is at most 16,000 cycles (less than
-// the launches cost) or 1.3 times the batch's mean per SM.
+// 400 are bound by the FP64 pipe (20,400 cycles per iteration on the SMs with
+// four blocks, where the pipe is busy throughout): 0.80 ms per 64 iterations and
+// check instead of 1.30 (1.74 with the lanes of the batch's former layout).
+//   What decides is how many clusters fit at once: clusters of 8 of one block per
+// SM only 15 times, of 4 36 times, so 16 problems of 4000 x 8000 in clusters of 8
+// take two rounds (27.7 us per iteration; the per-pass kernels 12.3).  Of the choices
+// of C, inside or streamed, and the per-pass kernels the one with the smallest
+// modelled time is taken: over the 178 batches 0.70 of the per-pass kernels' time on
+// average, at most 1.15 of it (24 of 2000 x 5000), and within 2% of the best choice on
+// average.  The backward has its own C (its vectors take more room); pass by pass it
+// takes 2.1 to 2.6 times an iteration, in clusters twice, so it stays in clusters up
+// to 1.15 of the per-pass kernels' modelled time.
 void plan_batch_resident(lp_batch *h, const HostSell &HA, const HostSell &HAT,
                          const std::vector<BInst> &hi) {
   constexpr int kMaxCheckEvery = 1024;  // the weights lie in shared memory
-  constexpr double kWarpOp = 19.0;      // cycles of an SM per FP64 instruction of a warp
-  constexpr double kLaunchCycles = 16e3, kImbalance = 1.3;
+  constexpr double kMarginBackward = 1.15;
   const lp_options &opt = h->opt;
   if (!opt.autotune || opt.check_every > kMaxCheckEvery) return;
   const size_t limit = resident_smem_limit(h->device, h->mixed);
   if (limit == 0) return;
   const int64_t elem = h->mixed ? 8 : 12;  // bytes of an index and a value
-  double total = 0.0, largest = 0.0;
-  for (const BInst &B : hi) {  // products, butterflies, projections and averages
-    double w = 0.0;
-    for (int s = B.cs0; s < B.cs1; ++s) w += 4 + (HAT.info[s].len_g >> 3) + (HAT.info[s].len_g & 7);
-    for (int s = B.rs0; s < B.rs1; ++s) w += 3 + (HA.info[s].len_g >> 3) + (HA.info[s].len_g & 7);
-    total += kWarpOp * w;
-    largest = std::max(largest, kWarpOp * w);
+  const int prec = h->mixed ? 1 : 0;
+  std::vector<double> steps(h->count, 0.0);  // of each problem
+  double all_steps = 0.0, chain = 0.0;
+  for (const HostSell *M : {&HA, &HAT}) {
+    int most = 0;
+    for (int s = 0; s < M->nslices; ++s) most = std::max(most, M->info[s].len_g >> 3);
+    chain += most;
   }
-  int C = 1;
-  while (C < kMaxCluster && (int64_t)h->count * C <= h->nsm) C *= 2;  // at most two blocks per SM
-  if (largest / C > std::max(kLaunchCycles, kImbalance * total / h->nsm)) return;
-  size_t with = 0, without = 0, adjoint = 0;
-  for (const BInst &B : hi)
-    for (int b = 0; b < C; ++b) {
-      int cols = 0, rows = 0, nc = 0, nr = 0;
-      int64_t elems = 0;
-      for (int s = B.cs0 + b; s < B.cs1; s += C, ++nc) {
-        cols += HAT.info[s + 1].row0 - HAT.info[s].row0;
-        elems += (HAT.info[s].len_g >> 3) * kWarp;
-      }
-      for (int s = B.rs0 + b; s < B.rs1; s += C, ++nr) {
-        rows += HA.info[s + 1].row0 - HA.info[s].row0;
-        elems += (HA.info[s].len_g >> 3) * kWarp;
-      }
-      const size_t fixed = resident_fixed_bytes(nc, nr, cols, rows, opt.check_every, h->mixed,
-                                                B.ncol, B.nrow);
-      without = std::max(without, fixed);
-      with = std::max(with, fixed + (size_t)(elems * elem));
-      adjoint = std::max(adjoint, adjoint_fixed_bytes(nc, nr, cols, rows, opt.check_every, B.ncol,
-                                                      B.nrow) + (size_t)(elems * elem));
+  for (int32_t q = 0; q < h->count; ++q) {
+    const BInst &B = hi[q];
+    for (int s = B.cs0; s < B.cs1; ++s) steps[q] += HAT.info[s].len_g >> 3;
+    for (int s = B.rs0; s < B.rs1; ++s) steps[q] += HA.info[s].len_g >> 3;
+    all_steps += steps[q];
+  }
+  const double all_slices = (double)HAT.nslices + HA.nslices;
+  const PassModel &pp = kPerPass[prec];
+  const double per_pass =
+      pp.base + (pp.slice * all_slices + pp.step * all_steps) / h->nsm + pp.chain * chain;
+  // time of the batch in clusters of C blocks, `active` of which fit at once, `layer`
+  // with one block per SM: rounds of the mean problem, the last one of the largest
+  auto modelled = [&](const ClusterModel &k, int C, int active, int layer) {
+    const int64_t at_once = std::min<int64_t>(h->count, active);
+    const double others =
+        (double)std::min<int64_t>((at_once + layer - 1) / layer, std::max(1, active / layer)) - 1.0;
+    const double rounds = (double)((h->count + (int64_t)active - 1) / active);
+    double most = 0.0;
+    for (int32_t q = 0; q < h->count; ++q) {
+      const BInst &B = hi[q];
+      most = std::max(most, k.slice * (B.cs1 - B.cs0 + B.rs1 - B.rs0) + k.step * steps[q]);
     }
-  const int64_t per_sm = ((int64_t)h->count * C + h->nsm - 1) / h->nsm;
-  h->res_inside = per_sm <= 2 && (int64_t)with * per_sm <= (int64_t)limit;
-  h->res_smem = h->res_inside ? with : without;
-  if (h->res_smem > limit || !cluster_fits(C, h->res_smem, h->mixed, h->res_inside, true)) return;
-  h->res.cluster = C;
-  if (!h->mixed && adjoint <= limit && adjoint_fits(1, 1, C, adjoint)) h->adj_smem = adjoint;
+    const double mean = (k.slice * all_slices + k.step * all_steps) / h->count;
+    const double shared = (k.slice_other * all_slices + k.step_other * all_steps) / h->count;
+    const double fixed = k.base + (C > 1 ? k.cluster : 0.0) + others * shared / C;
+    return rounds * (fixed + mean / C) + (most - mean) / C;
+  };
+  double best = per_pass, best_adjoint = kMarginBackward * per_pass;
+  for (int C = kMaxCluster; C >= 1; C /= 2) {
+    size_t with = 0, without = 0, adjoint = 0;
+    for (const BInst &B : hi)
+      for (int b = 0; b < C; ++b) {
+        int cols = 0, rows = 0, nc = 0, nr = 0;
+        int64_t elems = 0;
+        for (int s = B.cs0 + b; s < B.cs1; s += C, ++nc) {
+          cols += HAT.info[s + 1].row0 - HAT.info[s].row0;
+          elems += (HAT.info[s].len_g >> 3) * kWarp;
+        }
+        for (int s = B.rs0 + b; s < B.rs1; s += C, ++nr) {
+          rows += HA.info[s + 1].row0 - HA.info[s].row0;
+          elems += (HA.info[s].len_g >> 3) * kWarp;
+        }
+        const size_t fixed = resident_fixed_bytes(nc, nr, cols, rows, opt.check_every, h->mixed,
+                                                  B.ncol, B.nrow);
+        without = std::max(without, fixed);
+        with = std::max(with, fixed + (size_t)(elems * elem));
+        adjoint = std::max(adjoint, adjoint_fixed_bytes(nc, nr, cols, rows, opt.check_every,
+                                                        B.ncol, B.nrow) + (size_t)(elems * elem));
+      }
+    for (int inside = 1; inside >= 0; --inside) {
+      const size_t smem = inside ? with : without;
+      if (smem > limit) continue;
+      const int layer = cluster_active(C, limit, h->mixed, inside != 0, true);
+      const int active = cluster_active(C, smem, h->mixed, inside != 0, true);
+      if (layer == 0 || active == 0) continue;
+      const double t = modelled((inside ? kInside : kStreamed)[prec], C, active, layer);
+      if (t >= best) continue;
+      best = t;
+      h->res.cluster = C;
+      h->res_inside = inside != 0;
+      h->res_smem = smem;
+    }
+    if (h->mixed || adjoint > limit) continue;
+    const int layer = adjoint_active(C, limit), active = adjoint_active(C, adjoint);
+    if (layer == 0 || active == 0) continue;
+    const double t = modelled(kInside[0], C, active, layer);
+    if (t >= best_adjoint) continue;
+    best_adjoint = t;
+    h->adj_cluster = C;
+    h->adj_smem = adjoint;
+  }
 }
 
 double ms_since(std::chrono::steady_clock::time_point t0) {
@@ -1921,6 +1981,16 @@ lp_status lp_batch_refuse_resident(lp_batch_handle h) {
   return LP_OK;
 }
 
+// For tests, not part of the ABI in lp_batch.h: blocks per problem (0: the per-pass
+// kernels), negative when the matrix is streamed; blocks per problem of the backward.
+lp_status lp_batch_shape(lp_batch_handle h, int32_t *forward, int32_t *backward) {
+  err_msg().clear();
+  if (!h || !forward || !backward) return fail(LP_ERR_INVALID_ARG, "NULL argument");
+  *forward = h->res_inside ? h->res.cluster : -h->res.cluster;
+  *backward = h->res.cluster > 0 && h->adj_smem > 0 ? h->adj_cluster : 0;
+  return LP_OK;
+}
+
 lp_status lp_batch_set_state(lp_batch_handle h, const double *x, const double *y,
                              void *cuda_stream) {
   err_msg().clear();
@@ -2298,6 +2368,7 @@ lp_status lp_batch_backward(lp_batch_handle h, const double *dl_dx, const double
   if (h->res.cluster > 0 && h->adj_smem > 0) {  // one launch for all blocks, a cluster per problem
     AdjointArgs q{};
     q.r = h->res;
+    q.r.cluster = h->adj_cluster;
     q.adj = a;
     q.ckpt = h->ckpt;
     q.slot = slot;

@@ -14,7 +14,11 @@ constexpr int kWarpsPerBlock = kBlock / kWarp;
 constexpr int kBuckets = 256;         // buckets per pass of the multiplier search
 constexpr int kSearchPasses = 8;      // 8 x 8 bits cover a 64-bit key
 constexpr int kHistWarps = 4;         // warps per block of the histogram kernel
-constexpr int kNewtonMax = 1024;      // Newton steps of a search (each clamps at least one more)
+// Newton steps of a search.  f is concave, so a step leaves at most the share 1 - B'/B
+// of r^2 - f, where the slope (the sum of g^2 still free) falls from B to B': their
+// product shrinks at least fourfold.  lambda rises by an ulp or more per step, so it
+// takes at most 26 + log2(B_first / B_last) steps; 5 to 10 on the LPs measured.
+constexpr int kNewtonMax = 1024;
 constexpr uint64_t kNoKey = ~0ull;    // element that takes no part in the search
 constexpr int32_t kRunning = -1;      // DevState::status while iterating
 constexpr int32_t kStatusTimeout = 6;  // LP_ERR_TIMEOUT: a bounded wait ran out
@@ -379,11 +383,12 @@ size_t resident_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, bool mixed,
                             int nrow);
 size_t resident_smem_limit(int device, bool mixed);
 bool resident_fits(int P, int nsm, size_t smem, bool mixed, bool lean);
-bool cluster_fits(int C, size_t smem, bool mixed, bool res, bool batch);
+int cluster_active(int C, size_t smem, bool mixed, bool res, bool batch);
 cudaError_t launch_cluster(const ResidentArgs &a, int problems, size_t smem, bool mixed, bool res,
                            cudaStream_t s);
 size_t adjoint_fixed_bytes(int nc, int nr, int ncl, int nrl, int K, int ncol, int nrow);
-bool adjoint_fits(int P, int nsm, int cluster, size_t smem);
+bool adjoint_fits(int P, int nsm, size_t smem);
+int adjoint_active(int C, size_t smem);
 cudaError_t launch_adjoint(const AdjointArgs &q, int P, size_t smem, cudaStream_t s);
 cudaError_t launch_resident(const ResidentArgs &a, int P, size_t smem, bool mixed, bool lean,
                             cudaStream_t s);

@@ -15,27 +15,25 @@
 // those of the per-pass kernels bit for bit.
 //
 // Measured on GB300, 5k x 25k with 246k nonzeros, FP64, P = 152, cycles per
-// iteration: column pass 4,200, barrier 3,000, row pass 4,200, barrier 3,000
-// (7 us; the per-pass kernels 13.6 us).  The passes are bound by random
-// gathers from L2 (0.8 to 1 per cycle and SM; from L1, when a block gathers
-// the same line twice, 2.4), the barriers by the release fence and two trips
-// to L2 (2,500 cycles at 152 blocks with nothing else to do, 1,600 at 7).
-// Tagging every exchanged value with the number of its pass, so that gathers
-// wait for their own operand and no barrier is needed, was slower: the tagged
-// words bypass L1 and the repeated gathers fill it (9,500 cycles per pass).
-// So was copying the whole gathered vector into shared memory before a pass.
-// FP64 instructions are the other scarce thing: one of a warp holds its quarter
-// of the SM for 76 cycles whatever the number of active lanes.  So sums over
-// the block go through transposed butterflies, scalars are computed by one
-// warp, and the owned rows and columns are laid out one per thread where the
-// averages and the check's terms are formed.
+// iteration: column pass 3,800, barrier 3,300 (the averages included), row pass
+// 3,800, barrier 2,600 (6.8 us; the per-pass kernels 13.6 us).  The passes are bound
+// by the latency of random gathers from L2 (L1 18% busy, L2 13%), the barriers by
+// the release fence and two trips to L2; FP64 is 30% busy.  Tagging every exchanged
+// value with the number of its pass, so that gathers wait for their own operand and
+// no barrier is needed, was slower: the tagged words bypass L1 and the repeated
+// gathers fill it (9,500 cycles per pass).  FP64 instructions are the other scarce
+// thing: one of a warp holds its quarter of the SM for 76 cycles whatever the number
+// of active lanes.  So sums over the block go through transposed butterflies,
+// scalars are computed by one warp, and the owned rows and columns are laid out one
+// per thread where the averages and the check's terms are formed.
 //
 // In a cluster every block holds whole copies of xhat and y in shared memory and
-// the owners store into all of them, so a gather costs 30 cycles instead of 700
-// and the barrier 500 instead of 2,800: 200 x 400, 64 iterations and a check,
-// 0.25 ms on 8 blocks (0.33 on the grid, 0.49 with the per-pass kernels).  What
-// bounds a batch is the FP64 pipe: 512 problems of 200 x 400 run at 21,500
-// cycles per iteration with four blocks per SM, 19,800 of them FP64 issue.
+// the owners store into all of them, so a pass of 200 x 400 takes 1,600 cycles and
+// a barrier 700 instead of 2,500: 64 iterations and a check, 0.25 ms on 8 blocks
+// (0.33 on the grid, 0.49 with the per-pass kernels).  What bounds a batch is the
+// FP64 pipe: 512 problems of 200 x 400 run at 20,400 cycles per iteration with four
+// blocks per SM; the pipe is busy for 84% of an SM's active cycles, all of them where
+// four blocks run (512 blocks give some SMs three: 70% of elapsed).
 //
 // The multiplier lambda* of Section 6.3 is found by Newton's method on
 // F(mu) = sum min(d^2, mu g^2) = r^2, mu = lambda^2: F is concave and piecewise
@@ -210,7 +208,7 @@ __device__ __forceinline__ void put_shared(uint32_t addr, float v) {
 
 // Cluster: every block keeps whole copies of the two vectors in shared memory;
 // an owner stores its element into all of them (distributed shared memory) and
-// the hardware's cluster barrier orders the passes (500 cycles, no polling).
+// the hardware's cluster barrier orders the passes (no polling).
 template <typename T>
 struct ClusterLink {
   static constexpr bool kCluster = true;
@@ -1820,36 +1818,37 @@ cudaError_t launch_adjoint(const AdjointArgs &q, int P, size_t smem, cudaStream_
   return cudaLaunchKernelEx(&cfg, adjoint_kernel, q);
 }
 
-// Whether the adjoint kernel's blocks (clusters) fit.
-bool adjoint_fits(int P, int nsm, int cluster, size_t smem) {
-  int n = 0;
-  cudaError_t e;
-  if (cluster > 0) {
-    cudaLaunchAttribute at[1];
-    cudaLaunchConfig_t cfg = cluster_config(1, cluster, smem, at);
-    e = cudaOccupancyMaxActiveClusters(&n, adjoint_cluster_kernel, &cfg);
-    P = 1;
-    nsm = 1;
-  } else {
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, adjoint_kernel, kGridThreads, smem);
-  }
-  if (e != cudaSuccess) {
+// Whether P blocks of the adjoint kernel with smem bytes each can be resident at once.
+bool adjoint_fits(int P, int nsm, size_t smem) {
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, adjoint_kernel, kGridThreads, smem) !=
+      cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return (int64_t)n * nsm >= P;
+  return (int64_t)per_sm * nsm >= P;
 }
 
-// Whether the device can hold a cluster of C blocks with smem bytes each.
-bool cluster_fits(int C, size_t smem, bool mixed, bool res, bool batch) {
+// How many clusters of C blocks with smem bytes each the device holds at once (0: none).
+namespace {
+int active_clusters(const void *kernel, int C, size_t smem) {
   cudaLaunchAttribute at[1];
   cudaLaunchConfig_t cfg = cluster_config(1, C, smem, at);
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, cluster_of(mixed, res, batch), &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
-  return n > 0;
+  return n;
+}
+}  // namespace
+
+int cluster_active(int C, size_t smem, bool mixed, bool res, bool batch) {
+  return active_clusters((const void *)cluster_of(mixed, res, batch), C, smem);
+}
+
+int adjoint_active(int C, size_t smem) {
+  return active_clusters((const void *)adjoint_cluster_kernel, C, smem);
 }
 
 cudaError_t launch_cluster(const ResidentArgs &a, int problems, size_t smem, bool mixed, bool res,

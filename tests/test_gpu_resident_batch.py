@@ -5,6 +5,7 @@ iterates bit for bit, on every repeat.
 Among them problems whose first check restarts without a step of the multiplier
 search (every coordinate's full move to its bound lies inside the trust region): no
 barrier follows the check's there, so no block may still need another block's rows."""
+import ctypes as C
 import dataclasses
 
 import numpy as np
@@ -74,17 +75,40 @@ def uneven(count, m, n):
     return [lpgen.large_mixed(k, m=m + k % 7, n=n) for k in range(count)]
 
 
-# a problem gets 8, 4, 2 or 1 blocks while the batch leaves at most two per SM
+# batches that give a problem 8, 4, 2 and 1 blocks, the matrix inside or streamed (the
+# shapes that test_shapes_covered expects at 152 SMs)
 BATCHES = {
-    "box, 8 blocks": lambda: box_mix(sms() // 8),
-    "box, 4 blocks": lambda: box_mix(sms() // 3),
-    "box, 2 blocks": lambda: box_mix(2 * sms() // 3),
-    "box, 1 block": lambda: box_mix(sms() + 8),
-    "mixed rows, 2 blocks": lambda: uneven(2 * sms() // 3, 90, 200),
-    # two blocks per SM, each with more than half of its shared memory in matrix
-    "streamed, 2 blocks": lambda: [lpgen.tiny_standard_form(k % 3, m=1400, n=2800)
-                                   for k in range(2 * sms() // 3)],
+    "box, 19": lambda: box_mix(19),
+    "box, 50": lambda: box_mix(50),
+    "box, 101": lambda: box_mix(101),
+    "box, 160": lambda: box_mix(160),
+    "mixed rows, 101": lambda: uneven(101, 90, 200),
+    "200 x 400, 330": lambda: [lpgen.tiny_standard_form(k % 5) for k in range(330)],
+    "1000 x 2000, 101": lambda: [lpgen.tiny_standard_form(k % 3, m=1000, n=2000)
+                                 for k in range(101)],
+    "1400 x 2800, 40": lambda: [lpgen.tiny_standard_form(k % 3, m=1400, n=2800)
+                                for k in range(40)],
 }
+
+
+def shape(lpm, g):
+    f, b = C.c_int32(), C.c_int32()
+    assert lpm.load().lp_batch_shape(g.h, C.byref(f), C.byref(b)) == lpm.LP_OK
+    return f.value
+
+
+@pytest.mark.gpu
+def test_shapes_covered(lpm):
+    """Negative: the matrix is streamed."""
+    if sms() != 152:
+        pytest.skip("the choice depends on the number of SMs")
+    seen = {0: set(), 1: set()}
+    for precision in seen:
+        for make in BATCHES.values():
+            with lpm.LPBatch(make(), eta=ETA, check_every=K, precision=precision) as g:
+                seen[precision].add(shape(lpm, g))
+    for precision, got in seen.items():
+        assert {8, 4} <= got and {1, 2, -1, -2} & got and {-8, -4, -2} & got, (precision, got)
 
 
 @pytest.mark.gpu
