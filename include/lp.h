@@ -117,8 +117,12 @@ typedef struct {
                              unroll variant of the column and row passes is timed on this problem
                              and the fastest kept (overrides spmv_unroll and spmv_unroll_rows),
                              and the check's multiplier search is one launch instead of 16.
-                             Iterates do not depend on the choice: every variant sums each row in
-                             the same order.  0: the per-pass kernels with the unrolls given (1) */
+                             Every choice sums each row in the same order, so the iterates between
+                             two checks are the same bit for bit.  The check's own sums (KKT
+                             terms, gaps) are reduced in another order and agree to rounding: a
+                             restart or a stop that falls on its threshold to the last digits may
+                             come a check earlier or later.  0: the per-pass kernels with the
+                             unrolls given (1) */
   int32_t sigma_method;   /* estimator of sigma_max(A) when eta = 0: LP_SIGMA_LANCZOS (default;
                              at most min(power_iters, 1024) steps) or LP_SIGMA_POWER (Section 7's
                              power iteration); both stop when the estimate of sigma_max^2 changes

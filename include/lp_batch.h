@@ -28,10 +28,10 @@
  * a block boundary run together (one block of threads per problem for
  * reductions and for the multiplier search).  Problems that have stopped
  * cost nothing.  A batch of small problems (each fits into the shared memory of
- * a few SMs and none holds the others up; opt->autotune = 1) takes one launch
- * per block of K_base iterations and checks instead, every problem in a
- * thread-block cluster of its own, with the same iterates.  Errors, streams
- * and ownership as in lp.h.
+ * a few SMs; opt->autotune = 1) takes one launch per block of K_base iterations
+ * and checks instead, every problem in a thread-block cluster of its own, with
+ * the same iterates, where a model of both ways says that this is faster.
+ * Errors, streams and ownership as in lp.h.
  */
 #ifndef LP_GB300_LP_BATCH_H
 #define LP_GB300_LP_BATCH_H
